@@ -137,7 +137,9 @@ int lat_set_noise(lat_ctx* c, const double* noise, long long rows);
 
 /* Enqueue n time steps (Section 2: stream, drag, diffuse) on the context's stream.  In the
  * default launch mode the n steps are one CUDA-graph launch; the graph is captured on first use
- * of that n and cached (see lat_prepare). */
+ * of that n and cached (see lat_prepare).  1D FP32 lattices and ensembles with the upwind drag and
+ * N_v in {9, 17, 33, 65} take five steps per launch on chip while as many remain (the same bits),
+ * unless lat_set_launch chose a kernel. */
 int lat_step(lat_ctx* c, int n);
 
 /* Capture and instantiate the graph for n steps now, without running it, so that a later
@@ -257,7 +259,9 @@ int lat_adam(float* params, float* m, float* v, const float* grad, int n, int t,
 long long lat_steps_done(const lat_ctx* c);
 
 /* Launch shape of the step kernel.  Every variant gives the same bits.
- *  kernel: 0 keep; 1 plain coalesced loads (any size, FP32 or FP64).  The others bring the
+ *  kernel: 0 keep; a kernel of 1D lattices takes one step per launch (lat_autotune does not choose
+ *          in this sense: it sets the shape of the steps that are launched one by one);
+ *          1 plain coalesced loads (any size, FP32 or FP64).  The others bring the
  *          shifted plane windows into shared memory with bulk asynchronous copies (FP32; every
  *          N_x a multiple of 4 and >= 132):
  *          d = 1: 2..4 ring of that many item slots refilled after a block barrier;

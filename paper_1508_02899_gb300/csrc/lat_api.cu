@@ -74,6 +74,14 @@ struct lat_ctx {
     // width), ring slots, resident blocks per SM of the persistent grid, launch mode
     int variant = STEP1D_PLAIN, block = 256, slots = 3, bps = 4, mode = 0;
     bool ring_ok = false;
+    bool pinned = false;  // a kernel chosen by lat_set_launch: one step per launch
+
+    // several steps per launch (multi1d.cu): tiles (none where not built) and their widest places
+    MultiTile* d_tiles = nullptr;
+    int ntiles = 0, places = 0;
+    float2* d_basis = nullptr;    // flow-basis tables, their offsets per instance, and u / dv of a
+    long long* d_basis_off = nullptr;  // launch's steps (multi1d.cu)
+    float* d_wflow = nullptr;
 
     // cached graphs keyed by the number of steps (buffers are picked by the device step parity)
     std::map<int, cudaGraphExec_t> graphs;
@@ -178,6 +186,12 @@ Step1DArgs step_args(const lat_ctx* c, int k, int dry) {
     a.amp_stride = c->amp_stride;
     a.noise = c->d_noise;
     a.field = c->field;
+    a.basis = c->d_basis;
+    a.basis_off = c->d_basis_off;
+    a.wflow = c->d_wflow;
+    a.total_x = c->total_x;
+    a.nv = c->nv;
+    a.tile = c->block;
     a.st = c->d_state;
     a.dry = dry;
     a.frozen = c->frozen ? 1 : 0;
@@ -186,10 +200,86 @@ Step1DArgs step_args(const lat_ctx* c, int k, int dry) {
     return a;
 }
 
-// Enqueue n steps of a 1D context on stream s (used directly and under capture).
+constexpr int kMultiT = 5;  // steps per launch of the several-steps kernel
+
+// Tiles of the several-steps kernel, the flow-basis tables and the flow buffer it reads (beyond
+// kBasisBytes of tables, steps are launched one by one).  Called whenever the flow changes.
+constexpr size_t kBasisBytes = 64u << 20;
+constexpr int kMinTile = 64;  // narrower tiles are mostly margin
+
+int build_multi(lat_ctx* c) {
+    cudaFree(c->d_tiles);
+    cudaFree(c->d_basis);
+    cudaFree(c->d_basis_off);
+    c->d_tiles = nullptr;
+    c->d_basis = nullptr;
+    c->d_basis_off = nullptr;
+    c->ntiles = c->places = 0;
+    int places = 0, margin = 0;
+    if (c->dtype != LAT_F32 || !multi1d_shape(c->nv, kMultiT, &places, &margin)) return LAT_OK;
+    std::map<int, std::pair<int, long long>> sizes;  // N_x -> (an instance, table offset)
+    std::vector<long long> off(c->n_inst);
+    long long total = 0;
+    for (int i = 0; i < c->n_inst; ++i) {
+        const int nx = c->h_inst[i].nx;
+        const auto at = sizes.emplace(nx, std::make_pair(i, total));
+        if (at.second) total += (long long)nx * c->nmodes;
+        off[i] = at.first->second.second;
+    }
+    if (sizeof(float2) * (size_t)total > kBasisBytes) return LAT_OK;
+    if (cudaMalloc(&c->d_basis_off, sizeof(long long) * c->n_inst) != cudaSuccess ||
+        (total > 0 && cudaMalloc(&c->d_basis, sizeof(float2) * total) != cudaSuccess) ||
+        (!c->d_wflow &&
+         cudaMalloc(&c->d_wflow, sizeof(float) * kMultiT * c->total_x) != cudaSuccess)) {
+        cudaGetLastError();  // no room for them: steps are launched one by one
+        return LAT_OK;
+    }
+    CK(cudaMemcpy(c->d_basis_off, off.data(), sizeof(long long) * c->n_inst,
+                  cudaMemcpyHostToDevice));
+    if (total > 0) {
+        const Step1DArgs a = step_args(c, 0, 0);
+        for (const auto& e : sizes)
+            CK(launch_flow_basis(a, e.second.first, e.first, c->d_basis + e.second.second, c->stream));
+    }
+    // Tiles as wide as fit, or two per SM where there are fewer columns than that (64 instances
+    // of 200 to 1500 columns, N_v = 33, 50 steps: 268 us; one per SM 303 us; one step per launch
+    // 435 us).
+    const int wmax = (places - 2 * margin) / 8 * 8;
+    const int wfill = (int)(c->total_x / (2 * c->sm_count) / 8 * 8);
+    const int wtile = std::max(std::min(wfill, wmax), std::min(kMinTile, wmax));
+    std::vector<MultiTile> tiles;
+    for (int i = 0; i < c->n_inst; ++i) {
+        const Inst1D& in = c->h_inst[i];
+        const int nt = (in.nx + wtile - 1) / wtile;
+        const int w = std::min(wmax, ((in.nx + nt - 1) / nt + 7) / 8 * 8);
+        for (int x0 = 0; x0 < in.nx; x0 += w) {
+            tiles.push_back({in.off, in.xoff, in.nx, x0, std::min(w, in.nx - x0), (float)in.g,
+                             (float)in.r});
+            c->places = std::max(c->places, multi1d_places(c->nv, kMultiT, tiles.back().w));
+        }
+    }
+    if (cudaMalloc(&c->d_tiles, sizeof(MultiTile) * tiles.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return LAT_OK;
+    }
+    CK(cudaMemcpy(c->d_tiles, tiles.data(), sizeof(MultiTile) * tiles.size(),
+                  cudaMemcpyHostToDevice));
+    c->ntiles = (int)tiles.size();
+    return LAT_OK;
+}
+
+// Enqueue n steps of a 1D context on stream s (used directly and under capture): kMultiT steps per
+// launch on chip where that kernel is built and no launch shape was chosen, else one by one.
 int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
-    for (int k = 0; k < n; ++k) {
+    const bool multi = !c->pinned && c->mode != 1 && c->scheme == LAT_SCHEME_UPWIND && c->ntiles;
+    for (int k = 0, t; k < n; k += t) {
         Step1DArgs a = step_args(c, k, 0);
+        t = multi && n - k >= kMultiT ? kMultiT : 1;
+        if (t > 1) {
+            CK(launch_multi1d(c->nv, t, c->ntiles, c->places, a, c->d_tiles, k, c->ring_ok ? 1 : 0,
+                              s));
+            continue;
+        }
         if (c->mode == 1) {
             for (int i = 0; i < c->n_inst; ++i) {
                 a.item_begin = c->h_inst_begin[i];
@@ -318,6 +408,7 @@ int lat_ensemble_init(lat_ctx** out, int n_inst, const lat_instance* inst, int n
             c->bps = 4;
         }
         rc = build_items(c);
+        if (rc == LAT_OK) rc = build_multi(c);
     }
     if (rc != LAT_OK) {
         lat_free(c);
@@ -425,7 +516,7 @@ int lat_set_flow(lat_ctx* c, const lat_flow* fl) {
     k_set_noise_window<<<1, 1, 0, c->stream>>>(c->d_state, c->h_step, 0);
     CK(cudaGetLastError());
     drop_graphs(c);
-    return LAT_OK;
+    return build_multi(c);
 }
 
 int lat_set_noise(lat_ctx* c, const double* noise, long long rows) {
@@ -813,6 +904,7 @@ int lat_set_launch(lat_ctx* c, int kernel, int block, int blocks_per_sm, int mod
     c->block = nb;
     c->bps = nbps;
     c->mode = nmode;
+    if (kernel) c->pinned = true;
     drop_graphs(c);
     return retile ? build_items(c) : LAT_OK;
 }
@@ -865,6 +957,7 @@ int lat_autotune(lat_ctx* c, int reps, double* best) {
     // the dry runs may have flagged CFL on the current state; the next real step flags it again
     k_clear_status<<<1, 1, 0, c->stream>>>(c->d_state);
     int rc = lat_set_launch(c, bc.kernel, bc.block, bc.bps, mode_save);
+    c->pinned = false;  // the fastest shape of the single steps: batches stay on chip
     if (best) {
         best[0] = bc.kernel;
         best[1] = c->block;
@@ -1218,6 +1311,10 @@ void lat_free(lat_ctx* c) {
     cudaFree(c->d_items);
     cudaFree(c->d_inst_begin);
     cudaFree(c->d_partials);
+    cudaFree(c->d_tiles);
+    cudaFree(c->d_basis);
+    cudaFree(c->d_basis_off);
+    cudaFree(c->d_wflow);
     cudaFree(c->d_glob);
     cudaFree(c->d_amp);
     cudaFree(c->d_ampf);

@@ -75,6 +75,12 @@ struct Step1DArgs {
     long long amp_stride;    // n_inst * 2M
     const double* noise;     // [rows][n_inst][2M]
     const void* field;       // FIELD flow, per-cell array over all instances
+    // several steps per launch (multi1d.cu)
+    const float2* basis;         // (sin, cos) tables of the modes, one per grid size
+    const long long* basis_off;  // [n_inst] offset of the instance's table
+    float* wflow;                // [T][total_x] u / dv of the steps
+    long long total_x;
+    int nv, tile;                // N_v; columns per item
     DevState* st;
     int dry;                 // 1: do not advance the flow (autotuning)
     int frozen;              // 1: flow frozen (tau_f infinite)
@@ -88,6 +94,26 @@ struct Step1DArgs {
 };
 
 constexpr int kPcConsumerWarps = 4;
+
+// One tile of the several-steps kernel (multi1d.cu): columns x0 .. x0 + w - 1 of an instance, with
+// what the tile needs of the instance's parameters.
+struct MultiTile {
+    long long off;           // Inst1D::off
+    long long xoff;          // Inst1D::xoff
+    int nx, x0, w;
+    float g, r;
+};
+// T = 5, 9, 13 .. steps per launch for the N_v it is built for: the places a tile may take with its
+// margins (w + 2 margin <= max_places); false where there is no kernel.
+bool multi1d_shape(int nv, int T, int* max_places, int* margin);
+// Table of the flow's basis for instance inst's grid size: (sin, cos) of 2 pi k_m x / N_x, [m][x].
+cudaError_t launch_flow_basis(const Step1DArgs& a, int inst, int nx, float2* out, cudaStream_t s);
+// Places of a tile of w columns.
+int multi1d_places(int nv, int T, int w);
+// Steps kstep .. kstep + T - 1 of every tile, each on `places` (the widest tile's).  piped: N_x and x0
+// multiples of 4 throughout.
+cudaError_t launch_multi1d(int nv, int T, int ntiles, int places, const Step1DArgs& a,
+                           const MultiTile* tiles, int kstep, int piped, cudaStream_t s);
 
 // Arguments of the moment kernels (1D).
 struct Mom1DArgs {
