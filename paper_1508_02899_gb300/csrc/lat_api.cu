@@ -74,14 +74,17 @@ struct lat_ctx {
     // width), ring slots, resident blocks per SM of the persistent grid, launch mode
     int variant = STEP1D_PLAIN, block = 256, slots = 3, bps = 4, mode = 0;
     bool ring_ok = false;
+    bool stalled = false;  // lat_debug_stall
     bool pinned = false;  // a kernel chosen by lat_set_launch: one step per launch
 
     // several steps per launch (multi1d.cu): tiles (none where not built) and their widest places
     MultiTile* d_tiles = nullptr;
     int ntiles = 0, places = 0;
-    float2* d_basis = nullptr;    // flow-basis tables, their offsets per instance, and u / dv of a
+    bool line_ok = false;         // small enough for the cluster kernel (line1d.cu)
+    bool wflow_ok = false;        // the flow kernel's tables and buffer exist
+    void* d_basis = nullptr;      // flow-basis tables, their offsets per instance, and u / dv of a
     long long* d_basis_off = nullptr;  // launch's steps (multi1d.cu)
-    float* d_wflow = nullptr;
+    void* d_wflow = nullptr;
 
     // cached graphs keyed by the number of steps (buffers are picked by the device step parity)
     std::map<int, cudaGraphExec_t> graphs;
@@ -152,11 +155,18 @@ int build_items(lat_ctx* c) {
     return LAT_OK;
 }
 
-// The 1D globals [instances][M, P, E] of the last reduction to host memory: into the pinned
-// context buffer (wait: the caller synchronises and copies them on), or straight into the
+// A synchronising moment call of a few lattices: the last reduction writes the globals and the
+// status straight to pinned host memory (no copies, no clearing launch).
+bool direct_1d(const lat_ctx* c, bool wait) { return c->d == 1 && wait && c->n_inst <= kFinDirect; }
+
+// The last reduction of the 1D globals [instances][M, P, E], and their way to host memory: into the
+// pinned context buffer (wait: the caller synchronises and copies them on), or straight into the
 // caller's pinned buffer.
-int copy_globals_1d(lat_ctx* c, double* gdst, bool wait) {
-    if (!gdst) return LAT_OK;
+int finalize_1d(lat_ctx* c, int per_item, double* gdst, bool wait) {
+    const bool direct = direct_1d(c, wait);
+    CK(launch_finalize1d(c->d_partials, c->d_inst_begin, c->d_inst, c->n_inst, c->d_glob, per_item,
+                         c->d_state, direct ? c->h_glob : nullptr, &c->h_state->status, c->stream));
+    if (direct || !gdst) return LAT_OK;
     CK(cudaMemcpyAsync(wait ? c->h_glob : gdst, c->d_glob, sizeof(double) * 3 * c->n_inst,
                        cudaMemcpyDeviceToHost, c->stream));
     return LAT_OK;
@@ -201,13 +211,21 @@ Step1DArgs step_args(const lat_ctx* c, int k, int dry) {
 }
 
 constexpr int kMultiT = 5;  // steps per launch of the several-steps kernel
+static_assert(kMultiT <= kFlowSteps, "their flow is formed in one launch");
 
 // Tiles of the several-steps kernel, the flow-basis tables and the flow buffer it reads (beyond
 // kBasisBytes of tables, steps are launched one by one).  Called whenever the flow changes.
 constexpr size_t kBasisBytes = 64u << 20;
 constexpr int kMinTile = 64;  // narrower tiles are mostly margin
 
+int max_nx(const lat_ctx* c) {
+    int nx = 0;
+    for (const Inst1D& q : c->h_inst) nx = std::max(nx, q.nx);
+    return nx;
+}
+
 int build_multi(lat_ctx* c) {
+    c->line_ok = line1d_fits(c->dtype, c->n_inst, max_nx(c), c->nv, c->nmodes);
     cudaFree(c->d_tiles);
     cudaFree(c->d_basis);
     cudaFree(c->d_basis_off);
@@ -215,8 +233,8 @@ int build_multi(lat_ctx* c) {
     c->d_basis = nullptr;
     c->d_basis_off = nullptr;
     c->ntiles = c->places = 0;
-    int places = 0, margin = 0;
-    if (c->dtype != LAT_F32 || !multi1d_shape(c->nv, kMultiT, &places, &margin)) return LAT_OK;
+    c->wflow_ok = false;
+    const size_t elem = c->dtype == LAT_F64 ? sizeof(double) : sizeof(float);
     std::map<int, std::pair<int, long long>> sizes;  // N_x -> (an instance, table offset)
     std::vector<long long> off(c->n_inst);
     long long total = 0;
@@ -226,11 +244,11 @@ int build_multi(lat_ctx* c) {
         if (at.second) total += (long long)nx * c->nmodes;
         off[i] = at.first->second.second;
     }
-    if (sizeof(float2) * (size_t)total > kBasisBytes) return LAT_OK;
+    if (2 * elem * (size_t)total > kBasisBytes) return LAT_OK;
     if (cudaMalloc(&c->d_basis_off, sizeof(long long) * c->n_inst) != cudaSuccess ||
-        (total > 0 && cudaMalloc(&c->d_basis, sizeof(float2) * total) != cudaSuccess) ||
+        (total > 0 && cudaMalloc(&c->d_basis, 2 * elem * total) != cudaSuccess) ||
         (!c->d_wflow &&
-         cudaMalloc(&c->d_wflow, sizeof(float) * kMultiT * c->total_x) != cudaSuccess)) {
+         cudaMalloc(&c->d_wflow, elem * kFlowSteps * c->total_x) != cudaSuccess)) {
         cudaGetLastError();  // no room for them: steps are launched one by one
         return LAT_OK;
     }
@@ -239,8 +257,12 @@ int build_multi(lat_ctx* c) {
     if (total > 0) {
         const Step1DArgs a = step_args(c, 0, 0);
         for (const auto& e : sizes)
-            CK(launch_flow_basis(a, e.second.first, e.first, c->d_basis + e.second.second, c->stream));
+            CK(launch_flow_basis(c->dtype, a, e.second.first, e.first, c->d_basis, e.second.second,
+                                 c->stream));
     }
+    c->wflow_ok = true;
+    int places = 0, margin = 0;
+    if (c->dtype != LAT_F32 || !multi1d_shape(c->nv, kMultiT, &places, &margin)) return LAT_OK;
     // Tiles as wide as fit, or two per SM where there are fewer columns than that (64 instances
     // of 200 to 1500 columns, N_v = 33, 50 steps: 268 us; one per SM 303 us; one step per launch
     // 435 us).
@@ -268,10 +290,30 @@ int build_multi(lat_ctx* c) {
     return LAT_OK;
 }
 
-// Enqueue n steps of a 1D context on stream s (used directly and under capture): kMultiT steps per
-// launch on chip where that kernel is built and no launch shape was chosen, else one by one.
+// Whether batches of steps run on the cluster kernel of small lattices.
+bool line_1d(const lat_ctx* c) {
+    return c->d == 1 && !c->pinned && c->mode != 1 && c->scheme == LAT_SCHEME_UPWIND &&
+           c->line_ok && !c->stalled;
+}
+
+// Enqueue n steps of a 1D context on stream s (used directly and under capture).  Where no launch
+// shape was chosen: all of them in one launch for small lattices, kMultiT per launch where that
+// kernel is built; else one by one.
 int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
-    const bool multi = !c->pinned && c->mode != 1 && c->scheme == LAT_SCHEME_UPWIND && c->ntiles;
+    const bool chosen = c->pinned || c->mode == 1;
+    const bool on_chip = !chosen && c->scheme == LAT_SCHEME_UPWIND;
+    if (n > 1 && line_1d(c)) {
+        CK(launch_line1d(c->dtype, c->n_inst, max_nx(c), c->nv, step_args(c, 0, 0), 0, n, s));
+        if (c->n_inst > 1) CK(launch_advance_step(c->d_state, n, s));
+        return LAT_OK;
+    }
+    const bool multi = on_chip && c->ntiles;
+    // The plain-load kernels take the flow from the flow kernel (kFlowSteps steps at a time):
+    // evaluating the basis costs an FP64 column as much as half its sweep.
+    const bool pre = !chosen && c->variant == STEP1D_PLAIN && c->wflow_ok &&
+                     c->flow_kind == LAT_FLOW_MODES;
+    const size_t row = (c->dtype == LAT_F64 ? sizeof(double) : sizeof(float)) * c->total_x;
+    int formed = 0, first = 0;  // steps whose flow is formed, from step `first` on
     for (int k = 0, t; k < n; k += t) {
         Step1DArgs a = step_args(c, k, 0);
         t = multi && n - k >= kMultiT ? kMultiT : 1;
@@ -279,6 +321,15 @@ int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
             CK(launch_multi1d(c->nv, t, c->ntiles, c->places, a, c->d_tiles, k, c->ring_ok ? 1 : 0,
                               s));
             continue;
+        }
+        if (pre) {
+            if (k >= first + formed) {
+                first = k;
+                formed = std::min(kFlowSteps, n - k);
+                if (formed % 2 == 0) --formed;  // odd: the amplitudes move to the other parity
+                CK(launch_flow_steps(c->dtype, a, k, formed, s));
+            }
+            a.wpre = static_cast<char*>(c->d_wflow) + (k - first) * row;
         }
         if (c->mode == 1) {
             for (int i = 0; i < c->n_inst; ++i) {
@@ -406,6 +457,12 @@ int lat_ensemble_init(lat_ctx** out, int n_inst, const lat_instance* inst, int n
             c->variant = STEP1D_PLAIN;
             c->block = std::min(256, step1d_max_block(dtype, nv, STEP1D_PLAIN));
             c->bps = 4;
+            // FP64 columns are bound by the SM's FP64 pipe: few of them in narrow blocks, so that
+            // every SM gets some (N_x = 3000, N_v = 33: 26.6 us per step, 49.5 in blocks of 256)
+            while (dtype == LAT_F64 && c->block > 32 && c->total_x < 2ll * c->block * c->sm_count) {
+                c->block /= 2;
+                c->bps *= 2;
+            }
         }
         rc = build_items(c);
         if (rc == LAT_OK) rc = build_multi(c);
@@ -640,9 +697,14 @@ int enqueue_moments(lat_ctx* c, double* rho, double* mean_v, double* mean_v2, do
     a.st = c->d_state;
     const int grid = std::max(1, std::min(c->nitems, 8 * c->sm_count));
     CK(launch_moments1d(c->dtype, tile_of(c), 1, grid, a, c->stream));
-    CK(launch_finalize1d(c->d_partials, c->d_inst_begin, c->d_inst, c->n_inst, c->d_glob,
-                         tile_of(c) / 32, c->stream));
-    return copy_globals_1d(c, gdst, wait);
+    return finalize_1d(c, tile_of(c) / 32, gdst, wait);
+}
+
+// Wait for a moment call and take the pending status.
+int wait_status(lat_ctx* c) {
+    if (!direct_1d(c, true)) return lat_status(c);
+    CK(cudaStreamSynchronize(c->stream));
+    return status_code(c->h_state->status);
 }
 
 // n steps and the moments of the state the last one writes (fused into it where the launch
@@ -661,7 +723,7 @@ int enqueue_step_moments(lat_ctx* c, int n, double* rho, double* mean_v, double*
         return LAT_OK;
     }
     const bool fused = c->d == 1 && c->variant == STEP1D_PC && c->mode != 1 &&
-                       step1d_moments_supported(c->dtype, c->nv);
+                       step1d_moments_supported(c->dtype, c->nv) && !(n > 1 && line_1d(c));
     if (!fused) {
         int rc = lat_step(c, n);
         if (rc != LAT_OK) return rc;
@@ -678,11 +740,9 @@ int enqueue_step_moments(lat_ctx* c, int n, double* rho, double* mean_v, double*
     a.m_partials = c->d_partials;
     CK(launch_step1d_moments(c->nv, persistent_grid(c), a, c->stream));
     CK(launch_advance_step(c->d_state, 1, c->stream));
-    CK(launch_finalize1d(c->d_partials, c->d_inst_begin, c->d_inst, c->n_inst, c->d_glob,
-                         kPcConsumerWarps, c->stream));
     c->h_step += 1;
     c->cur = (int)(c->h_step & 1);
-    return copy_globals_1d(c, gdst, wait);
+    return finalize_1d(c, kPcConsumerWarps, gdst, wait);
 }
 
 }  // namespace
@@ -693,7 +753,7 @@ int lat_moments(lat_ctx* c, double* rho, double* mean_v, double* mean_v2, double
     if (!c) return LAT_EINVAL;
     int rc = enqueue_moments(c, rho, mean_v, mean_v2, globals, true);
     if (rc != LAT_OK) return rc;
-    rc = lat_status(c);  // synchronises
+    rc = wait_status(c);
     if (globals && c->d == 1) memcpy(globals, c->h_glob, sizeof(double) * 3 * c->n_inst);
     return rc;
 }
@@ -703,7 +763,7 @@ int lat_step_moments(lat_ctx* c, int n, double* rho, double* mean_v, double* mea
     if (!c || n < 1) return LAT_EINVAL;
     int rc = enqueue_step_moments(c, n, rho, mean_v, mean_v2, globals, true);
     if (rc != LAT_OK) return rc;
-    rc = lat_status(c);  // synchronises
+    rc = wait_status(c);
     if (globals && c->d == 1) memcpy(globals, c->h_glob, sizeof(double) * 3 * c->n_inst);
     return rc;
 }
@@ -1298,6 +1358,8 @@ int lat_set_state(lat_ctx* c, const void* image, long long bytes) {
 int lat_debug_stall(lat_ctx* c, int on) {
     if (!c) return LAT_EINVAL;
     CK(launch_set_stall(c->d_state, on ? 1u : 0u, c->stream));
+    c->stalled = on != 0;  // batches take a kernel with a copy pipeline
+    drop_graphs(c);
     return LAT_OK;
 }
 

@@ -76,9 +76,10 @@ struct Step1DArgs {
     const double* noise;     // [rows][n_inst][2M]
     const void* field;       // FIELD flow, per-cell array over all instances
     // several steps per launch (multi1d.cu)
-    const float2* basis;         // (sin, cos) tables of the modes, one per grid size
+    const void* basis;           // (sin, cos) tables of the modes, one per grid size
     const long long* basis_off;  // [n_inst] offset of the instance's table
-    float* wflow;                // [T][total_x] u / dv of the steps
+    void* wflow;                 // [T][total_x] u / dv of the steps
+    const void* wpre;            // u / dv of this step's columns (a row of wflow), or null
     long long total_x;
     int nv, tile;                // N_v; columns per item
     DevState* st;
@@ -106,8 +107,19 @@ struct MultiTile {
 // T = 5, 9, 13 .. steps per launch for the N_v it is built for: the places a tile may take with its
 // margins (w + 2 margin <= max_places); false where there is no kernel.
 bool multi1d_shape(int nv, int T, int* max_places, int* margin);
-// Table of the flow's basis for instance inst's grid size: (sin, cos) of 2 pi k_m x / N_x, [m][x].
-cudaError_t launch_flow_basis(const Step1DArgs& a, int inst, int nx, float2* out, cudaStream_t s);
+// Steps kstep .. kstep + n - 1 of small 1D lattices (upwind drag), one cluster per lattice with the
+// state in shared memory throughout (line1d.cu).
+bool line1d_fits(int dtype, int n_inst, int nx_max, int nv, int nmodes);
+cudaError_t launch_line1d(int dtype, int n_inst, int nx_max, int nv, const Step1DArgs& a, int kstep,
+                          int n, cudaStream_t s);
+// Table of the flow's basis for instance inst's grid size, at entry `at` of the table:
+// (sin, cos) of 2 pi k_m x / N_x, [m][x].
+cudaError_t launch_flow_basis(int dtype, const Step1DArgs& a, int inst, int nx, void* table,
+                              long long at, cudaStream_t s);
+// u / dv of steps kstep .. kstep + T - 1 into wflow (T <= kFlowSteps, odd: the amplitudes move to the
+// step after them, in the parity that no block reads).  One block per item.
+constexpr int kFlowSteps = 5;
+cudaError_t launch_flow_steps(int dtype, const Step1DArgs& a, int kstep, int T, cudaStream_t s);
 // Places of a tile of w columns.
 int multi1d_places(int nv, int T, int w);
 // Steps kstep .. kstep + T - 1 of every tile, each on `places` (the widest tile's).  piped: N_x and x0
@@ -162,9 +174,12 @@ cudaError_t launch_set_devstate(DevState* st, long long step, long long noise_ba
                                 long long noise_rows, cudaStream_t s);
 cudaError_t launch_set_stall(DevState* st, unsigned on, cudaStream_t s);
 
+// host != null (pinned memory, n_inst <= kFinDirect): the globals go there, and the status word to
+// *host_status, cleared in *st.
+constexpr int kFinDirect = 4;
 cudaError_t launch_finalize1d(const double* partials, const int* inst_item_begin,
                               const Inst1D* inst, int n_inst, double* glob, int per_item,
-                              cudaStream_t s);
+                              DevState* st, double* host, unsigned* host_status, cudaStream_t s);
 cudaError_t launch_advance_step(DevState* st, long long n, cudaStream_t s);
 
 }  // namespace lat

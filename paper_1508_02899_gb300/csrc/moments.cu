@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(1024) k_moments1d(const Mom1DArgs a, const int
         if (sizeof(T) == sizeof(double)) {
             Comp s0{0, 0}, s1{0, 0}, s2{0, 0};
             if (on) {
+#pragma unroll 4
                 for (int jj = 0; jj < nv; ++jj) {
                     const double v = __dmul_rn((double)(jj - J), in.dv);
                     const double fv = (double)f[(size_t)jj * in.nx + x];
@@ -67,6 +68,7 @@ __global__ void __launch_bounds__(1024) k_moments1d(const Mom1DArgs a, const int
             if (on && nv >= 5) {
                 // two half-columns, as the fused step epilogue sums them (ColumnSums2)
                 ColumnSums2 s2;
+#pragma unroll 8
                 for (int p = 1; p <= J; ++p) {
                     const float f0 = (float)f[(size_t)(p - 1) * in.nx + x];
                     const float f1 = (float)f[(size_t)(p - 1 + J) * in.nx + x];
@@ -109,7 +111,8 @@ __global__ void __launch_bounds__(1024) k_moments1d(const Mom1DArgs a, const int
 constexpr int kFinLanes = 8;
 
 __global__ void k_finalize1d(const double* partials, const int* begin, const Inst1D* inst,
-                             int n_inst, double* glob, int per_item) {
+                             int n_inst, double* glob, int per_item, DevState* st,
+                             unsigned* host_status) {
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * (32 / kFinLanes) + lane / kFinLanes;
     const int l = lane % kFinLanes;
@@ -134,6 +137,10 @@ __global__ void k_finalize1d(const double* partials, const int* begin, const Ins
         glob[i * 3 + 0] = nval(t0) * w;
         glob[i * 3 + 1] = nval(t1) * w;
         glob[i * 3 + 2] = nval(t2) * w;
+    }
+    if (host_status && threadIdx.x == 0) {
+        *host_status = st->status;
+        st->status = 0u;
     }
 }
 
@@ -236,11 +243,13 @@ cudaError_t launch_moments1d(int dtype, int block, int xpt, int grid, const Mom1
 
 cudaError_t launch_finalize1d(const double* partials, const int* inst_item_begin,
                               const Inst1D* inst, int n_inst, double* glob, int per_item,
-                              cudaStream_t s) {
+                              DevState* st, double* host, unsigned* host_status, cudaStream_t s) {
     if (n_inst <= 0) return cudaSuccess;
     const int groups = 32 / kFinLanes;
+    static_assert(kFinDirect <= 32 / kFinLanes, "one block writes the status");
     k_finalize1d<<<(n_inst + groups - 1) / groups, 32, 0, s>>>(partials, inst_item_begin, inst,
-                                                               n_inst, glob, per_item);
+                                                               n_inst, host ? host : glob, per_item, st,
+                                                               host ? host_status : nullptr);
     return cudaGetLastError();
 }
 

@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kMaxPlaces / 2, 2)
     const int par = (int)(step & 1);
     const float* fin = static_cast<const float*>(par ? a.f[1] : a.f[0]) + tile.off;
     float* fout = static_cast<float*>(par ? a.f[0] : a.f[1]) + tile.off;
-    const float* w_in = a.wflow + tile.xoff;
+    const float* w_in = static_cast<const float*>(a.wflow) + tile.xoff;
     const int tid = threadIdx.x;
     if (tid == 0) mbar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -362,8 +362,15 @@ __global__ void __launch_bounds__(kMaxPlaces / 2, 2)
 // tables (one per grid size, flow_basis's values): evaluated per column and step, as the one-step
 // kernels do, the eight sincospi would cost as much as a fifth of the sweeps.
 constexpr int kFlowGroup = 5;  // steps formed together
-__global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kstep, int T, float* W) {
-    extern __shared__ float amp[];  // [M][2 T], T rounded up to whole groups: A, B of each step
+template <typename F> struct Pair;
+template <> struct Pair<float> { using type = float2; };
+template <> struct Pair<double> { using type = double2; };
+
+template <typename F>
+__global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kstep, int T) {
+    using F2 = typename Pair<F>::type;
+    extern __shared__ double2 amp_raw[];
+    F* amp = reinterpret_cast<F*>(amp_raw);  // [M][2 T], T in whole groups: A, B of each step
     const int Tg = round_up(T, kFlowGroup);
     const int2 item = a.items[blockIdx.x];
     const Inst1D& in = a.inst[item.x];
@@ -374,7 +381,7 @@ __global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kste
     if (tid < 2 * M) {
         const long long at = (long long)item.x * 2 * M + tid;
         double v = a.amp[par * a.amp_stride + at];
-        float* row_q = amp + (tid < M ? tid : tid - M) * 2 * Tg + (tid < M ? 0 : 1);
+        F* row_q = amp + (tid < M ? tid : tid - M) * 2 * Tg + (tid < M ? 0 : 1);
         const long long row0 = step - a.st->noise_base, rows = a.st->noise_rows;
         const double e = in.ou_e, sg = in.ou_s;
         bool missing = false;
@@ -390,7 +397,7 @@ __global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kste
             }
 #pragma unroll
             for (int s = 0; s < kFlowGroup; ++s) {
-                row_q[2 * (s0 + s)] = (float)v;
+                row_q[2 * (s0 + s)] = F(v);
                 if (!a.frozen && s0 + s < T) v = __dadd_rn(__dmul_rn(v, e), __dmul_rn(sg, xi[s]));
             }
         }
@@ -401,39 +408,53 @@ __global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kste
         }
     }
     __syncthreads();
-    const float inv_dv = float(in.inv_dv), g = float(in.g);
-    const float J = float((a.nv - 1) / 2);
+    const F inv_dv = F(in.inv_dv), g = F(in.g);
+    const F J = F((a.nv - 1) / 2);
+    const F cf = a.scheme == LAT_SCHEME_KOREN ? F(1) + F(a.mu) : F(1);  // Eq. (cfl) of the scheme
     bool cfl = false;
     for (int x = item.y + tid; x < min(nx, item.y + a.tile); x += blockDim.x) {
-        const float2* basis = a.basis + a.basis_off[item.x] + x;
-        float* w = W + in.xoff + x;
+        const F2* basis = static_cast<const F2*>(a.basis) + a.basis_off[item.x] + x;
+        F* w = static_cast<F*>(a.wflow) + in.xoff + x;
 #pragma unroll 1
         for (int s0 = 0; s0 < T; s0 += kFlowGroup) {
-            float u[kFlowGroup];
-            const float v = a.flow_kind == LAT_FLOW_FIELD
-                                ? static_cast<const float*>(a.field)[in.xoff + x]
-                                : 0.f;
+            F u[kFlowGroup];
+            const F v = a.flow_kind == LAT_FLOW_FIELD
+                                ? static_cast<const F*>(a.field)[in.xoff + x]
+                            : F(0);
 #pragma unroll
             for (int s = 0; s < kFlowGroup; ++s) u[s] = v;
 #pragma unroll 8
             for (int m = 0; m < M; ++m) {
-                const float2 sc = __ldg(basis + (size_t)m * nx);
-                const float2* ab = reinterpret_cast<const float2*>(amp + m * 2 * Tg) + s0;
+                const F2 sc = __ldg(basis + (size_t)m * nx);
+                const F2* ab = reinterpret_cast<const F2*>(amp + m * 2 * Tg) + s0;
 #pragma unroll
                 for (int s = 0; s < kFlowGroup; ++s)
-                    u[s] = flow_add<float>(u[s], ab[s].x, ab[s].y, sc.x, sc.y);
+                    u[s] = flow_add<F>(u[s], ab[s].x, ab[s].y, sc.x, sc.y);
             }
 #pragma unroll
             for (int s = 0; s < kFlowGroup; ++s) {
                 if (s0 + s >= T) break;
-                const float ws = u[s] * inv_dv;
+                const F ws = u[s] * inv_dv;
                 w[(s0 + s) * a.total_x] = ws;
-                cfl |= g * (J + fabsf(ws)) > 1.f;
+                cfl |= cf * (g * (J + fabs(ws))) > F(1);
             }
         }
     }
     if (cfl) atomicOr(&a.st->status, ST_CFL);
 }
+
+}  // namespace
+
+cudaError_t launch_flow_steps(int dtype, const Step1DArgs& a, int kstep, int T, cudaStream_t s) {
+    const int M = a.flow_kind == LAT_FLOW_MODES ? a.nmodes : 0;
+    const int words = 2 * M * round_up(T, kFlowGroup), threads = std::min(256, a.tile);
+    if (dtype == LAT_F64)
+        k_flow_steps<double><<<a.item_end, threads, sizeof(double) * words, s>>>(a, kstep, T);
+    else k_flow_steps<float><<<a.item_end, threads, sizeof(float) * words, s>>>(a, kstep, T);
+    return cudaGetLastError();
+}
+
+namespace {
 
 template <int NV>
 cudaError_t launch_t(int T, int ntiles, int places, const Step1DArgs& a, const MultiTile* tiles,
@@ -445,9 +466,8 @@ cudaError_t launch_t(int T, int ntiles, int places, const Step1DArgs& a, const M
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const int M = a.flow_kind == LAT_FLOW_MODES ? a.nmodes : 0;
-    k_flow_steps<<<a.item_end, std::min(256, a.tile), sizeof(float) * 2 * M * round_up(T, kFlowGroup),
-                   s>>>(a, kstep, T, a.wflow);
+    cudaError_t e = launch_flow_steps(LAT_F32, a, kstep, T, s);
+    if (e != cudaSuccess) return e;
     const size_t smem = 4 * ((size_t)NV * Shape<NV>::kPitch + side_words(Shape<NV>::J, T, places));
     k_multi1d<NV><<<ntiles, places / 2, smem, s>>>(a, tiles, kstep, T, piped);
     return cudaGetLastError();

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(MaxThreads<T, NV>::value)
             const T g = T(in.g), r = T(in.r);
             const T* __restrict__ src = static_cast<const T*>(a.f[par]) + in.off;
             T* __restrict__ dst = static_cast<T*>(a.f[par ^ 1]) + in.off + x;
-            const T w = flow_at<T>(a, in, amp_ptr<T>(a, par, item.x), x) * T(in.inv_dv);
+            const T w = flow_w<T>(a, in, amp_ptr<T>(a, par, item.x), x);
             T f[NV];
             if (nx >= J) {
 #pragma unroll
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(MaxThreads<T, NV>::value)
                 [&](int jj, T v) { dst[(size_t)jj * nx] = v; });
             cfl_flag<T, J, LIM>(a, g, w);
         }
-        if (!a.dry && !a.frozen && a.flow_kind == LAT_FLOW_MODES && item.y == 0)
+        if (!a.dry && !a.frozen && !a.wpre && a.flow_kind == LAT_FLOW_MODES && item.y == 0)
             advance_amplitudes(a, item.x, in, step, par);
     }
 }
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(512) k_step1d_any(const Step1DArgs a, const in
             const T g = T(in.g), r = T(in.r);
             const T* __restrict__ src = static_cast<const T*>(a.f[par]) + in.off;
             T* __restrict__ dst = static_cast<T*>(a.f[par ^ 1]) + in.off + x;
-            const T w = flow_at<T>(a, in, amp_ptr<T>(a, par, item.x), x) * T(in.inv_dv);
+            const T w = flow_w<T>(a, in, amp_ptr<T>(a, par, item.x), x);
             sweep_column_any<T>(
                 NV, w, g, r,
                 [&](int jj) {
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(512) k_step1d_any(const Step1DArgs a, const in
                 [&](int jj, T v) { dst[(size_t)jj * nx] = v; });
             if (g * (T(J) + fabs(w)) > T(1)) atomicOr(&a.st->status, ST_CFL);
         }
-        if (!a.dry && !a.frozen && a.flow_kind == LAT_FLOW_MODES && item.y == 0)
+        if (!a.dry && !a.frozen && !a.wpre && a.flow_kind == LAT_FLOW_MODES && item.y == 0)
             advance_amplitudes(a, item.x, in, step, par);
     }
 }
@@ -356,13 +356,14 @@ __global__ void __launch_bounds__(PC1_THREADS) k_step1d_pc(const Step1DArgs a, c
 }
 
 // The flow's basis of one grid size: sin and cos of 2 pi k_m x / N_x, [m][x].
-__global__ void k_flow_basis(const Step1DArgs a, int inst, float2* out) {
+template <typename T, typename T2>
+__global__ void k_flow_basis(const Step1DArgs a, int inst, T2* out) {
     const Inst1D in = a.inst[inst];
-    const float two_over_nx = float(in.two_over_nx);
+    const T two_over_nx = T(in.two_over_nx);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.nmodes * in.nx;
          i += gridDim.x * blockDim.x) {
         const int m = i / in.nx;
-        flow_basis<float>(a.k[m], in, two_over_nx, i - m * in.nx, &out[i].x, &out[i].y);
+        flow_basis<T>(a.k[m], in, two_over_nx, i - m * in.nx, &out[i].x, &out[i].y);
     }
 }
 
@@ -568,8 +569,12 @@ cudaError_t launch_step1d(int dtype, int nv, int variant, int block, int slots, 
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_flow_basis(const Step1DArgs& a, int inst, int nx, float2* out, cudaStream_t s) {
-    k_flow_basis<<<(a.nmodes * nx + 255) / 256, 256, 0, s>>>(a, inst, out);
+cudaError_t launch_flow_basis(int dtype, const Step1DArgs& a, int inst, int nx, void* table,
+                              long long at, cudaStream_t s) {
+    const int grid = (a.nmodes * nx + 255) / 256;
+    if (dtype == LAT_F64)
+        k_flow_basis<double><<<grid, 256, 0, s>>>(a, inst, static_cast<double2*>(table) + at);
+    else k_flow_basis<float><<<grid, 256, 0, s>>>(a, inst, static_cast<float2*>(table) + at);
     return cudaGetLastError();
 }
 

@@ -29,6 +29,13 @@ struct Ops<double> {
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 };
 
+// max(v, 0) and min(v, 0).  FP64 by the sign bit: comparisons run on the FP64 pipe, which bounds the
+// FP64 kernels on this part (two operations per clock and SM).
+__device__ __forceinline__ float pos_part(float v) { return fmaxf(v, 0.f); }
+__device__ __forceinline__ float neg_part(float v) { return fminf(v, 0.f); }
+__device__ __forceinline__ double pos_part(double v) { return __double2hiint(v) < 0 ? 0.0 : v; }
+__device__ __forceinline__ double neg_part(double v) { return __double2hiint(v) < 0 ? v : 0.0; }
+
 // c a_j = (dt/dv) * (-(v_j - u)/tau_p) = g (w - j), g = dt/tau_p, w = u/dv
 template <typename T>
 __device__ __forceinline__ T cacc(T g, T w, int j) {
@@ -37,7 +44,7 @@ __device__ __forceinline__ T cacc(T g, T w, int j) {
 // c F_{j+1/2} = (c a_j)^+ f_j + (c a_{j+1})^- f_{j+1}   (cell-centred upwind)
 template <typename T>
 __device__ __forceinline__ T dflux(T caj, T can, T fj, T fn) {
-    return Ops<T>::fma(fmax(caj, T(0)), fj, Ops<T>::mul(fmin(can, T(0)), fn));
+    return Ops<T>::fma(pos_part(caj), fj, Ops<T>::mul(neg_part(can), fn));
 }
 
 // Sliding-window sweep of one column.  get(jj) returns f*(x, jj - J); put(jj, v) stores.
@@ -165,8 +172,8 @@ __device__ __forceinline__ void sweep_column_lim(T w, T g, T r, T mu, const Get&
         if (k < NV) {
             x[k] = get(k);
             const T ca = cacc<T>(g, w, k - J);
-            P0[k] = O::mul(fmax(ca, T(0)), x[k]);
-            M0[k] = O::mul(fmin(ca, T(0)), x[k]);
+            P0[k] = O::mul(pos_part(ca), x[k]);
+            M0[k] = O::mul(neg_part(ca), x[k]);
         }
         if (k - 2 >= 0 && k - 2 <= NV - 2) F0[k - 1] = lim_face<T, NV>(P0, M0, k - 2, mu);
         if (k - 2 >= 0 && k - 2 < NV) {
@@ -175,8 +182,8 @@ __device__ __forceinline__ void sweep_column_lim(T w, T g, T r, T mu, const Get&
             const T Fr = j == NV - 1 ? T(0) : F0[j + 1];
             y[j] = O::sub(x[j], O::sub(Fr, Fl));
             const T ca = cacc<T>(g, w, j - J);
-            P1[j] = O::mul(fmax(ca, T(0)), y[j]);
-            M1[j] = O::mul(fmin(ca, T(0)), y[j]);
+            P1[j] = O::mul(pos_part(ca), y[j]);
+            M1[j] = O::mul(neg_part(ca), y[j]);
         }
         if (k - 4 >= 0 && k - 4 <= NV - 2) F1[k - 3] = lim_face<T, NV>(P1, M1, k - 4, mu);
         if (k - 4 >= 0 && k - 4 < NV) {
@@ -276,6 +283,14 @@ __device__ __forceinline__ T flow_at(const Step1DArgs& a, const Inst1D& in, cons
         u = flow_add<T>(u, __ldg(amp + m), __ldg(amp + M + m), s, c);
     }
     return u;
+}
+
+// u / dv of column x: formed here, or taken from the array the flow kernel of multi1d.cu filled
+// (which then also advances the amplitudes).
+template <typename T>
+__device__ __forceinline__ T flow_w(const Step1DArgs& a, const Inst1D& in, const T* amp, int x) {
+    if (a.wpre) return static_cast<const T*>(a.wpre)[in.xoff + x];
+    return flow_at<T>(a, in, amp, x) * T(in.inv_dv);
 }
 
 // Exact Ornstein-Uhlenbeck update of the instance's amplitudes (Eq. A1d), t_n -> t_{n+1}.
