@@ -808,12 +808,42 @@ __device__ __forceinline__ double to_d(T v) { return (double)v; }
 
 constexpr int kMom2DWarps = 8;  // warps per moment block (256 threads)
 
+// f of one cell (both lanes the same) or of two neighbouring cells.
+template <typename T, bool PAIR>
+__device__ __forceinline__ f2 load_cells(const T* p) {
+    if constexpr (!PAIR) {
+        const float v = (float)*p;
+        return pk(v, v);
+    } else if constexpr (sizeof(T) == 4) {
+        return *reinterpret_cast<const f2*>(p);
+    } else {
+        T h[2];
+        *reinterpret_cast<unsigned*>(h) = *reinterpret_cast<const unsigned*>(p);
+        return pk((float)h[0], (float)h[1]);
+    }
+}
+// FComp::add_exact and FComp::merge in two lanes
+__device__ __forceinline__ void two_sum_add(f2& s, f2& c, f2 x) {
+    const f2 t = add2(s, x);
+    const f2 bb = sub2(t, s);
+    const f2 e = add2(sub2(s, sub2(t, bb)), sub2(x, bb));
+    s = t;
+    c = sub2(c, e);
+}
+__device__ __forceinline__ void two_sum_merge(f2& s, f2& c, f2 os, f2 oc) {
+    const f2 t = add2(s, os);
+    const f2 bb = sub2(t, s);
+    const f2 e = add2(sub2(s, sub2(t, bb)), sub2(os, bb));
+    s = t;
+    c = sub2(add2(c, oc), e);
+}
+
 // Per cell: sums over the N_v^2 velocity cells of f, jx f, jy f, (jx^2 + jy^2) f; per-cell moments
 // and one compensated partial per block: partials[block][4][2] (warps fold in warp order).
 //   FP64 storage: Neumaier FP64 throughout.
 //   FP32 / FP16 / BF16 storage: FP32 Kahan sums per cell and across a thread's cells and the
 //   warp (exact integer weights); FP64 from the warp partials on (FP64 is slow on this GPU).
-template <typename T>
+template <typename T, bool PAIR = false>
 __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* scales, int nv,
                                                    int nx, int ny, double dv, double* rho,
                                                    double* mv, double* mv2, double* partials,
@@ -822,6 +852,7 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
     const int J = (nv - 1) / 2;
     const long long ncell = (long long)nx * ny;
     const double dv2 = __dmul_rn(dv, dv);
+    const f2 zero2 = opaque2(0ull);  // keeps a packed product from fusing with an addition
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double* p = partials + (size_t)blockIdx.x * 8;  // one partial per block
     bool bad = false;
@@ -868,47 +899,59 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
         // per cell: the mass exact up to the roundings of its compensation (TwoSum per velocity
         // row, rows merged); the weighted sums one FMA per value (the integer weights exact, the
         // product exact inside the FMA), error at most (N_v^2 - 1) u of the sum of
-        // |weight f|, u = 2^-24
+        // |weight f|, u = 2^-24.  PAIR: two neighbouring cells per thread in the lanes of f32x2
+        // pairs, one load for both (1024^2 x 33^2: FP16 1.34 -> 0.60 ms, a scalar thread per cell
+        // is bound by its instructions).
         FComp t[4];
-        for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < ncell;
-             c += (long long)gridDim.x * blockDim.x) {
-            FComp s0;
-            float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        const long long nunit = PAIR ? ncell / 2 : ncell;
+        for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nunit;
+             q += (long long)gridDim.x * blockDim.x) {
+            const long long c = PAIR ? 2 * q : q;
             // scales of this cell's row: [jy][jx padded]
             const float* sc_c = scales ? scales + (size_t)(c / nx) * nv * nv_padded(nv) : nullptr;
+            f2 S = 0ull, C = 0ull, s1 = 0ull, s2 = 0ull, s3 = 0ull;  // mass (sum, -error); weighted
             for (int jy = 0; jy < nv; ++jy) {
                 const float fy = (float)(jy - J);
                 const float fy2 = fy * fy;
-                FComp ey;         // sum f of the velocity row
-                float ex = 0.f;   // sum jx f of the velocity row
-#pragma unroll 4
+                f2 rs = 0ull, rc = 0ull, ex = 0ull;  // the velocity row: mass, sum jx f
+                const T* fr = f + (size_t)jy * nv * ncell + c;
+#pragma unroll 8
                 for (int jx = 0; jx < nv; ++jx) {
                     const float fx = (float)(jx - J);
-                    const size_t plane = (size_t)jy * nv + jx;
-                    float fvv = (float)f[plane * ncell + c];
-                    if (sc_c) fvv = fvv * sc_c[jy * nv_padded(nv) + jx];  // exact: powers of two
-                    ey.add_exact(fvv);
-                    ex = __fmaf_rn(fx, fvv, ex);
-                    s3 = __fmaf_rn(__fmaf_rn(fx, fx, fy2), fvv, s3);
+                    f2 v = load_cells<T, PAIR>(fr + (size_t)jx * ncell);
+                    if (sc_c) {  // exact: powers of two
+                        const float sv = sc_c[jy * nv_padded(nv) + jx];
+                        v = fma2(v, pk(sv, sv), zero2);
+                    }
+                    two_sum_add(rs, rc, v);
+                    ex = fma2(pk(fx, fx), v, ex);
+                    const float w3 = __fmaf_rn(fx, fx, fy2);
+                    s3 = fma2(pk(w3, w3), v, s3);
                 }
-                s0.merge(ey);
-                s1 = __fadd_rn(s1, ex);
-                s2 = __fmaf_rn(fy, __fsub_rn(ey.s, ey.c), s2);
+                two_sum_merge(S, C, rs, rc);
+                s1 = add2(s1, ex);
+                s2 = fma2(pk(fy, fy), sub2(rs, rc), s2);
             }
-            bad |= !isfinite(s0.s) || !isfinite(s3);
-            if (rho || mv || mv2) {  // FP64 per cell only when asked for (FP64 is slow here)
-                const double m0 = nval(s0.to_comp(1.0));
-                if (rho) rho[c] = m0 * dv2;
-                if (mv) {
-                    mv[c] = m0 != 0.0 ? __dmul_rn((double)s1, dv) / m0 : 0.0;
-                    mv[ncell + c] = m0 != 0.0 ? __dmul_rn((double)s2, dv) / m0 : 0.0;
+#pragma unroll
+            for (int e = 0; e < (PAIR ? 2 : 1); ++e) {
+                const FComp s0{e ? hi(S) : lo(S), e ? hi(C) : lo(C)};
+                const float m1 = e ? hi(s1) : lo(s1), m2 = e ? hi(s2) : lo(s2),
+                            m3 = e ? hi(s3) : lo(s3);
+                bad |= !isfinite(s0.s) || !isfinite(m3);
+                if (rho || mv || mv2) {  // FP64 per cell only when asked for (FP64 is slow here)
+                    const double m0 = nval(s0.to_comp(1.0));
+                    if (rho) rho[c + e] = m0 * dv2;
+                    if (mv) {
+                        mv[c + e] = m0 != 0.0 ? __dmul_rn((double)m1, dv) / m0 : 0.0;
+                        mv[ncell + c + e] = m0 != 0.0 ? __dmul_rn((double)m2, dv) / m0 : 0.0;
+                    }
+                    if (mv2) mv2[c + e] = m0 != 0.0 ? __dmul_rn((double)m3, dv2) / m0 : 0.0;
                 }
-                if (mv2) mv2[c] = m0 != 0.0 ? __dmul_rn((double)s3, dv2) / m0 : 0.0;
+                t[0].merge(s0);
+                t[1].merge(FComp{m1, 0.f});
+                t[2].merge(FComp{m2, 0.f});
+                t[3].merge(FComp{m3, 0.f});
             }
-            t[0].merge(s0);
-            t[1].merge(FComp{s1, 0.f});
-            t[2].merge(FComp{s2, 0.f});
-            t[3].merge(FComp{s3, 0.f});
         }
         for (int q = 0; q < 4; ++q) warp_reduce(t[q]);
         __shared__ FComp wsum[kMom2DWarps][4];
@@ -1755,18 +1798,20 @@ int copy_globals(Ctx2D* c, double* globals, bool wait, cudaStream_t s) {
 int ctx2d_moments(Ctx2D* c, const void* f, int cur, double* rho, double* mean_v,
                   double* mean_v2, double* globals, bool wait, cudaStream_t s) {
     const float* sc = c->half ? c->d_sc + (size_t)cur * c->nlines : nullptr;
+    auto run = [&](auto kernel) {
+        kernel<<<c->mom_blocks, 32 * kMom2DWarps, 0, s>>>(f, sc, c->nv, c->nx, c->ny, c->dv, rho,
+                                                         mean_v, mean_v2, c->d_partials, c->st);
+    };
+    // pairs of cells where a pair lies in one grid row and is aligned
+    const bool pair = c->nx % 2 == 0 && (uintptr_t)f % 8 == 0;
     if (c->dtype == LAT_F16)
-        k_moments2d<__half><<<c->mom_blocks, 32 * kMom2DWarps, 0, s>>>(f, sc, c->nv, c->nx, c->ny, c->dv,
-                                                         rho, mean_v, mean_v2, c->d_partials, c->st);
+        pair ? run(k_moments2d<__half, true>) : run(k_moments2d<__half>);
     else if (c->dtype == LAT_BF16)
-        k_moments2d<__nv_bfloat16><<<c->mom_blocks, 32 * kMom2DWarps, 0, s>>>(f, sc, c->nv, c->nx, c->ny, c->dv,
-                                                         rho, mean_v, mean_v2, c->d_partials, c->st);
+        pair ? run(k_moments2d<__nv_bfloat16, true>) : run(k_moments2d<__nv_bfloat16>);
     else if (c->dtype == LAT_F64)
-        k_moments2d<double><<<c->mom_blocks, 32 * kMom2DWarps, 0, s>>>(f, nullptr, c->nv, c->nx, c->ny, c->dv,
-                                                         rho, mean_v, mean_v2, c->d_partials, c->st);
+        run(k_moments2d<double>);
     else
-        k_moments2d<float><<<c->mom_blocks, 32 * kMom2DWarps, 0, s>>>(f, nullptr, c->nv, c->nx, c->ny, c->dv,
-                                                        rho, mean_v, mean_v2, c->d_partials, c->st);
+        pair ? run(k_moments2d<float, true>) : run(k_moments2d<float>);
     CK2(cudaGetLastError());
     k_finalize2d<<<1, kFin2DThreads, 0, s>>>(c->d_partials, c->mom_blocks,
                                              c->dx * c->dx * c->dv * c->dv, c->d_glob);

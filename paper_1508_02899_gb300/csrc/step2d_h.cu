@@ -565,15 +565,34 @@ __global__ void __launch_bounds__(256) k_encode(const float* src, S* f, const fl
     if (bad) atomicOr(&st->status, ST_OVERFLOW);
 }
 
-template <typename S>
+// One warp per line.  VEC: 16-byte loads and stores (N_x a multiple of 8, both arrays aligned to 16
+// bytes).  Bound by HBM (6 bytes per value); one value per thread with its 64-bit divisions took
+// 4.65 ms for 1024^2 x 33^2 (with the moments, 3.3 ms of a 25.8 ms batch of six steps saved).
+template <typename S, bool VEC>
 __global__ void __launch_bounds__(256) k_decode(const S* f, const float* sc, float* dst,
-                                                long long n, int nx, int ny, int nv) {
-    const long long ncell = (long long)nx * ny;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int p = (int)(i / ncell);
-        const int y = (int)((i % ncell) / nx);
-        dst[i] = __fmul_rn(HTraits<S>::dec(f[i]), sc[scale_index(p, y, nv)]);
+                                                long long nlines, int nx, int ny, int nv) {
+    const int lane = threadIdx.x & 31;
+    const long long w0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long l = w0; l < nlines; l += nw) {
+        const float s = sc[scale_index((int)(l / ny), (int)(l % ny), nv)];
+        const S* row = f + (size_t)l * nx;
+        float* out = dst + (size_t)l * nx;
+        if constexpr (VEC) {
+#pragma unroll 4
+            for (int c = lane; c < nx / 8; c += 32) {
+                const uint4 v = reinterpret_cast<const uint4*>(row)[c];
+                const S* h = reinterpret_cast<const S*>(&v);
+                float4 o[2];
+                float* q = reinterpret_cast<float*>(o);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) q[e] = __fmul_rn(HTraits<S>::dec(h[e]), s);
+                reinterpret_cast<float4*>(out)[2 * c] = o[0];
+                reinterpret_cast<float4*>(out)[2 * c + 1] = o[1];
+            }
+        } else {
+            for (int x = lane; x < nx; x += 32) out[x] = __fmul_rn(HTraits<S>::dec(row[x]), s);
+        }
     }
 }
 
@@ -756,18 +775,23 @@ cudaError_t launch_encode_h(int dtype, const float* src, void* f, float* sc, uns
     return launch_linemax_h(dtype, f, sc, mx, nv, nx, ny, s);
 }
 
+namespace {
+template <typename S>
+void decode_t(const void* f, const float* sc, float* dst, int nv, int nx, int ny, cudaStream_t s) {
+    const long long nl = (long long)nv * nv * ny;
+    const int grid = (int)std::min<long long>((nl + 7) / 8, 1 << 20);
+    const bool vec = nx % 8 == 0 && ((uintptr_t)f | (uintptr_t)dst) % 16 == 0;
+    const S* src = static_cast<const S*>(f);
+    if (vec) k_decode<S, true><<<grid, 256, 0, s>>>(src, sc, dst, nl, nx, ny, nv);
+    else k_decode<S, false><<<grid, 256, 0, s>>>(src, sc, dst, nl, nx, ny, nv);
+}
+}  // namespace
+
 cudaError_t launch_decode_h(int dtype, const void* f, const float* sc, float* dst, int nv, int nx,
                             int ny, cudaStream_t s) {
-    const long long n = (long long)nv * nv * nx * ny;
-    const int grid = grid_for(n, 256);
-    if (dtype == LAT_F16)
-        k_decode<__half><<<grid, 256, 0, s>>>(static_cast<const __half*>(f), sc, dst, n, nx, ny,
-                                              nv);
-    else if (dtype == LAT_BF16)
-        k_decode<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(f), sc, dst,
-                                                     n, nx, ny, nv);
-    else
-        return cudaErrorInvalidValue;
+    if (dtype == LAT_F16) decode_t<__half>(f, sc, dst, nv, nx, ny, s);
+    else if (dtype == LAT_BF16) decode_t<__nv_bfloat16>(f, sc, dst, nv, nx, ny, s);
+    else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
