@@ -20,6 +20,16 @@ __device__ __forceinline__ void nadd(Comp& a, double x) {
     else a.c = __dadd_rn(a.c, __dadd_rn(__dsub_rn(x, t), a.s));
     a.s = t;
 }
+// The same with the magnitudes compared as integers (the FP64 comparison takes the FP64 pipe); no
+// NaN is told apart, which only decides between two NaN results.
+__device__ __forceinline__ void nadd_fast(Comp& a, double x) {
+    const double t = __dadd_rn(a.s, x);
+    const long long ia = __double_as_longlong(a.s) & 0x7fffffffffffffffll,
+                    ix = __double_as_longlong(x) & 0x7fffffffffffffffll;
+    const double big = ia >= ix ? a.s : x, small = ia >= ix ? x : a.s;
+    a.c = __dadd_rn(a.c, __dadd_rn(__dsub_rn(big, t), small));
+    a.s = t;
+}
 __device__ __forceinline__ void nmerge(Comp& a, const Comp& b) {
     nadd(a, b.s);
     a.c = __dadd_rn(a.c, b.c);

@@ -65,7 +65,7 @@ struct Flow2DArgs {
     int frozen, dry;
 };
 
-// ---- plain-load kernel (any N_x, N_y; FP32 or FP64) -----------------------------------------
+// ---- plain-load kernel (any N_x, N_y) -------------------------------------------------------
 template <typename T, int NV>
 __global__ void __launch_bounds__(TW) k_step2d_plain(const Step2DArgs a, int kstep) {
     const long long step = a.st->step + kstep;
@@ -857,31 +857,46 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
     double* p = partials + (size_t)blockIdx.x * 8;  // one partial per block
     bool bad = false;
     if constexpr (sizeof(T) == sizeof(double)) {
+        // A block takes 32 cells at a time, warp w their velocity rows w, w + 8, ..; warp 0 merges
+        // the warps in order (128^2 cells with a thread each are 64 blocks: 2.35 ms).
+        __shared__ Comp part[kMom2DWarps - 1][4][32];
         Comp t[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-        for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < ncell;
-             c += (long long)gridDim.x * blockDim.x) {
+        for (long long c0 = (long long)blockIdx.x * 32; c0 < ncell; c0 += (long long)gridDim.x * 32) {
+            const long long c = c0 + lane;
             Comp s[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-            for (int jy = 0; jy < nv; ++jy) {
-                const double vy = __dmul_rn((double)(jy - J), dv);
-                for (int jx = 0; jx < nv; ++jx) {
-                    const double vx = __dmul_rn((double)(jx - J), dv);
-                    const size_t plane = (size_t)jy * nv + jx;
-                    const double fvv = to_d(f[plane * ncell + c]);
-                    bad |= !isfinite(fvv);
-                    nadd(s[0], fvv);
-                    nadd(s[1], __dmul_rn(vx, fvv));
-                    nadd(s[2], __dmul_rn(vy, fvv));
-                    nadd(s[3], __dmul_rn(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)), fvv));
+            if (c < ncell) {
+                for (int jy = warp; jy < nv; jy += kMom2DWarps) {
+                    const double vy = __dmul_rn((double)(jy - J), dv);
+                    const double vy2 = __dmul_rn(vy, vy);
+#pragma unroll 4
+                    for (int jx = 0; jx < nv; ++jx) {
+                        const double vx = __dmul_rn((double)(jx - J), dv);
+                        const size_t plane = (size_t)jy * nv + jx;
+                        const double fvv = to_d(f[plane * ncell + c]);
+                        bad |= !isfinite(fvv);
+                        nadd_fast(s[0], fvv);
+                        nadd_fast(s[1], __dmul_rn(vx, fvv));
+                        nadd_fast(s[2], __dmul_rn(vy, fvv));
+                        nadd_fast(s[3], __dmul_rn(__dadd_rn(__dmul_rn(vx, vx), vy2), fvv));
+                    }
                 }
+                if (warp > 0)
+                    for (int q = 0; q < 4; ++q) part[warp - 1][q][lane] = s[q];
             }
-            const double m0 = nval(s[0]);
-            if (rho) rho[c] = m0 * dv * dv;
-            if (mv) {
-                mv[c] = m0 != 0.0 ? nval(s[1]) / m0 : 0.0;
-                mv[ncell + c] = m0 != 0.0 ? nval(s[2]) / m0 : 0.0;
+            __syncthreads();
+            if (warp == 0 && c < ncell) {
+                for (int w = 0; w < kMom2DWarps - 1; ++w)
+                    for (int q = 0; q < 4; ++q) nmerge(s[q], part[w][q][lane]);
+                const double m0 = nval(s[0]);
+                if (rho) rho[c] = m0 * dv * dv;
+                if (mv) {
+                    mv[c] = m0 != 0.0 ? nval(s[1]) / m0 : 0.0;
+                    mv[ncell + c] = m0 != 0.0 ? nval(s[2]) / m0 : 0.0;
+                }
+                if (mv2) mv2[c] = m0 != 0.0 ? nval(s[3]) / m0 : 0.0;
+                for (int q = 0; q < 4; ++q) nmerge(t[q], s[q]);
             }
-            if (mv2) mv2[c] = m0 != 0.0 ? nval(s[3]) / m0 : 0.0;
-            for (int q = 0; q < 4; ++q) nmerge(t[q], s[q]);
+            __syncthreads();
         }
         for (int q = 0; q < 4; ++q) warp_reduce(t[q]);
         __shared__ Comp wsum[kMom2DWarps][4];
@@ -1232,12 +1247,11 @@ bool pc_supported(int nv) {
     }
 }
 
-cudaError_t launch_step2d(int dtype, int nv, bool ring, int chunks, int pcv, int grid,
+cudaError_t launch_step2d(int nv, bool ring, int chunks, int pcv, int grid,
                           const Step2DArgs& a, int k, cudaStream_t s) {
     switch (nv) {
 #define X(n)                                                                   \
     case n:                                                                    \
-        if (dtype == LAT_F64) return launch_plain<double, n>(grid, a, k, s);   \
         if (ring && pcv) return launch_pc_v<n>(pcv, grid, a, k, s);            \
         if (ring) return launch_ring_c<n>(chunks, grid, a, k, s);              \
         return launch_plain<float, n>(grid, a, k, s);
@@ -1507,8 +1521,10 @@ int enqueue2d(Ctx2D* c, void* const f[2], int n, cudaStream_t s, int dry) {
             const Step2DHArgs ha = half_args(c, a);
             CK2(launch_scale2d(c->nv, c->ny, ha, k, s));
             CK2(launch_step2d_h(c->dtype, c->nv, c->ring ? c->pcv : 0, grid, ha, k, s));
+        } else if (c->dtype == LAT_F64) {
+            CK2(launch_step2d_f64(c->nv, c->sm_count, a, k, s));
         } else {
-            CK2(launch_step2d(c->dtype, c->nv, c->ring, c->chunks, c->pcv, grid, a, k, s));
+            CK2(launch_step2d(c->nv, c->ring, c->chunks, c->pcv, grid, a, k, s));
         }
     }
     if (!dry) {
@@ -1575,7 +1591,9 @@ int ctx2d_create(Ctx2D** out, const lat_grid* g, DevState* st, int sm_count, cud
     c->pcv = c->ring && pc_ok(c) ? (half ? 6 : 9) : 0;
     if (half && !c->pcv) c->ring = false;
     const long long ncell = (long long)c->nx * c->ny;
-    c->mom_blocks = (int)std::min<long long>((ncell + 255) / 256, 8LL * sm_count);
+    // a thread per cell, or (FP64) a block per 32 cells
+    const int mom_cells = c->dtype == LAT_F64 ? 32 : 256;
+    c->mom_blocks = (int)std::min<long long>((ncell + mom_cells - 1) / mom_cells, 8LL * sm_count);
     // room for the moment kernel's block partials or the fused step's warp partials
     const size_t npart = std::max<size_t>(c->mom_blocks, (size_t)8 * sm_count * (TW / 32));
     if (cudaMalloc(&c->d_partials, sizeof(double) * 8 * npart) != cudaSuccess ||
