@@ -613,8 +613,10 @@ __global__ void k_pack(const float* P, unsigned char* img) {
 //   [dz2 | dz1]^T [h1 1 0]  -> rows 0..63: dW2^T with db2 in column 64   (M = 128, N = 80),
 //   [dz2 | dz1]^T X         -> rows 64..127: dW1^T, db1 = column 15      (M = 128, N = 16),
 //   [h2 1 0]^T dz3          -> rows 0..63: dW3, row 64: db3               (M = 128, N = 16).
-// The weight-gradient operands are the tile's values transposed (rows = features, K = cells):
-// every thread scatters its cell's BF16 values into column `cell` of those K-major tiles.
+// The weight-gradient operands are the very tiles of the network's MMAs, rows = cells: read with the
+// features as the M and N index (contiguous in memory, "MN-major" operands) and the cells as K.  So
+// nothing is transposed, and two CTAs fit an SM (with transposed copies, 270 conflicting 2-byte stores
+// per cell and one CTA per SM, the kernel took 2.40 ms at 256^2 x 9^2).
 // Backward B operands, packed from the FP32 parameters after the forward image:
 //   B4 [n = i][k = o] = W3[i][o] (o < 2),  B5 [n = i][k = j] = W2[i][j],  B6 [n = q][k = i] = W1[q][i].
 constexpr int kB4 = kImage;                   // N 64 x K 16 (2 KB)
@@ -651,31 +653,19 @@ constexpr int kBA3 = kBA2 + 128 * kK2 * 2;              // [h2 1 0] [128][80]
 constexpr int kBZ3 = kBA3 + 128 * kK2 * 2;              // dz3      [128][16]
 constexpr int kBZ2 = kBZ3 + 128 * 16 * 2;               // dz2      [128][64]
 constexpr int kBZ1 = kBZ2 + 128 * 64 * 2;               // dz1      [128][64]
-constexpr int kTDZ = kBZ1 + 128 * 64 * 2;               // [dz2 | dz1]^T [128][128 cells]
-constexpr int kTH1 = kTDZ + 128 * 128 * 2;              // [h1 1 0]^T    [80][128]
-constexpr int kTX = kTH1 + 80 * 128 * 2;                // X^T           [16][128]
-constexpr int kTH2 = kTX + 16 * 128 * 2;                // [h2 1 0]^T    [128][128]
-constexpr int kTZ3 = kTH2 + 128 * 128 * 2;              // dz3^T         [16][128]
-constexpr int kBBar = kTZ3 + 16 * 128 * 2;
+constexpr int kBBar = kBZ1 + 128 * 64 * 2;
 constexpr int kBSmem = kBBar + 16;
-static_assert(kBSmem <= 227 * 1024, "backward kernel's shared memory");
+static_assert(2 * (kBSmem + 1024) <= 228 * 1024, "two backward CTAs per SM");
+static_assert(kBA3 + 16 * 2048 <= kBBar && kBZ1 - kBZ2 == 8 * 2048,
+              "128 features from A3 on, and from Z2 on, in steps of 2048 bytes");
 // tensor memory: per-tile accumulator, then the three weight-gradient accumulators
 constexpr int kBTmemCols = 256;
 constexpr int kTD = 0, kTW2 = 64, kTW1 = 144, kTW3 = 160;
 
-__device__ __forceinline__ void put_bf16(unsigned char* tile, unsigned off, float v) {
-    *reinterpret_cast<__nv_bfloat16*>(tile + off) = __float2bfloat16_rn(v);
-}
-__device__ __forceinline__ void put_bits(unsigned char* tile, unsigned off, unsigned short b) {
-    *reinterpret_cast<unsigned short*>(tile + off) = b;
-}
-
-// ReLU of 64 accumulator columns of this thread's row (cell r) into row r of A (as epilogue64)
-// and into column r of the transposed tile T (rows = features, `trows` rows); bit k of mask is
-// set where column k was positive.
-__device__ __forceinline__ void epilogue64_t(unsigned taddr, unsigned char* A, unsigned char* T,
-                                             int trows, int r, unsigned (&mask)[2]) {
-    mask[0] = mask[1] = 0u;
+// The product of a backward MMA (64 accumulator columns of cell r), masked by the ReLU of the
+// activations H (row r of their tile: positive or zero), as BF16 into row r of D.
+__device__ __forceinline__ void epilogue64_mask(unsigned taddr, const unsigned char* H,
+                                                unsigned char* D, int r) {
 #pragma unroll
     for (int c0 = 0; c0 < 64; c0 += 32) {
         unsigned v[2][16];
@@ -685,47 +675,14 @@ __device__ __forceinline__ void epilogue64_t(unsigned taddr, unsigned char* A, u
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
             const unsigned* u = v[g >> 1] + 8 * (g & 1);
+            const uint4 h4 = *reinterpret_cast<const uint4*>(H + tile_off(r, c0 + 8 * g, 128));
+            const unsigned h[4] = {h4.x, h4.y, h4.z, h4.w};
             unsigned w[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float a = __uint_as_float(u[2 * e]), b = __uint_as_float(u[2 * e + 1]);
-                w[e] = pack_relu_bf16(a, b);
-                const int col = c0 + 8 * g + 2 * e;
-                mask[col >> 5] |= (a > 0.f ? 1u : 0u) << (col & 31);
-                mask[col >> 5] |= (b > 0.f ? 1u : 0u) << ((col + 1) & 31);
-                put_bits(T, tile_off(col, r, trows), (unsigned short)(w[e] & 0xffffu));
-                put_bits(T, tile_off(col + 1, r, trows), (unsigned short)(w[e] >> 16));
-            }
-            *reinterpret_cast<uint4*>(A + tile_off(r, c0 + 8 * g, 128)) =
-                make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    }
-}
-
-// The masked product of a backward MMA (64 accumulator columns of cell r) as BF16 into row r
-// of D and into rows row0 .. row0 + 63 of column r of the transposed tile T (128 rows).
-__device__ __forceinline__ void epilogue64_mask(unsigned taddr, const unsigned (&mask)[2],
-                                                bool on, unsigned char* D, unsigned char* T,
-                                                int row0, int r) {
-#pragma unroll
-    for (int c0 = 0; c0 < 64; c0 += 32) {
-        unsigned v[2][16];
-        tmem_ld16(taddr + c0, v[0]);
-        tmem_ld16(taddr + c0 + 16, v[1]);
-        tmem_wait();
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const unsigned* u = v[g >> 1] + 8 * (g & 1);
-            unsigned w[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int col = c0 + 8 * g + 2 * e;
-                const bool ma = on && ((mask[col >> 5] >> (col & 31)) & 1u);
-                const bool mb = on && ((mask[(col + 1) >> 5] >> ((col + 1) & 31)) & 1u);
-                w[e] = pack_bf16(ma ? __uint_as_float(u[2 * e]) : 0.f,
-                                 mb ? __uint_as_float(u[2 * e + 1]) : 0.f);
-                put_bits(T, tile_off(row0 + col, r, 128), (unsigned short)(w[e] & 0xffffu));
-                put_bits(T, tile_off(row0 + col + 1, r, 128), (unsigned short)(w[e] >> 16));
+                const __nv_bfloat162 hp = *reinterpret_cast<const __nv_bfloat162*>(&h[e]);
+                w[e] = pack_bf16(__uint_as_float(u[2 * e]), __uint_as_float(u[2 * e + 1])) &
+                       __hgt2_mask(hp, __nv_bfloat162(__float2bfloat16(0.f), __float2bfloat16(0.f)));
             }
             *reinterpret_cast<uint4*>(D + tile_off(r, c0 + 8 * g, 128)) =
                 make_uint4(w[0], w[1], w[2], w[3]);
@@ -741,12 +698,22 @@ __device__ __forceinline__ void mma_k(unsigned dt, unsigned a, unsigned a_lbo, u
             idesc_n(n_out), (acc || kk > 0) ? 1 : 0);
 }
 
-// One CTA of 128 threads per SM (about 199 KB of shared memory) walks tiles of 128 phase cells
+// D (+)= A^T B summed over a tile's 128 cells: A and B are tiles of 128 rows (cells), their columns the
+// M = 128 and N indices of D (8 K-steps of 16 cells; 128 bytes between groups of 8 cells, 2048 between
+// groups of 8 columns).
+__device__ __forceinline__ void mma_cells(unsigned dt, unsigned a, unsigned b, unsigned n_out,
+                                          bool acc) {
+    for (int kk = 0; kk < 8; ++kk)
+        mma(dt, sdesc(a + kk * 256, 128, 2048), sdesc(b + kk * 256, 128, 2048),
+            idesc_n(n_out) | (1u << 15) | (1u << 16), (acc || kk > 0) ? 1 : 0);
+}
+
+// Two CTAs of 128 threads per SM (about 107 KB of shared memory each) walk tiles of 128 phase cells
 // in storage order; thread t owns cell t of the tile.  Outputs as learn.cu's k_mlp_bwd: cxy,
 // lfs, dX9 per cell, lrho (atomic per spatial cell) and the parameter gradient (atomic, once per
 // CTA at the end).
 template <int NV>
-__global__ void __launch_bounds__(128, 1) k_mlp_bwd_tc(const LearnBwdArgs b,
+__global__ void __launch_bounds__(128, 2) k_mlp_bwd_tc(const LearnBwdArgs b,
                                                       const unsigned char* image) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const LearnArgs& a = b.fw;
@@ -757,11 +724,6 @@ __global__ void __launch_bounds__(128, 1) k_mlp_bwd_tc(const LearnBwdArgs b,
     unsigned char* Z3 = sm + kBZ3;
     unsigned char* Z2 = sm + kBZ2;
     unsigned char* Z1 = sm + kBZ1;
-    unsigned char* TDZ = sm + kTDZ;
-    unsigned char* TH1 = sm + kTH1;
-    unsigned char* TX = sm + kTX;
-    unsigned char* TH2 = sm + kTH2;
-    unsigned char* TZ3 = sm + kTZ3;
     uint64_t* bar = reinterpret_cast<uint64_t*>(sm + kBBar);
     unsigned* tslot = reinterpret_cast<unsigned*>(sm + kBBar + 8);
     const int t = threadIdx.x, warp = t >> 5;
@@ -775,9 +737,6 @@ __global__ void __launch_bounds__(128, 1) k_mlp_bwd_tc(const LearnBwdArgs b,
         *reinterpret_cast<uint4*>(A3 + tile_off(t, 64, 128)) = one;
         *reinterpret_cast<uint4*>(A3 + tile_off(t, 72, 128)) = zero;
         *reinterpret_cast<uint4*>(Z3 + tile_off(t, 8, 128)) = zero;
-        for (int rr = 64; rr < 80; ++rr) put_bf16(TH1, tile_off(rr, t, 80), rr == 64 ? 1.f : 0.f);
-        for (int rr = 64; rr < 128; ++rr) put_bf16(TH2, tile_off(rr, t, 128), rr == 64 ? 1.f : 0.f);
-        for (int rr = 2; rr < 16; ++rr) put_bf16(TZ3, tile_off(rr, t, 16), 0.f);
     }
     if (t == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(bar)) : "memory");
@@ -842,24 +801,21 @@ __global__ void __launch_bounds__(128, 1) k_mlp_bwd_tc(const LearnBwdArgs b,
             v.w = pack_bf16(X[8 * h + 6], X[8 * h + 7]);
             *reinterpret_cast<uint4*>(A1 + tile_off(t, 8 * h, 128)) = v;
         }
-#pragma unroll
-        for (int q = 0; q < kLNF; ++q) put_bf16(TX, tile_off(q, t, 16), X[q]);
-        // forward: layers 1-3, keeping the activations (rows and transposed) and ReLU masks
-        unsigned m1[2], m2[2];
+        // forward: layers 1-3, keeping the activations
         sync_for_mma();
         if (t == 0) {
             mma_k(tmem + kTD, su32(A1), 2048, w + kW1T, 1024, 64, 1, false);
             commit(bar);
         }
         if (!wait_mma()) { failed = true; break; }
-        epilogue64_t(trow + kTD, A2, TH1, 80, t, m1);
+        epilogue64(trow + kTD, A2, t);
         sync_for_mma();
         if (t == 0) {
             mma_k(tmem + kTD, su32(A2), 2048, w + kW2T, 1024, 64, kK2 / 16, false);
             commit(bar);
         }
         if (!wait_mma()) { failed = true; break; }
-        epilogue64_t(trow + kTD, A3, TH2, 128, t, m2);
+        epilogue64(trow + kTD, A3, t);
         sync_for_mma();
         if (t == 0) {
             mma_k(tmem + kTD, su32(A3), 2048, w + kW3T, 256, 16, kK2 / 16, false);
@@ -899,8 +855,6 @@ __global__ void __launch_bounds__(128, 1) k_mlp_bwd_tc(const LearnBwdArgs b,
         }
         *reinterpret_cast<uint4*>(Z3 + tile_off(t, 0, 128)) =
             make_uint4(pack_bf16(dz30, dz31), 0u, 0u, 0u);
-        put_bf16(TZ3, tile_off(0, t, 16), dz30);
-        put_bf16(TZ3, tile_off(1, t, 16), dz31);
         // network backward: dz2 = (dz3 W3^T)[h2 > 0], dz1 = (dz2 W2^T)[h1 > 0], dX = dz1 W1^T
         sync_for_mma();
         if (t == 0) {
@@ -908,21 +862,22 @@ __global__ void __launch_bounds__(128, 1) k_mlp_bwd_tc(const LearnBwdArgs b,
             commit(bar);
         }
         if (!wait_mma()) { failed = true; break; }
-        epilogue64_mask(trow + kTD, m2, on, Z2, TDZ, 0, t);
+        epilogue64_mask(trow + kTD, A3, Z2, t);
         sync_for_mma();
         if (t == 0) {
             mma_k(tmem + kTD, su32(Z2), 2048, w + kB5, 1024, 64, 4, false);
             commit(bar);
         }
         if (!wait_mma()) { failed = true; break; }
-        epilogue64_mask(trow + kTD, m1, on, Z1, TDZ, 64, t);
+        epilogue64_mask(trow + kTD, A2, Z1, t);
         sync_for_mma();
         if (t == 0) {
             mma_k(tmem + kTD, su32(Z1), 2048, w + kB6, 256, 16, 4, false);
             // weight gradients, summed over the tile's cells into the CTA's accumulators
-            mma_k(tmem + kTW2, su32(TDZ), 2048, su32(TH1), 1280, 80, 8, !first);
-            mma_k(tmem + kTW1, su32(TDZ), 2048, su32(TX), 256, 16, 8, !first);
-            mma_k(tmem + kTW3, su32(TH2), 2048, su32(TZ3), 256, 16, 8, !first);
+            // ([dz2 | dz1], Z1 following Z2; the columns past A3's 80 only reach unused rows)
+            mma_cells(tmem + kTW2, su32(Z2), su32(A2), 80, !first);
+            mma_cells(tmem + kTW1, su32(Z2), su32(A1), 16, !first);
+            mma_cells(tmem + kTW3, su32(A3), su32(Z3), 16, !first);
             commit(bar);
         }
         if (!wait_mma()) { failed = true; break; }
@@ -1013,7 +968,7 @@ cudaError_t launch_learn_tc_pack(const float* params, void* wtc, cudaStream_t s)
 cudaError_t launch_mlp_bwd_tc(int nv, const LearnBwdArgs& b, const void* wtc, int sm_count,
                               cudaStream_t s) {
     const long long n = (long long)b.fw.nx * b.fw.ny * nv * nv;
-    const int grid = (int)std::max<long long>(1, std::min<long long>((n + 127) / 128, sm_count));
+    const int grid = (int)std::max<long long>(1, std::min<long long>((n + 127) / 128, 2LL * sm_count));
     const unsigned char* img = static_cast<const unsigned char*>(wtc);
     switch (nv) {
 #define X(nn)                                                                                   \
