@@ -87,21 +87,25 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
                  : "memory");
 }
 
-__device__ __forceinline__ bool wait_parity(uint64_t* bar, unsigned parity) {
+__device__ __forceinline__ bool try_parity(unsigned bar, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+__device__ __noinline__ bool wait_parity_slow(uint64_t* bar, unsigned parity) {
     const unsigned long long t0 = [] {
         unsigned long long t;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
         return t;
     }();
     for (long long it = 0; it < (1ll << 26); ++it) {
-        unsigned ok;
-        asm volatile(
-            "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, q;\n\t}"
-            : "=r"(ok)
-            : "r"(su32(bar)), "r"(parity)
-            : "memory");
-        if (ok) return true;
+        if (try_parity(su32(bar), parity)) return true;
         if ((it & 255) == 0) {
             unsigned long long t;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -109,6 +113,10 @@ __device__ __forceinline__ bool wait_parity(uint64_t* bar, unsigned parity) {
         }
     }
     return false;
+}
+
+__device__ __forceinline__ bool wait_parity(uint64_t* bar, unsigned parity) {
+    return try_parity(su32(bar), parity) || wait_parity_slow(bar, parity);
 }
 
 // 16 consecutive accumulator columns of this thread's row (completion: tmem_wait)
@@ -459,7 +467,11 @@ __device__ __forceinline__ void run_network(Feed& feed, unsigned char* sm,
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tslot;
     const unsigned trow = tmem + ((unsigned)(warp * 32) << 16);  // this warp's lanes
-    const unsigned wbase = su32(W), a1 = su32(A1), a2 = su32(A2);
+    // descriptors of the MMAs' first operands: the others are offsets in their address field (which
+    // counts 16 bytes; no carry out of its 14 bits here)
+    const uint64_t da1 = sdesc(su32(A1), 2048, 128), da2 = sdesc(su32(A2), 2048, 128),
+                   dw1 = sdesc(su32(W) + kW1T, 1024, 128), dw2 = sdesc(su32(W) + kW2T, 1024, 128),
+                   dw3 = sdesc(su32(W) + kW3T, 256, 128);
     unsigned phase = 0;
     // features of q into row t of A1 (zeros past the end)
     auto stage = [&](typename Feed::Slot& q) {
@@ -495,7 +507,7 @@ __device__ __forceinline__ void run_network(Feed& feed, unsigned char* sm,
         // layer 1: D = A1 (128 x 16) W1^T, while the next tile's inputs load
         sync_for_mma();
         if (t == 0) {
-            mma(tmem, sdesc(a1, 2048, 128), sdesc(wbase + kW1T, 1024, 128), idesc_n(64), 0);
+            mma(tmem, da1, dw1, idesc_n(64), 0);
             commit(bar);
         }
         feed.load(nxt);
@@ -505,9 +517,9 @@ __device__ __forceinline__ void run_network(Feed& feed, unsigned char* sm,
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         sync_for_mma();
         if (t == 0) {
+#pragma unroll
             for (int kk = 0; kk < kK2 / 16; ++kk)
-                mma(tmem, sdesc(a2 + kk * 2 * 2048, 2048, 128),
-                    sdesc(wbase + kW2T + kk * 2 * 1024, 1024, 128), idesc_n(64), kk);
+                mma(tmem, da2 + kk * (2 * 2048 / 16), dw2 + kk * (2 * 1024 / 16), idesc_n(64), kk);
             commit(bar);
         }
         stage(nxt);
@@ -517,9 +529,9 @@ __device__ __forceinline__ void run_network(Feed& feed, unsigned char* sm,
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         sync_for_mma();
         if (t == 0) {
+#pragma unroll
             for (int kk = 0; kk < kK2 / 16; ++kk)
-                mma(tmem, sdesc(a2 + kk * 2 * 2048, 2048, 128),
-                    sdesc(wbase + kW3T + kk * 2 * 256, 256, 128), idesc_n(16), kk);
+                mma(tmem, da2 + kk * (2 * 2048 / 16), dw3 + kk * (2 * 256 / 16), idesc_n(16), kk);
             commit(bar);
         }
         if (!wait_mma()) return false;
