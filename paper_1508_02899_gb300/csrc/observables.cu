@@ -6,6 +6,8 @@
 // Lattice forms: r = w dx for whole numbers w of cells, the window of cell i covering cells
 // i .. i + w - 1 (periodic; w x w squares in 2D); separations s dx; velocity differences
 // |j - j'| dv.  All reductions are compensated FP64 sums in a fixed order (deterministic).
+#include <algorithm>
+
 #include "lat_internal.h"
 #include "lat_reduce.h"
 
@@ -178,43 +180,127 @@ __global__ void __launch_bounds__(kObsThreads)
 //   U_j = sum_{j' > j} b_j' (j' - j),  U_{j-1} = U_j + sum_{j' >= j} b_j'   (backward),
 // then times dv^3; the denominator rho_i rho_{i+s}.  T = float for FP32 states (errors about
 // N_v u of the positive sums), double for FP64 states.
+//
+// A block takes a run of columns of one instance, a thread cpt cells of it, and kS1Group separations
+// in one pair of sweeps: a_j is loaded for all of them, and what remains per separation and velocity
+// cell is one load and three operations in either direction (1024 instances, N_v = 65, eight
+// separations: 2.4 ms; a block per instance and separation 6.5 ms).  The cells' sums are FP64 Neumaier
+// sums per thread; the 2 kS1Group sums of a warp's lanes are folded by halving (every lane ends with
+// one of them) rather than by as many butterflies, which took longer than the sweeps.  The blocks'
+// sums go to part[instance][chunk][num, den of each][sum, compensation], folded in order.
+constexpr int kS1Group = 8;
+constexpr int kS1Threads = 128;
+
+__device__ __forceinline__ Comp shfl_xor(const Comp& a, int m) {
+    return Comp{__shfl_xor_sync(0xffffffffu, a.s, m), __shfl_xor_sync(0xffffffffu, a.c, m)};
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kObsThreads)
-    k_s1_1d(const T* f, const Inst1D* inst, int n_inst, int nv, const double* rho,
-            const int* seps, int ns, double* num, double* den) {
-    for (int b = blockIdx.x; b < n_inst * ns; b += gridDim.x) {
-        const int k = b / ns, q = b % ns;
-        const Inst1D in = inst[k];
-        const int n = in.nx, s = seps[q];
+__global__ void __launch_bounds__(kS1Threads)
+    k_s1_1d(const T* f, const Inst1D* inst, int n_inst, int cpt, int nv, const double* rho,
+            const int* seps, int q0, int nq, double* part) {
+    constexpr int NS = 2 * kS1Group;  // sums: 2 q the numerator, 2 q + 1 the denominator
+    __shared__ Comp wsum[kS1Threads / 32][NS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = blockIdx.y; k < n_inst; k += gridDim.y) {
+        const Inst1D& in = inst[k];
+        const int n = in.nx, x0 = blockIdx.x * kS1Threads * cpt;
+        if (x0 >= n) continue;
         const T* fk = f + in.off;
-        Comp tn{0, 0}, td{0, 0};
-        for (int i = threadIdx.x; i < n; i += kObsThreads) {
-            const int i2 = i + s < n ? i + s : i + s - n;
-            T acc = T(0), B = T(0), run = T(0);
+        Comp t[NS];
+#pragma unroll
+        for (int q = 0; q < NS; ++q) t[q] = Comp{0, 0};
+        for (int e = 0; e < cpt; ++e) {
+            const int i = x0 + e * kS1Threads + threadIdx.x;
+            if (i >= n) break;
+            int i2[kS1Group];
+            T acc[kS1Group], B[kS1Group], run[kS1Group];
+#pragma unroll
+            for (int q = 0; q < kS1Group; ++q) {
+                const int s = q < nq ? seps[q0 + q] : 0;
+                i2[q] = i + s < n ? i + s : i + s - n;
+                acc[q] = B[q] = run[q] = T(0);
+            }
+            const T* row = fk;
+#pragma unroll 2
             for (int j = 0; j < nv; ++j) {
-                const T a = fk[(size_t)j * n + i];
-                acc += a * run;
-                B += fk[(size_t)j * n + i2];
-                run += B;
+                const T a = row[i];
+#pragma unroll
+                for (int q = 0; q < kS1Group; ++q) {
+                    acc[q] += a * run[q];
+                    B[q] += row[i2[q]];
+                    run[q] += B[q];
+                }
+                row += n;
             }
-            B = T(0);
-            run = T(0);
+#pragma unroll
+            for (int q = 0; q < kS1Group; ++q) B[q] = run[q] = T(0);
+#pragma unroll 2
             for (int j = nv - 1; j >= 0; --j) {
-                const T a = fk[(size_t)j * n + i];
-                acc += a * run;
-                B += fk[(size_t)j * n + i2];
-                run += B;
+                row -= n;
+                const T a = row[i];
+#pragma unroll
+                for (int q = 0; q < kS1Group; ++q) {
+                    acc[q] += a * run[q];
+                    B[q] += row[i2[q]];
+                    run[q] += B[q];
+                }
             }
-            nadd(tn, (double)acc);
-            nadd(td, rho[in.xoff + i] * rho[in.xoff + i2]);
+            const double* rk = rho + in.xoff;
+            const double ri = rk[i];
+#pragma unroll
+            for (int q = 0; q < kS1Group; ++q) {
+                nadd(t[2 * q], (double)acc[q]);
+                nadd(t[2 * q + 1], ri * rk[i2[q]]);
+            }
         }
-        const Comp zn = block_reduce(tn);
-        const Comp zd = block_reduce(td);
-        if (threadIdx.x == 0) {
-            num[b] = nval(zn) * in.dv * in.dv * in.dv / n;
-            den[b] = nval(zd) / n;
+        // halve the sums a lane holds, level by level: after it lane l holds sum l / 2 over the
+        // lanes of its parity, then over all
+#pragma unroll
+        for (int h = NS / 2, m = 16; h >= 1; h >>= 1, m >>= 1) {
+            const bool up = (lane & m) != 0;
+#pragma unroll
+            for (int q = 0; q < h; ++q) {
+                const Comp keep = up ? t[q + h] : t[q], give = up ? t[q] : t[q + h];
+                t[q] = keep;
+                nmerge(t[q], shfl_xor(give, m));
+            }
         }
+        nmerge(t[0], shfl_xor(t[0], 1));
+        if ((lane & 1) == 0) wsum[warp][lane / 2] = t[0];
+        __syncthreads();
+        if (threadIdx.x < NS) {
+            Comp z{0, 0};
+            for (int w = 0; w < kS1Threads / 32; ++w) nmerge(z, wsum[w][threadIdx.x]);
+            double* p = part + (((size_t)k * gridDim.x + blockIdx.x) * NS + threadIdx.x) * 2;
+            p[0] = z.s;
+            p[1] = z.c;
+        }
+        __syncthreads();
     }
+}
+
+// One half-warp per instance folds its chunks' sums in order.
+__global__ void k_s1_fold(const double* part, int nchunk, int cpt, const Inst1D* inst, int n_inst,
+                          int q0, int nq, int ns, double* num, double* den) {
+    constexpr int NS = 2 * kS1Group;
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) / NS, q = threadIdx.x % NS;
+    if (k >= n_inst || q >= 2 * nq) return;
+    const Inst1D& in = inst[k];
+    Comp z{0, 0};
+    for (int c = 0; c * kS1Threads * cpt < in.nx; ++c) {
+        const double* p = part + (((size_t)k * nchunk + c) * NS + q) * 2;
+        nmerge(z, Comp{p[0], p[1]});
+    }
+    const size_t o = (size_t)k * ns + q0 + q / 2;
+    if (q % 2 == 0) num[o] = nval(z) * in.dv * in.dv * in.dv / in.nx;
+    else den[o] = nval(z) / in.nx;
+}
+
+// Cells per thread: eight where that still leaves sixteen blocks per SM.
+int s1_cells(long long total_x, int sm_count) {
+    const long long c = total_x / ((long long)kS1Threads * 16 * sm_count);
+    return (int)std::max(1ll, std::min(8ll, c));
 }
 
 int obs_grid(long long blocks, int sm_count) {
@@ -251,18 +337,28 @@ cudaError_t launch_coarse2d(const double* rho, int nx, int ny, double dx, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_s1_1d(int dtype, const void* f, const Inst1D* inst, int n_inst, int nv,
-                         const double* rho, const int* seps, int ns, double* num, double* den,
-                         int sm_count, cudaStream_t s) {
-    const int grid = obs_grid((long long)n_inst * ns, sm_count);
-    if (dtype == LAT_F32)
-        k_s1_1d<float><<<grid, kObsThreads, 0, s>>>(static_cast<const float*>(f), inst, n_inst,
-                                                    nv, rho, seps, ns, num, den);
-    else if (dtype == LAT_F64)
-        k_s1_1d<double><<<grid, kObsThreads, 0, s>>>(static_cast<const double*>(f), inst,
-                                                     n_inst, nv, rho, seps, ns, num, den);
-    else
-        return cudaErrorInvalidValue;
+size_t s1_scratch(int n_inst, int nx_max, long long total_x, int sm_count) {
+    const int per = kS1Threads * s1_cells(total_x, sm_count);
+    return (size_t)n_inst * ((nx_max + per - 1) / per) * 4 * kS1Group;
+}
+
+cudaError_t launch_s1_1d(int dtype, const void* f, const Inst1D* inst, int n_inst, int nx_max,
+                         long long total_x, int nv, const double* rho, const int* seps, int ns,
+                         double* part, double* num, double* den, int sm_count, cudaStream_t s) {
+    if (dtype != LAT_F32 && dtype != LAT_F64) return cudaErrorInvalidValue;
+    const int cpt = s1_cells(total_x, sm_count), per = kS1Threads * cpt;
+    const dim3 grid((nx_max + per - 1) / per, std::min(n_inst, 65535));
+    for (int q0 = 0; q0 < ns; q0 += kS1Group) {
+        const int nq = std::min(kS1Group, ns - q0);
+        if (dtype == LAT_F32)
+            k_s1_1d<float><<<grid, kS1Threads, 0, s>>>(static_cast<const float*>(f), inst, n_inst,
+                                                       cpt, nv, rho, seps, q0, nq, part);
+        else
+            k_s1_1d<double><<<grid, kS1Threads, 0, s>>>(static_cast<const double*>(f), inst, n_inst,
+                                                        cpt, nv, rho, seps, q0, nq, part);
+        k_s1_fold<<<(n_inst + 7) / 8, 16 * kS1Group, 0, s>>>(part, grid.x, cpt, inst, n_inst, q0, nq,
+                                                             ns, num, den);
+    }
     return cudaGetLastError();
 }
 

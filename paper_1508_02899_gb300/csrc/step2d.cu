@@ -874,10 +874,10 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
                         const size_t plane = (size_t)jy * nv + jx;
                         const double fvv = to_d(f[plane * ncell + c]);
                         bad |= !isfinite(fvv);
-                        nadd_fast(s[0], fvv);
-                        nadd_fast(s[1], __dmul_rn(vx, fvv));
-                        nadd_fast(s[2], __dmul_rn(vy, fvv));
-                        nadd_fast(s[3], __dmul_rn(__dadd_rn(__dmul_rn(vx, vx), vy2), fvv));
+                        nadd(s[0], fvv);
+                        nadd(s[1], __dmul_rn(vx, fvv));
+                        nadd(s[2], __dmul_rn(vy, fvv));
+                        nadd(s[3], __dmul_rn(__dadd_rn(__dmul_rn(vx, vx), vy2), fvv));
                     }
                 }
                 if (warp > 0)
