@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(kMaxPlaces / 2, 2)
             }
         }
     }
+    __syncwarp();  // lanes that wait early would hold back those that still issue copies
     bool failed = false;
     if (piped) failed = !mbar_wait_bounded(bar, 0u);
     else asm volatile("cp.async.wait_all;" ::: "memory");
