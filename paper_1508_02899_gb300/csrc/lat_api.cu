@@ -24,6 +24,12 @@ __global__ void k_set_noise_window(DevState* st, long long base, long long rows)
 }
 __global__ void k_clear_status(DevState* st) { st->status = 0u; }
 
+// Tiles of columns of an on-chip kernel (none where not built) and their widest places.
+struct TileSet {
+    lat::MultiTile* d = nullptr;
+    int n = 0, places = 0;
+};
+
 }  // namespace
 
 struct lat_ctx {
@@ -77,9 +83,7 @@ struct lat_ctx {
     bool stalled = false;  // lat_debug_stall
     bool pinned = false;  // a kernel chosen by lat_set_launch: one step per launch
 
-    // several steps per launch (multi1d.cu): tiles (none where not built) and their widest places
-    MultiTile* d_tiles = nullptr;
-    int ntiles = 0, places = 0;
+    TileSet tiles[2];  // several upwind steps per launch (multi1d.cu); the limited step (lim1d.cu)
     bool line_ok = false;         // small enough for the cluster kernel (line1d.cu)
     bool wflow_ok = false;        // the flow kernel's tables and buffer exist
     void* d_basis = nullptr;      // flow-basis tables, their offsets per instance, and u / dv of a
@@ -216,6 +220,7 @@ static_assert(kMultiT <= kFlowSteps, "their flow is formed in one launch");
 // Tiles of the several-steps kernel, the flow-basis tables and the flow buffer it reads (beyond
 // kBasisBytes of tables, steps are launched one by one).  Called whenever the flow changes.
 constexpr size_t kBasisBytes = 64u << 20;
+constexpr long long kLimRestCells = 8 << 20;  // see enqueue_steps_1d
 constexpr int kMinTile = 64;  // narrower tiles are mostly margin
 
 int max_nx(const lat_ctx* c) {
@@ -224,15 +229,81 @@ int max_nx(const lat_ctx* c) {
     return nx;
 }
 
+int tile_places(const lat_ctx* c, bool lim, int w) {
+    return lim ? lim1d_places(w) : multi1d_places(c->nv, kMultiT, w);
+}
+
+// Instances are cut into equal tiles of at most w columns.
+int tile_cut(int nx, int w, int wmax) {
+    const int nt = (nx + w - 1) / w;
+    return std::min(wmax, ((nx + nt - 1) / nt + 7) / 8 * 8);
+}
+
+// Tiles of the kernel that takes several upwind steps per launch, or of the limited one.  Their width
+// is the one of least time when `held` tiles share an SM at a time and k of them take (P + 64)
+// (0.7 + k), P the places of a tile (the parts are of its sweep and of its latencies); the widest of
+// equals.  Upwind, N_v = 33, 64 instances of 200 to 1500 columns, 50 steps: two tiles per SM 268 us,
+// one 303 us, one step per launch 435 us.
+int build_tiles(lat_ctx* c, bool lim) {
+    TileSet& t = c->tiles[lim];
+    int places = 0, margin = 0;
+    if (!(lim ? lim1d_shape(c->nv, &places) : multi1d_shape(c->nv, kMultiT, &places, &margin)))
+        return LAT_OK;
+    const int wmax = (places - 2 * margin) / 8 * 8;
+    const int held = lim ? 3 : 2;
+    std::map<int, int> sizes;  // N_x -> instances
+    for (const Inst1D& in : c->h_inst) ++sizes[in.nx];
+    int wtile = wmax;
+    double best = 0.0;
+    for (int w = wmax; w >= std::min(kMinTile, wmax); w -= 8) {
+        long long n = 0;
+        int widest = 0;
+        for (const auto& e : sizes) {
+            const int cut = tile_cut(e.first, w, wmax);
+            n += (long long)e.second * ((e.first + cut - 1) / cut);
+            widest = std::max(widest, std::min(cut, e.first));
+        }
+        // tiles per SM: whole ones of the last wave while waves are few, else half a wave of it
+        const double per_sm = double(n) / c->sm_count;
+        const int whole = (int)ceil(per_sm), left = whole % held;
+        const double waves = per_sm > 3 * held
+                                 ? (per_sm / held + 0.5) * (0.7 + held)
+                                 : whole / held * (0.7 + held) + (left ? 0.7 + left : 0.0);
+        const double cost = (tile_places(c, lim, widest) + 64) * waves;
+        if (w == wmax || cost < best) {
+            best = cost;
+            wtile = w;
+        }
+    }
+    std::vector<MultiTile> tiles;
+    for (int i = 0; i < c->n_inst; ++i) {
+        const Inst1D& in = c->h_inst[i];
+        const int w = tile_cut(in.nx, wtile, wmax);
+        for (int x0 = 0; x0 < in.nx; x0 += w) {
+            const int cols = std::min(w, in.nx - x0);
+            tiles.push_back({in.off, in.xoff, in.nx, x0, cols, (float)in.g, (float)in.r});
+            t.places = std::max(t.places, tile_places(c, lim, cols));
+        }
+    }
+    if (cudaMalloc(&t.d, sizeof(MultiTile) * tiles.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return LAT_OK;
+    }
+    CK(cudaMemcpy(t.d, tiles.data(), sizeof(MultiTile) * tiles.size(), cudaMemcpyHostToDevice));
+    t.n = (int)tiles.size();
+    return LAT_OK;
+}
+
 int build_multi(lat_ctx* c) {
     c->line_ok = line1d_fits(c->dtype, c->n_inst, max_nx(c), c->nv, c->nmodes);
-    cudaFree(c->d_tiles);
+    for (TileSet& t : c->tiles) {
+        cudaFree(t.d);
+        t = TileSet{};
+    }
     cudaFree(c->d_basis);
     cudaFree(c->d_basis_off);
-    c->d_tiles = nullptr;
     c->d_basis = nullptr;
     c->d_basis_off = nullptr;
-    c->ntiles = c->places = 0;
     c->wflow_ok = false;
     const size_t elem = c->dtype == LAT_F64 ? sizeof(double) : sizeof(float);
     std::map<int, std::pair<int, long long>> sizes;  // N_x -> (an instance, table offset)
@@ -261,33 +332,9 @@ int build_multi(lat_ctx* c) {
                                  c->stream));
     }
     c->wflow_ok = true;
-    int places = 0, margin = 0;
-    if (c->dtype != LAT_F32 || !multi1d_shape(c->nv, kMultiT, &places, &margin)) return LAT_OK;
-    // Tiles as wide as fit, or two per SM where there are fewer columns than that (64 instances
-    // of 200 to 1500 columns, N_v = 33, 50 steps: 268 us; one per SM 303 us; one step per launch
-    // 435 us).
-    const int wmax = (places - 2 * margin) / 8 * 8;
-    const int wfill = (int)(c->total_x / (2 * c->sm_count) / 8 * 8);
-    const int wtile = std::max(std::min(wfill, wmax), std::min(kMinTile, wmax));
-    std::vector<MultiTile> tiles;
-    for (int i = 0; i < c->n_inst; ++i) {
-        const Inst1D& in = c->h_inst[i];
-        const int nt = (in.nx + wtile - 1) / wtile;
-        const int w = std::min(wmax, ((in.nx + nt - 1) / nt + 7) / 8 * 8);
-        for (int x0 = 0; x0 < in.nx; x0 += w) {
-            tiles.push_back({in.off, in.xoff, in.nx, x0, std::min(w, in.nx - x0), (float)in.g,
-                             (float)in.r});
-            c->places = std::max(c->places, multi1d_places(c->nv, kMultiT, tiles.back().w));
-        }
-    }
-    if (cudaMalloc(&c->d_tiles, sizeof(MultiTile) * tiles.size()) != cudaSuccess) {
-        cudaGetLastError();
-        return LAT_OK;
-    }
-    CK(cudaMemcpy(c->d_tiles, tiles.data(), sizeof(MultiTile) * tiles.size(),
-                  cudaMemcpyHostToDevice));
-    c->ntiles = (int)tiles.size();
-    return LAT_OK;
+    if (c->dtype != LAT_F32) return LAT_OK;
+    int rc = build_tiles(c, false);
+    return rc != LAT_OK ? rc : build_tiles(c, true);
 }
 
 // Whether batches of steps run on the cluster kernel of small lattices.
@@ -307,22 +354,30 @@ int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
         if (c->n_inst > 1) CK(launch_advance_step(c->d_state, n, s));
         return LAT_OK;
     }
-    const bool multi = on_chip && c->ntiles;
-    // The plain-load kernels take the flow from the flow kernel (kFlowSteps steps at a time):
-    // evaluating the basis costs an FP64 column as much as half its sweep.
-    const bool pre = !chosen && c->variant == STEP1D_PLAIN && c->wflow_ok &&
-                     c->flow_kind == LAT_FLOW_MODES;
+    const bool multi = on_chip && c->tiles[0].n;
+    const bool lim = !chosen && c->scheme == LAT_SCHEME_KOREN && c->tiles[1].n;
+    // The plain-load and the limited kernels take the flow from the flow kernel, kFlowSteps steps at
+    // a time (evaluating the basis costs an FP64 column as much as half its sweep).  The launch is
+    // not worth it for fewer FP32 steps (1000 instances of 601 columns, N_v = 33, one upwind step:
+    // 52 us, with the launch 58 us) unless the limited step is long (1200 instances of 1024 columns,
+    // one step: N_v = 65 175 us, one column per thread 303 us; N_v = 17 89 and 82 us; 48 instances of
+    // 4096 columns, N_v = 33: 28 and 25 us).
+    const bool pre = lim || (!chosen && c->variant == STEP1D_PLAIN && c->wflow_ok &&
+                             c->flow_kind == LAT_FLOW_MODES);
+    const bool rest = c->dtype == LAT_F64 ||
+                      (lim && c->nv >= 33 && c->total_x * c->nv >= kLimRestCells);
     const size_t row = (c->dtype == LAT_F64 ? sizeof(double) : sizeof(float)) * c->total_x;
     int formed = 0, first = 0;  // steps whose flow is formed, from step `first` on
     for (int k = 0, t; k < n; k += t) {
         Step1DArgs a = step_args(c, k, 0);
         t = multi && n - k >= kMultiT ? kMultiT : 1;
         if (t > 1) {
-            CK(launch_multi1d(c->nv, t, c->ntiles, c->places, a, c->d_tiles, k, c->ring_ok ? 1 : 0,
-                              s));
+            CK(launch_multi1d(c->nv, t, c->tiles[0].n, c->tiles[0].places, a, c->tiles[0].d, k,
+                              c->ring_ok ? 1 : 0, s));
             continue;
         }
-        if (pre) {
+        const bool from_row = pre && (k < first + formed || rest || n - k >= kFlowSteps);
+        if (from_row) {
             if (k >= first + formed) {
                 first = k;
                 formed = std::min(kFlowSteps, n - k);
@@ -330,6 +385,11 @@ int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
                 CK(launch_flow_steps(c->dtype, a, k, formed, s));
             }
             a.wpre = static_cast<char*>(c->d_wflow) + (k - first) * row;
+        }
+        if (lim && from_row) {
+            CK(launch_lim1d(c->nv, c->tiles[1].n, c->tiles[1].places, a, c->tiles[1].d, k,
+                            static_cast<const float*>(a.wpre), c->ring_ok ? 1 : 0, s));
+            continue;
         }
         if (c->mode == 1) {
             for (int i = 0; i < c->n_inst; ++i) {
@@ -1375,7 +1435,7 @@ void lat_free(lat_ctx* c) {
     cudaFree(c->d_items);
     cudaFree(c->d_inst_begin);
     cudaFree(c->d_partials);
-    cudaFree(c->d_tiles);
+    for (TileSet& t : c->tiles) cudaFree(t.d);
     cudaFree(c->d_basis);
     cudaFree(c->d_basis_off);
     cudaFree(c->d_wflow);

@@ -107,6 +107,12 @@ struct MultiTile {
 // T = 5, 9, 13 .. steps per launch for the N_v it is built for: the places a tile may take with its
 // margins (w + 2 margin <= max_places); false where there is no kernel.
 bool multi1d_shape(int nv, int T, int* max_places, int* margin);
+// One flux-limited step of every tile (lim1d.cu, FP32): columns of a tile at most, places (threads x 2)
+// of a tile of w columns; wrow the step's row of wflow.
+bool lim1d_shape(int nv, int* max_places);
+int lim1d_places(int w);
+cudaError_t launch_lim1d(int nv, int ntiles, int places, const Step1DArgs& a, const MultiTile* tiles,
+                         int kstep, const float* wrow, int piped, cudaStream_t s);
 // Steps kstep .. kstep + n - 1 of small 1D lattices (upwind drag), one cluster per lattice with the
 // state in shared memory throughout (line1d.cu).
 bool line1d_fits(int dtype, int n_inst, int nx_max, int nv, int nmodes);
