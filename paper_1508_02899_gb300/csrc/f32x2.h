@@ -51,6 +51,17 @@ __device__ __forceinline__ f2 sub2s(f2 a, f2 b) {
 }
 __device__ __forceinline__ f2 max0(f2 v) { return pk(fmaxf(lo(v), 0.f), fmaxf(hi(v), 0.f)); }
 __device__ __forceinline__ f2 min0(f2 v) { return pk(fminf(lo(v), 0.f), fminf(hi(v), 0.f)); }
+// max(0, min(a, b, c)) where a > 0, min(0, max(a, b, c)) where a < 0, zero where a = 0, lane by lane:
+// the limited increment of the sign of a, by three-input instructions.
+__device__ __forceinline__ float lim_min(float a, float b, float c) {
+    float lo3, hi3;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(lo3) : "f"(a), "f"(b), "f"(c));
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(hi3) : "f"(a), "f"(b), "f"(c));
+    return fmaxf(fminf(hi3, 0.f), lo3);
+}
+__device__ __forceinline__ f2 lim_min2(f2 a, f2 b, f2 c) {
+    return pk(lim_min(lo(a), lo(b), lo(c)), lim_min(hi(a), hi(b), hi(c)));
+}
 // Hides a value from the compiler's constant folding and hoisting.
 __device__ __forceinline__ f2 opaque2(f2 v) {
     asm volatile("mov.b64 %0, %0;" : "+l"(v));

@@ -6,14 +6,13 @@
 //  * the arithmetic of two columns c and c + 32 runs in the lanes of one instruction;
 //  * where c a has one sign over the rows at hand and the warp's columns, the part of the split flux
 //    that is zero is not formed (rows go in chunks, the test is per chunk and uniform);
-//  * the limiter takes min(dp, b, c) and max(dp, b, c) by three-input instructions:
-//    psi dp = max(0, min(dp, b, c)) + min(0, max(dp, b, c)), one term zero by the sign of dp, which
-//    is lim_inc's value up to the sign of a zero.
+//  * the limiter takes min(dp, b, c) and max(dp, b, c) by three-input instructions (lim_min):
+//    lim_inc's value up to the sign of a zero.
 // The streaming is the place the tile's windows are copied from; the flow comes from k_flow_steps.
 //
-// Measured (1024 instances, N_x 1024 .. 8192, N_v = 65): 391 us per step at 5.3 TB/s, issue slots 57 %
+// Measured (1024 instances, N_x 1024 .. 8192, N_v = 65): 385 us per step at 5.4 TB/s, issue slots 57 %
 // busy, 12 warps per SM (three tiles' planes fill the shared memory); one column per thread 945 us;
-// ten steps, moments and globals 9.96 -> 4.73 ms.  Tiles of 128 columns, six per SM: 4.77 ms; a barrier
+// ten steps, moments and globals 9.96 -> 4.65 ms.  Tiles of 128 columns, six per SM: 4.77 ms; a barrier
 // per eight rows, so that a sweep starts on its first ones: 4.78 ms (128 columns: 4.93 ms).
 #include <math.h>
 #include <stdint.h>
@@ -33,28 +32,13 @@ constexpr int kChunk = 8;       // rows per pass of the loop
 constexpr int kPlaces = 256;    // columns of a tile at most
 constexpr int kPitch = kPlaces + 4;
 
-__device__ __forceinline__ float min3(float a, float b, float c) {
-    float d;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
 struct LimConst {
     f2 g2, r2, mu2, third2, sixth2, half2, one2, zero2;
 };
 
 // psi(theta) dp in two lanes (lim_inc)
 __device__ __forceinline__ f2 inc2(f2 dp, f2 dm, const LimConst& k) {
-    const f2 b = fma2(dm, k.sixth2, mul2(dp, k.third2));
-    const f2 c = mul2(k.mu2, dm);
-    const f2 up = pk(fmaxf(0.f, min3(lo(dp), lo(b), lo(c))), fmaxf(0.f, min3(hi(dp), hi(b), hi(c))));
-    const f2 dn = pk(fminf(0.f, max3(lo(dp), lo(b), lo(c))), fminf(0.f, max3(hi(dp), hi(b), hi(c))));
-    return add2(up, dn);
+    return lim_min2(dp, fma2(dm, k.sixth2, mul2(dp, k.third2)), mul2(k.mu2, dm));
 }
 
 enum { kBoth = 0, kPos = 1, kNeg = 2 };

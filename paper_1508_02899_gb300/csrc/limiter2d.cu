@@ -582,8 +582,11 @@ cudaError_t launch_fused_t(const Lim2DArgs& a, int k, int sm_count, cudaStream_t
 // As k_lim2d_fused with a thread on two neighbouring cells of the tile (one velocity column):
 // their values travel as pairs (8-byte shared-memory accesses) and the arithmetic of both cells
 // runs in the two lanes of the f32x2 instructions; min/max and the sign tests stay per lane.
-// Every lane performs the scalar kernel's operations in the same order, so the bits are the
-// same.  LPC = TC / 2 lanes per column, CPW = 32 / LPC columns per warp.
+// Limiter by three-input minima and maxima (lim_min), products that feed one packed add or subtract as
+// fma2(a, b, 0): 1024 x 1024, N_v = 19, a step 2.97 -> 2.82 ms (with copysign and products lane by
+// lane; 331 instructions per pair and velocity, issue slots 56 % busy).
+// Every lane gets the values of the scalar kernel up to the sign of a zero.
+// LPC = TC / 2 lanes per column, CPW = 32 / LPC columns per warp.
 template <int NV, int TC>
 struct LimPacked {
     static constexpr int J = (NV - 1) / 2;
@@ -598,47 +601,40 @@ struct LimPacked {
     static_assert(TC % 2 == 0 && 32 % LPC == 0 && kThreads <= 1024, "tile shape");
 };
 
-// a * b lane by lane with scalar instructions (the rounding of mul2), for a product whose only
-// use is a packed add or subtract (see sub2s in f32x2.h and face_vals_x2 below).
-__device__ __forceinline__ f2 mul2s(f2 a, f2 b) {
-    return pk(__fmul_rn(lo(a), lo(b)), __fmul_rn(hi(a), hi(b)));
-}
 __device__ __forceinline__ f2 ld2s(const float* p) { return *reinterpret_cast<const f2*>(p); }
 __device__ __forceinline__ void st2s(float* p, f2 v) { *reinterpret_cast<f2*>(p) = v; }
 __device__ __forceinline__ f2 splat(float a) { return pk(a, a); }
 
-// lim_inc2<float> lane by lane
-__device__ __forceinline__ f2 lim_inc2_x2(f2 dp, f2 dm, f2 mu2) {
-    const float dp0 = lo(dp), dp1 = hi(dp);
-    const f2 s = pk(copysignf(1.f, dp0), copysignf(1.f, dp1));
-    const f2 b = mul2(s, fma2(dm, splat((float)(1.0 / 6.0)), mul2(dp, splat((float)(1.0 / 3.0)))));
-    const f2 c = mul2(s, mul2(mu2, dm));
-    const float m0 = fmaxf(0.f, fminf(fabsf(dp0), fminf(lo(b), lo(c))));
-    const float m1 = fmaxf(0.f, fminf(fabsf(dp1), fminf(hi(b), hi(c))));
-    return mul2(s, pk(m0, m1));
+// Limiter constants of a pair; zero2 is an opaque zero: a product that only feeds a packed add or
+// subtract is formed as fma2(a, b, zero2), which keeps it from being contracted into that
+// instruction (the scalar kernel rounds it).
+struct LimPair {
+    f2 mu2, third2, sixth2, zero2;
+};
+
+// lim_inc2<float> lane by lane (up to the sign of a zero)
+__device__ __forceinline__ f2 lim_inc2_x2(f2 dp, f2 dm, const LimPair& k) {
+    return lim_min2(dp, fma2(dm, k.sixth2, mul2(dp, k.third2)), mul2(k.mu2, dm));
 }
-__device__ __forceinline__ f2 pos_part_x2(f2 P0, f2 P1, f2 P2, f2 mu2) {
-    return add2(P1, lim_inc2_x2(sub2(P2, P1), sub2(P1, P0), mu2));
+__device__ __forceinline__ f2 pos_part_x2(f2 P0, f2 P1, f2 P2, const LimPair& k) {
+    return add2(P1, lim_inc2_x2(sub2(P2, P1), sub2(P1, P0), k));
 }
-__device__ __forceinline__ f2 neg_part_x2(f2 M1, f2 M2, f2 M3, f2 mu2) {
-    return add2(M2, lim_inc2_x2(sub2(M1, M2), sub2(M2, M3), mu2));
+__device__ __forceinline__ f2 neg_part_x2(f2 M1, f2 M2, f2 M3, const LimPair& k) {
+    return add2(M2, lim_inc2_x2(sub2(M1, M2), sub2(M2, M3), k));
 }
 __device__ __forceinline__ f2 face_parts_x2(int kind, f2 P0, f2 P1, f2 P2, f2 M1, f2 M2, f2 M3,
-                                            f2 mu2) {
-    if (kind == kPosPart) return pos_part_x2(P0, P1, P2, mu2);
-    if (kind == kNegPart) return neg_part_x2(M1, M2, M3, mu2);
-    return add2(pos_part_x2(P0, P1, P2, mu2), neg_part_x2(M1, M2, M3, mu2));
+                                            const LimPair& k) {
+    if (kind == kPosPart) return pos_part_x2(P0, P1, P2, k);
+    if (kind == kNegPart) return neg_part_x2(M1, M2, M3, k);
+    return add2(pos_part_x2(P0, P1, P2, k), neg_part_x2(M1, M2, M3, k));
 }
-// The split fluxes of a vx face are formed lane by lane (mul2s): each is used by this face
-// only, and with mul.rn.f32x2 the kernels built by this toolchain differed from the scalar
-// kernel by one unit in the last place in some faces, while every packed instruction on its own
-// rounds exactly.
 __device__ __forceinline__ f2 face_vals_x2(int kind, f2 x0, f2 x1, f2 x2, f2 x3, f2 cp0, f2 cp1,
-                                           f2 cp2, f2 cm1, f2 cm2, f2 cm3, f2 mu2) {
-    if (kind == kPosPart) return pos_part_x2(mul2s(cp0, x0), mul2s(cp1, x1), mul2s(cp2, x2), mu2);
-    if (kind == kNegPart) return neg_part_x2(mul2s(cm1, x1), mul2s(cm2, x2), mul2s(cm3, x3), mu2);
-    return add2(pos_part_x2(mul2s(cp0, x0), mul2s(cp1, x1), mul2s(cp2, x2), mu2),
-                neg_part_x2(mul2s(cm1, x1), mul2s(cm2, x2), mul2s(cm3, x3), mu2));
+                                           f2 cp2, f2 cm1, f2 cm2, f2 cm3, const LimPair& k) {
+    auto mul = [&](f2 a, f2 b) { return fma2(a, b, k.zero2); };
+    if (kind == kPosPart) return pos_part_x2(mul(cp0, x0), mul(cp1, x1), mul(cp2, x2), k);
+    if (kind == kNegPart) return neg_part_x2(mul(cm1, x1), mul(cm2, x2), mul(cm3, x3), k);
+    return add2(pos_part_x2(mul(cp0, x0), mul(cp1, x1), mul(cp2, x2), k),
+                neg_part_x2(mul(cm1, x1), mul(cm2, x2), mul(cm3, x3), k));
 }
 
 // f* of cells x and x + 1 (column jx, all rows) into a plane; zeros beyond N_x.
@@ -669,7 +665,7 @@ __device__ __forceinline__ void limp_load(const float* fin, float* plane, int nx
 // One Heun stage on column jx for the cell pair at offset c (as lim_fused_stage).
 template <int NV, int TC, int STAGE, int UNR>
 __device__ __forceinline__ void limp_stage(const float* src, float* dst, int jx, int c, bool store,
-                                           f2 g2, f2 wy2, f2 mu2, const f2 (&cxp)[5],
+                                           f2 g2, f2 wy2, const LimPair& lk, const f2 (&cxp)[5],
                                            const f2 (&cxm)[5], int kl, int kr, int kyp, int kyn) {
     using L = LimPacked<NV, TC>;
     constexpr int J = L::J, R = L::kRow;
@@ -683,8 +679,8 @@ __device__ __forceinline__ void limp_stage(const float* src, float* dst, int jx,
         const int jr = k - 1;
         v[k] = jr < NV ? ld2s(col + jr * R) : z;
         const f2 ca = mul2(g2, sub2(wy2, splat((float)(jr - J))));
-        P[k] = mul2(max0(ca), v[k]);
-        M[k] = mul2(min0(ca), v[k]);
+        P[k] = fma2(max0(ca), v[k], lk.zero2);
+        M[k] = fma2(min0(ca), v[k], lk.zero2);
     }
     f2 Fyl = z;
 #pragma unroll(UNR)
@@ -692,14 +688,14 @@ __device__ __forceinline__ void limp_stage(const float* src, float* dst, int jx,
         f2 Fyr = z;
         if (jy < NV - 1)
             Fyr = face_parts_x2(face_kind(jy - 1, kyp, kyn), P[0], P[1], P[2], M[1], M[2], M[3],
-                                mu2);
+                                lk);
         const float* rp = col + jy * R;
         const f2 xm2 = ld2s(rp - 2 * TC), xm1 = ld2s(rp - TC), x0 = v[1], xp1 = ld2s(rp + TC),
                  xp2 = ld2s(rp + 2 * TC);
         f2 Fxl = face_vals_x2(kl, xm2, xm1, x0, xp1, cxp[0], cxp[1], cxp[2], cxm[1], cxm[2],
-                              cxm[3], mu2);
+                              cxm[3], lk);
         f2 Fxr = face_vals_x2(kr, xm1, x0, xp1, xp2, cxp[1], cxp[2], cxp[3], cxm[2], cxm[3],
-                              cxm[4], mu2);
+                              cxm[4], lk);
         if (jx == 0) Fxl = z;
         if (jx == NV - 1) Fxr = z;
         const f2 sv = sub2(sub2(x0, sub2(Fxr, Fxl)), sub2(Fyr, Fyl));
@@ -718,15 +714,15 @@ __device__ __forceinline__ void limp_stage(const float* src, float* dst, int jx,
         const f2 vn = ld2s(col + (jn < NV ? jn : NV - 1) * R);
         v[3] = jn < NV ? vn : z;
         const f2 ca = mul2(g2, sub2(wy2, splat((float)(jn - J))));
-        P[3] = mul2(max0(ca), v[3]);
-        M[3] = mul2(min0(ca), v[3]);
+        P[3] = fma2(max0(ca), v[3], lk.zero2);
+        M[3] = fma2(min0(ca), v[3], lk.zero2);
     }
 }
 
 // Diffusion of column jx for the cell pair (as lim_fused_diffuse); st0/st1: the cells to store.
 template <int NV, int TC, int UNR>
 __device__ __forceinline__ void limp_diffuse(const float* plane, float* gout, size_t ncell, int jx,
-                                             int c, bool st0, bool st1, bool vec, f2 r2) {
+                                             int c, bool st0, bool st1, bool vec, f2 r2, f2 zero2) {
     using L = LimPacked<NV, TC>;
     constexpr int R = L::kRow;
     const float* col = plane + (jx + 2) * TC + c;
@@ -737,13 +733,11 @@ __device__ __forceinline__ void limp_diffuse(const float* plane, float* gout, si
         const f2 hnext = ld2s(col + (jy < NV - 1 ? jy + 1 : jy) * R);
         const f2 hp = jy < NV - 1 ? hnext : z;
         const f2 hl = ld2s(col + jy * R - TC), hr = ld2s(col + jy * R + TC);
-        const f2 Dxr = jx < NV - 1 ? mul2(r2, sub2(hr, h0)) : z;
-        const f2 Dxl = jx > 0 ? mul2(r2, sub2(h0, hl)) : z;
-        const f2 Dyr = jy < NV - 1 ? mul2(r2, sub2(hp, h0)) : z;
-        const f2 Dyl = jy > 0 ? mul2(r2, sub2(h0, hm)) : z;
-        // the differences of two products by r lane by lane (sub2s): with sub.rn.f32x2 there,
-        // a few cells came out one unit in the last place away from the scalar kernel's
-        const f2 o = add2(add2(h0, sub2s(Dxr, Dxl)), sub2s(Dyr, Dyl));
+        const f2 Dxr = jx < NV - 1 ? fma2(r2, sub2(hr, h0), zero2) : z;
+        const f2 Dxl = jx > 0 ? fma2(r2, sub2(h0, hl), zero2) : z;
+        const f2 Dyr = jy < NV - 1 ? fma2(r2, sub2(hp, h0), zero2) : z;
+        const f2 Dyl = jy > 0 ? fma2(r2, sub2(h0, hm), zero2) : z;
+        const f2 o = add2(add2(h0, sub2(Dxr, Dxl)), sub2(Dyr, Dyl));
         float* gp = gout + (size_t)jy * NV * ncell;
         if (vec) {
             st2s(gp, o);
@@ -773,7 +767,8 @@ __global__ void __launch_bounds__(LimPacked<NV, TC>::kThreads, MINB)
     const float* u = static_cast<const float*>(a.u);
     const float g = (float)a.g, mu = (float)a.mu, inv_dv = (float)a.inv_dv;
     const float cflf = O::mul(g, O::add(1.f, mu));
-    const f2 g2 = splat(g), mu2 = splat(mu), r2 = splat((float)a.r);
+    const f2 g2 = splat(g), r2 = splat((float)a.r);
+    const LimPair lk{splat(mu), splat((float)(1.0 / 3.0)), splat((float)(1.0 / 6.0)), opaque2(0ull)};
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = 2 * (lane % L::LPC);
     const int jx_raw = warp * L::CPW + lane / L::LPC;
@@ -833,9 +828,9 @@ __global__ void __launch_bounds__(LimPacked<NV, TC>::kThreads, MINB)
         const int kr = uniform_kind(face_kind(jx - 1, kxp, kxn));
         cp_async_wait_all();
         __syncthreads();
-        limp_stage<NV, TC, 1, UNR>(pa, pb, jx, c, active, g2, wy2, mu2, cxp, cxm, kl, kr, kyp, kyn);
+        limp_stage<NV, TC, 1, UNR>(pa, pb, jx, c, active, g2, wy2, lk, cxp, cxm, kl, kr, kyp, kyn);
         __syncthreads();
-        limp_stage<NV, TC, 2, UNR>(pb, pa, jx, c, active, g2, wy2, mu2, cxp, cxm, kl, kr, kyp, kyn);
+        limp_stage<NV, TC, 2, UNR>(pb, pa, jx, c, active, g2, wy2, lk, cxp, cxm, kl, kr, kyp, kyn);
         __syncthreads();
         const long long tn = t + gridDim.x;
         if (tn < ntiles && active) {
@@ -844,7 +839,7 @@ __global__ void __launch_bounds__(LimPacked<NV, TC>::kThreads, MINB)
         }
         float* gout = fout + ((size_t)jx * ny + y) * nx + (in0 ? x : 0);
         limp_diffuse<NV, TC, UNR>(pa, gout, ncell, jx, c, active && in0, active && in1,
-                                  active && in1 && even, r2);
+                                  active && in1 && even, r2, lk.zero2);
         float* tmp = pa;
         pa = pb;
         pb = tmp;
