@@ -755,7 +755,7 @@ int enqueue_moments(lat_ctx* c, double* rho, double* mean_v, double* mean_v2, do
     a.mean_v2 = mean_v2;
     a.partials = c->d_partials;
     a.st = c->d_state;
-    const int grid = std::max(1, std::min(c->nitems, 8 * c->sm_count));
+    const int grid = std::max(1, c->nitems);
     CK(launch_moments1d(c->dtype, tile_of(c), 1, grid, a, c->stream));
     return finalize_1d(c, tile_of(c) / 32, gdst, wait);
 }

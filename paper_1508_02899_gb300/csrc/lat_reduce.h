@@ -170,11 +170,19 @@ __device__ __forceinline__ void warp_partial_1d(const ColumnSums& cs_, double dv
     warp_reduce(a0);
     warp_reduce(a1);
     warp_reduce(a2);
-    if ((threadIdx.x & 31) == 0) {
-        const Comp t0 = a0.to_comp(1.0), t1 = a1.to_comp(dv), t2 = a2.to_comp(__dmul_rn(dv, dv));
-        p[0] = t0.s; p[1] = t0.c;
-        p[2] = t1.s; p[3] = t1.c;
-        p[4] = t2.s; p[5] = t2.c;
+    // lanes 0, 1, 2 scale one sum each: four FP64 instructions of the warp instead of twelve
+    const int lane = threadIdx.x & 31;
+    auto of = [&](float v0, float v1, float v2) {
+        v0 = __shfl_sync(0xffffffffu, v0, 0);
+        v1 = __shfl_sync(0xffffffffu, v1, 0);
+        v2 = __shfl_sync(0xffffffffu, v2, 0);
+        return lane == 0 ? v0 : lane == 1 ? v1 : v2;
+    };
+    const FComp a{of(a0.s, a1.s, a2.s), of(a0.c, a1.c, a2.c)};
+    if (lane < 3) {
+        const Comp t = a.to_comp(lane == 0 ? 1.0 : lane == 1 ? dv : __dmul_rn(dv, dv));
+        p[2 * lane] = t.s;
+        p[2 * lane + 1] = t.c;
     }
 }
 
