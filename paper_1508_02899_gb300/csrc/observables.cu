@@ -33,12 +33,17 @@ __device__ __forceinline__ Comp block_reduce(Comp t) {
 }
 
 // Exclusive prefix sums of rho per instance, compensated (hi + lo): instance k's n + 1 sums
-// start at xoff_k + k.  One block per instance; chunks of the block width in order, a warp scan
-// per chunk.  Window sums are then differences of prefix sums, accurate to about u of the window
-// (u = 2^-53) however long the instance.
-__global__ void __launch_bounds__(kObsThreads)
+// start at xoff_k + k.  One block per instance; chunks of kPrefixThreads kPrefixCells cells in order.
+// Window sums are then differences of prefix sums, accurate to about u of the window (u = 2^-53)
+// however long the instance.
+// Bound by the FP64 pipe: a thread adds kPrefixCells cells one after the other, so that the scan of the
+// threads' totals (a merge costs as much as a cell's addition, five per warp scan) is shared by them.
+// 1024 instances, N_x 1024 .. 8192: 226 us; a cell per thread 776 us.
+constexpr int kPrefixThreads = 128, kPrefixCells = 8;
+
+__global__ void __launch_bounds__(kPrefixThreads)
     k_prefix1d(const double* rho, const Inst1D* inst, int n_inst, double* Ph, double* Pl) {
-    __shared__ Comp wtot[kObsThreads / 32];
+    __shared__ Comp wtot[kPrefixThreads / 32];
     __shared__ Comp carry;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = blockIdx.x; k < n_inst; k += gridDim.x) {
@@ -48,9 +53,18 @@ __global__ void __launch_bounds__(kObsThreads)
         double* pl = Pl + in.xoff + k;
         if (threadIdx.x == 0) carry = Comp{0, 0};
         __syncthreads();
-        for (int base = 0; base < in.nx; base += kObsThreads) {
-            const int i = base + threadIdx.x;
-            Comp incl{i < in.nx ? r[i] : 0.0, 0.0};
+        for (int base = 0; base < in.nx; base += kPrefixThreads * kPrefixCells) {
+            const int i0 = base + (int)threadIdx.x * kPrefixCells;
+            double v[kPrefixCells];
+#pragma unroll
+            for (int q = 0; q < kPrefixCells; ++q) v[q] = i0 + q < in.nx ? r[i0 + q] : 0.0;
+            Comp part[kPrefixCells];  // the sums before each of the thread's cells
+            Comp incl{0, 0};
+#pragma unroll
+            for (int q = 0; q < kPrefixCells; ++q) {
+                part[q] = incl;
+                nadd(incl, v[q]);
+            }
             for (int off = 1; off < 32; off <<= 1) {  // inclusive scan, predecessors first
                 const Comp o = shfl_up(incl, off);
                 if (lane >= off) {
@@ -65,14 +79,18 @@ __global__ void __launch_bounds__(kObsThreads)
             __syncthreads();
             Comp before = carry;
             for (int w = 0; w < warp; ++w) nmerge(before, wtot[w]);
-            if (i < in.nx) {
-                Comp v = before;
-                nmerge(v, excl);
-                ph[i] = v.s;
-                pl[i] = v.c;
+            Comp own = before;
+            nmerge(own, excl);
+#pragma unroll
+            for (int q = 0; q < kPrefixCells; ++q) {
+                if (i0 + q >= in.nx) break;
+                Comp t = own;
+                nmerge(t, part[q]);
+                ph[i0 + q] = t.s;
+                pl[i0 + q] = t.c;
             }
             __syncthreads();
-            if (threadIdx.x == kObsThreads - 1) {
+            if (threadIdx.x == kPrefixThreads - 1) {
                 nmerge(before, incl);
                 carry = before;
             }
@@ -314,7 +332,7 @@ cudaError_t launch_coarse1d(const double* rho, const Inst1D* inst, int n_inst, l
                             const int* widths, int nw, double* P, double* out, int sm_count,
                             cudaStream_t s) {
     double* Pl = P + total_x + n_inst;
-    k_prefix1d<<<obs_grid(n_inst, sm_count), kObsThreads, 0, s>>>(rho, inst, n_inst, P, Pl);
+    k_prefix1d<<<obs_grid(n_inst, sm_count), kPrefixThreads, 0, s>>>(rho, inst, n_inst, P, Pl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     k_coarse1d<<<obs_grid((long long)n_inst * nw, sm_count), kObsThreads, 0, s>>>(
