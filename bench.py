@@ -114,9 +114,10 @@ CLOSURE_PARAMS = os.path.join(ROOT, "paper_1508_02899_gb300", "closure_params.np
 EVAL_FINE_STEPS = (100, 400)
 
 KERNEL_PROFILES = {
-    "ensemble": ("step1d_ensemble_fp32_nv65.md", (_CSRC + "step1d.cu", _CSRC + "f32x2.h")),
-    "ensemble_koren": ("step1d_ensemble_koren_fp32_nv65.md",
-                       (_CSRC + "step1d.cu", _CSRC + "f32x2.h")),
+    "ensemble": ("multi1d_ensemble_fp32_nv65.md",
+                 (_CSRC + "multi1d.cu", _CSRC + "step1d_dev.h", _CSRC + "f32x2.h")),
+    "ensemble_koren": ("lim1d_ensemble_koren_fp32_nv65.md",
+                       (_CSRC + "lim1d.cu", _CSRC + "step1d_dev.h", _CSRC + "f32x2.h")),
     "2d": ("step2d_512_fp32_nv33.md", (_CSRC + "step2d.cu", _CSRC + "step2d_dev.h",
                                        _CSRC + "step2d_x2.h", _CSRC + "f32x2.h")),
     "2d_f16": ("step2d_1024_f16_nv33.md", (_CSRC + "step2d_h.cu", _CSRC + "step2d_dev.h")),
@@ -483,8 +484,31 @@ def end_to_end(ctx, noise, first, glob, steps, torch, pipelined=True):
     return time.perf_counter() - t0, int(rows[0].numel() * 8), int(glob.size * 8), masses
 
 
-def kernel_label(workload, best, nv):
+MULTI_STEPS = 5  # steps of a launch of the several-steps kernel
+
+
+def on_chip_ensemble(nv):
+    """Whether batches of steps of an FP32 ensemble run on the kernels that hold a tile's column on
+    chip (k_multi1d, k_lim1d) unless a launch kernel is chosen."""
+    return nv in (9, 17, 33, 65)
+
+
+def ensemble_launches(K, nv, cells, scheme):
+    """Kernels of one enqueued batch of K steps of the ensemble, by default (no launch kernel chosen)."""
+    if not on_chip_ensemble(nv):
+        return K + 1
+    full, rest = divmod(K, MULTI_STEPS)
+    if scheme == "upwind":  # the flow of five steps and the steps; then one by one
+        return 2 * full + rest + 1
+    # the flow of five steps, one limited step per launch; the flow of odd counts for the rest
+    flows = (0, 1, 2, 1, 2)[rest] if nv >= 33 and cells >= 8 << 20 else 0
+    return full + flows + K + 1
+
+
+def kernel_label(workload, best, nv, chosen=False, scheme="upwind"):
     k = best["kernel"] if best else 0
+    if workload == "ensemble" and not chosen and on_chip_ensemble(nv):
+        return f"k_multi1d<{nv}>" if scheme == "upwind" else f"k_lim1d<{nv}>"
     if workload in ("2d_f16", "2d_bf16"):
         t = "__half" if workload == "2d_f16" else "__nv_bfloat16"
         if k >= 4:
@@ -590,7 +614,14 @@ def main():
     # one read and one write of every cell; 16-bit storage adds per line its input scale, its
     # output scale and its recorded maximum (4 bytes each)
     bytes_per_launch = cells * bytes_per_cell + lines * 12
-    achieved = bytes_per_launch / (ms_max / K / 1e3) / 1e9
+    launches, steps_per_launch = launches_per_step * K + 1, 1
+    if args.workload == "ensemble" and not args.launch:
+        # a batch reads its flow from rows formed ahead; the upwind kernel takes five steps per launch
+        launches = ensemble_launches(K, nv, cells, args.scheme)
+        if on_chip_ensemble(nv):
+            steps_per_launch = MULTI_STEPS if args.scheme == "upwind" and K >= MULTI_STEPS else 1
+            bytes_per_launch += steps_per_launch * 4 * (cells // nv)
+    achieved = bytes_per_launch / (ms_max / K * steps_per_launch / 1e3) / 1e9
     roof = None
     if args.workload == "2d_learned":
         # dominant kernel: the tensor-core network, timed alone with CUDA events
@@ -601,7 +632,8 @@ def main():
         roof = {"bound": "tensor", "achieved": tf, "peak": tpeak, "unit": "TFLOP/s",
                 "frac": tf / tpeak, "traffic": None, "peak_source": tsrc,
                 "kernel": "k_mlp_tc_units<9>", "flop_per_launch": flops, "ms_per_launch": net_ms}
-    tr = profile_traffic(prof, src)
+    # (the ensemble's summaries are those of its default kernels)
+    tr = None if args.workload == "ensemble" and args.launch else profile_traffic(prof, src)
     traffic = None
     if tr is not None:
         tb, units = tr
@@ -659,7 +691,8 @@ def main():
             g2 = c2 * 40 / (ms2 / 1e3) / 1e9
             forms["ensemble_koren_fp32_nv65"] = {
                 "gcups": g2, "ms_per_step": ms2 / 40, "hbm_frac": g2 * 8 / peak,
-                "kernel": kernel_label("ensemble", b2, NV), "steps": 40, "status": st2}
+                "kernel": kernel_label("ensemble", b2, NV, scheme="koren"), "steps": 40,
+                "status": st2}
             lt.close()
             del lt
             torch.cuda.empty_cache()
@@ -782,15 +815,17 @@ def main():
             "roofline": roof or {"bound": "hbm", "achieved": achieved, "peak": peak,
                                  "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
                                  "peak_source": peak_src,
-                                 "kernel": kernel_label(args.workload, best, nv),
-                                 "bytes_per_launch": bytes_per_launch},
+                                 "kernel": kernel_label(args.workload, best, nv,
+                                                        bool(args.launch), args.scheme),
+                                 "bytes_per_launch": bytes_per_launch,
+                                 "steps_per_launch": steps_per_launch},
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": UNIT, "steps": K_e2e,
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "api": "lat_step_moments_async, globals read one step behind",
                     "sync_value": e2e_sync, "sync_api": "lat_step_moments (synchronises)",
                     "status": e2e_status, "mass_rel_spread": mass_drift},
-            "gpu_launches": launches_per_step * K + 1,
+            "gpu_launches": launches,
             "clocks": ck,
         }
         if per_inst_ms is not None:

@@ -12,7 +12,8 @@
 // mbarrier) into a 4-slot ring, two rows ahead of the sweep: the streaming shift is applied by
 // the copy's source address (x window rounded down to 16 bytes, split in two at the periodic
 // wrap; y wraps by choosing the source row).  A plain-load variant with the same arithmetic
-// serves FP64 and grids the copy path does not cover (N_x not a multiple of 4, or < 132).
+// serves grids the copy path does not cover (N_x not a multiple of 4, or < 132); FP64 lattices have
+// their own kernel (step2d_f64.cu).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
