@@ -924,7 +924,8 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
              q += (long long)gridDim.x * blockDim.x) {
             const long long c = PAIR ? 2 * q : q;
             // scales of this cell's row: [jy][jx padded]
-            const float* sc_c = scales ? scales + (size_t)(c / nx) * nv * nv_padded(nv) : nullptr;
+            const float* sc_c =
+                sizeof(T) == 2 ? scales + (size_t)(c / nx) * nv * nv_padded(nv) : nullptr;
             f2 S = 0ull, C = 0ull, s1 = 0ull, s2 = 0ull, s3 = 0ull;  // mass (sum, -error); weighted
             for (int jy = 0; jy < nv; ++jy) {
                 const float fy = (float)(jy - J);
@@ -935,7 +936,7 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
                 for (int jx = 0; jx < nv; ++jx) {
                     const float fx = (float)(jx - J);
                     f2 v = load_cells<T, PAIR>(fr + (size_t)jx * ncell);
-                    if (sc_c) {  // exact: powers of two
+                    if constexpr (sizeof(T) == 2) {  // exact: powers of two
                         const float sv = sc_c[jy * nv_padded(nv) + jx];
                         v = fma2(v, pk(sv, sv), zero2);
                     }
@@ -1814,6 +1815,11 @@ int copy_globals(Ctx2D* c, double* globals, bool wait, cudaStream_t s) {
     return LAT_OK;
 }
 
+// Cells from which the moments take two per thread: a smaller grid does not fill the SMs with a thread
+// per cell (one step and moments, pair against single: 456 x 213, N_v = 19 253 and 235 us; 64^2, 17
+// 140 and 127 us; 512 x 400, 19 325 and 377 us).
+constexpr long long kPairCells = 1 << 17;
+
 int ctx2d_moments(Ctx2D* c, const void* f, int cur, double* rho, double* mean_v,
                   double* mean_v2, double* globals, bool wait, cudaStream_t s) {
     const float* sc = c->half ? c->d_sc + (size_t)cur * c->nlines : nullptr;
@@ -1821,8 +1827,9 @@ int ctx2d_moments(Ctx2D* c, const void* f, int cur, double* rho, double* mean_v,
         kernel<<<c->mom_blocks, 32 * kMom2DWarps, 0, s>>>(f, sc, c->nv, c->nx, c->ny, c->dv, rho,
                                                          mean_v, mean_v2, c->d_partials, c->st);
     };
-    // pairs of cells where a pair lies in one grid row and is aligned
-    const bool pair = c->nx % 2 == 0 && (uintptr_t)f % 8 == 0;
+    // pairs of cells where a pair lies in one grid row and is aligned, on grids that fill the SMs
+    const bool pair = c->nx % 2 == 0 && (uintptr_t)f % 8 == 0 &&
+                      (long long)c->nx * c->ny >= kPairCells;
     if (c->dtype == LAT_F16)
         pair ? run(k_moments2d<__half, true>) : run(k_moments2d<__half>);
     else if (c->dtype == LAT_BF16)

@@ -591,7 +591,15 @@ __global__ void __launch_bounds__(256) k_decode(const S* f, const float* sc, flo
                 reinterpret_cast<float4*>(out)[2 * c + 1] = o[1];
             }
         } else {
-            for (int x = lane; x < nx; x += 32) out[x] = __fmul_rn(HTraits<S>::dec(row[x]), s);
+            for (int x = lane; x < nx; x += 128) {  // four loads in flight
+                S h[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (x + 32 * e < nx) h[e] = row[x + 32 * e];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (x + 32 * e < nx) out[x + 32 * e] = __fmul_rn(HTraits<S>::dec(h[e]), s);
+            }
         }
     }
 }
