@@ -152,9 +152,9 @@ int build_items(lat_ctx* c) {
                    sizeof(double) * 6 * std::max(kPcConsumerWarps, tile / 32) * items.size()) !=
             cudaSuccess)
         return LAT_ENOMEM;
-    CK(cudaMemcpy(c->d_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->d_inst_begin, c->h_inst_begin.data(), sizeof(int) * (c->n_inst + 1),
-                  cudaMemcpyHostToDevice));
+    CK(upload(c->d_items, items.data(), sizeof(int2) * items.size(), c->stream));
+    CK(upload(c->d_inst_begin, c->h_inst_begin.data(), sizeof(int) * (c->n_inst + 1),
+              c->stream));
     drop_graphs(c);
     return LAT_OK;
 }
@@ -289,7 +289,7 @@ int build_tiles(lat_ctx* c, bool lim) {
         cudaGetLastError();
         return LAT_OK;
     }
-    CK(cudaMemcpy(t.d, tiles.data(), sizeof(MultiTile) * tiles.size(), cudaMemcpyHostToDevice));
+    CK(upload(t.d, tiles.data(), sizeof(MultiTile) * tiles.size(), c->stream));
     t.n = (int)tiles.size();
     return LAT_OK;
 }
@@ -323,8 +323,7 @@ int build_multi(lat_ctx* c) {
         cudaGetLastError();  // no room for them: steps are launched one by one
         return LAT_OK;
     }
-    CK(cudaMemcpy(c->d_basis_off, off.data(), sizeof(long long) * c->n_inst,
-                  cudaMemcpyHostToDevice));
+    CK(upload(c->d_basis_off, off.data(), sizeof(long long) * c->n_inst, c->stream));
     if (total > 0) {
         const Step1DArgs a = step_args(c, 0, 0);
         for (const auto& e : sizes)
@@ -499,8 +498,7 @@ int lat_ensemble_init(lat_ctx** out, int n_inst, const lat_instance* inst, int n
     if (rc == LAT_OK && cudaMallocHost(&c->h_glob, sizeof(double) * 4 * n_inst) != cudaSuccess)
         rc = LAT_ENOMEM;
     if (rc == LAT_OK &&
-        cudaMemcpy(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * n_inst, cudaMemcpyHostToDevice) !=
-            cudaSuccess)
+        upload(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * n_inst, c->stream) != cudaSuccess)
         rc = LAT_ECUDA;
     if (rc == LAT_OK) {
         // default launch shape: the producer/consumer bulk-copy pipeline where every instance
@@ -600,10 +598,10 @@ int lat_set_flow(lat_ctx* c, const lat_flow* fl) {
         }
         // both parities start from amp0 so that a frozen flow reads the same values every step
         std::vector<float> a32(fl->amp0, fl->amp0 + stride);
-        CK(cudaMemcpy(amp, fl->amp0, sizeof(double) * stride, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(amp + stride, fl->amp0, sizeof(double) * stride, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(ampf, a32.data(), sizeof(float) * stride, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(ampf + stride, a32.data(), sizeof(float) * stride, cudaMemcpyHostToDevice));
+        CK(upload(amp, fl->amp0, sizeof(double) * stride, c->stream));
+        CK(upload(amp + stride, fl->amp0, sizeof(double) * stride, c->stream));
+        CK(upload(ampf, a32.data(), sizeof(float) * stride, c->stream));
+        CK(upload(ampf + stride, a32.data(), sizeof(float) * stride, c->stream));
         if (c->d_amp) cudaFree(c->d_amp);
         if (c->d_ampf) cudaFree(c->d_ampf);
         c->d_amp = amp;
@@ -624,8 +622,7 @@ int lat_set_flow(lat_ctx* c, const lat_flow* fl) {
                 q.ou_s = fl->sigma * sqrt(1.0 - q.ou_e * q.ou_e);
             }
         }
-        CK(cudaMemcpy(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * c->n_inst,
-                      cudaMemcpyHostToDevice));
+        CK(upload(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * c->n_inst, c->stream));
     } else {
         return LAT_EINVAL;
     }

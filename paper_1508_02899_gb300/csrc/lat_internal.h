@@ -18,6 +18,14 @@
 
 namespace lat {
 
+// A host array into a device table that kernels of stream s read, done on return.  Always on the
+// context's own stream: a copy from pageable memory on the default stream may return before its last
+// transfer is done, and a non-blocking stream (such as PyTorch's) does not wait for that one.
+inline cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(s);
+}
+
 // Device status bits; translated to LAT_E* codes by the host.
 enum : unsigned {
     ST_CFL = 1u,       // Eq. (cfl) violated by the evolving flow
