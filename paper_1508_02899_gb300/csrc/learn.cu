@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "learn.h"
+#include "per_device.h"
 
 namespace lat {
 namespace {
@@ -549,14 +550,12 @@ cudaError_t launch_mlp_f32(int nv, const LearnArgs& a, int k, cudaStream_t s) {
 // would leave its last blocks to run their whole tile loops after the others finish.
 template <int NV>
 int corr_grid(int sm_count, int ntiles) {
-    static int occ = 0;
-    if (occ == 0) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step2d_corr<NV>, TW, 0) !=
-            cudaSuccess)
-            nb = 1;
-        occ = nb > 0 ? nb : 1;
-    }
+    static PerDevice resident;
+    int occ = 1;
+    if (resident.get(&occ, [](int* n) {
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_step2d_corr<NV>, TW, 0);
+        }) != cudaSuccess)
+        occ = 1;
     return std::max(1, std::min(ntiles, occ * sm_count));
 }
 

@@ -30,6 +30,7 @@
 #include <algorithm>
 
 #include "learn.h"
+#include "per_device.h"
 
 namespace lat {
 namespace {
@@ -985,14 +986,9 @@ cudaError_t launch_mlp_bwd_tc(int nv, const LearnBwdArgs& b, const void* wtc, in
     switch (nv) {
 #define X(nn)                                                                                   \
     case nn: {                                                                                  \
-        static bool attr = false;                                                               \
-        if (!attr) {                                                                            \
-            cudaError_t e = cudaFuncSetAttribute(k_mlp_bwd_tc<nn>,                              \
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                                 kBSmem);                                       \
-            if (e != cudaSuccess) return e;                                                     \
-            attr = true;                                                                        \
-        }                                                                                       \
+        static PerDevice limit;                                                                 \
+        const cudaError_t e = raise_smem(limit, k_mlp_bwd_tc<nn>, kBSmem);                      \
+        if (e != cudaSuccess) return e;                                                         \
         k_mlp_bwd_tc<nn><<<grid, 128, kBSmem, s>>>(b, img);                                     \
         return cudaGetLastError();                                                              \
     }
@@ -1013,17 +1009,10 @@ cudaError_t launch_mlp_tc(int nv, const LearnArgs& a, const void* wtc, int sm_co
     switch (nv) {
 #define X(nn)                                                                                   \
     case nn: {                                                                                  \
-        static bool attr = false;                                                               \
-        if (!attr) {                                                                            \
-            cudaError_t e = cudaFuncSetAttribute(k_mlp_tc<nn>,                                  \
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                                 kSmemReq);                                     \
-            if (e == cudaSuccess)                                                               \
-                e = cudaFuncSetAttribute(k_mlp_tc_units<nn>,                                    \
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemReq); \
-            if (e != cudaSuccess) return e;                                                     \
-            attr = true;                                                                        \
-        }                                                                                       \
+        static PerDevice limit, limit_units;                                                    \
+        cudaError_t e = raise_smem(limit, k_mlp_tc<nn>, kSmemReq);                              \
+        if (e == cudaSuccess) e = raise_smem(limit_units, k_mlp_tc_units<nn>, kSmemReq);        \
+        if (e != cudaSuccess) return e;                                                         \
         if (by_units) k_mlp_tc_units<nn><<<grid, 128, kSmemReq, s>>>(a, img, k);                \
         else k_mlp_tc<nn><<<grid, 128, kSmemReq, s>>>(a, img, k);                               \
         return cudaGetLastError();                                                              \

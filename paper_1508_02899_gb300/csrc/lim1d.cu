@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "lat_internal.h"
+#include "per_device.h"
 #include "step1d_dev.h"
 
 namespace lat {
@@ -270,13 +271,9 @@ template <int NV>
 cudaError_t launch_t(int ntiles, int places, const Step1DArgs& a, const MultiTile* tiles, int kstep,
                      const float* wrow, int piped, cudaStream_t s) {
     constexpr int kSmem = 4 * ((NV + 1) * kPitch + kPlaces) + 16;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_lim1d<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice limit;
+    const cudaError_t e = raise_smem(limit, k_lim1d<NV>, kSmem);
+    if (e != cudaSuccess) return e;
     k_lim1d<NV><<<ntiles, places / 2, kSmem, s>>>(a, tiles, kstep, wrow, piped);
     return cudaGetLastError();
 }

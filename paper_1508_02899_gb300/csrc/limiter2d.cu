@@ -18,6 +18,7 @@
 // lets one block finish a tile of cells without touching its neighbours.
 #include "f32x2.h"
 #include "lat_internal.h"
+#include "per_device.h"
 #include "step2d_dev.h"
 
 namespace lat {
@@ -560,20 +561,13 @@ __global__ void __launch_bounds__(LimFused<T, NV, TC>::kThreads, MINB)
 template <typename T, int NV, int TC, int MINB, int UNR = 4>
 cudaError_t launch_fused_t(const Lim2DArgs& a, int k, int sm_count, cudaStream_t s) {
     using L = LimFused<T, NV, TC>;
-    static bool attr = false;
-    static int per_sm = 0;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_lim2d_fused<T, NV, TC, MINB, UNR>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)L::kSmem);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lim2d_fused<T, NV, TC, MINB, UNR>,
-                                                          L::kThreads, L::kSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice resident;
+    int per_sm = 0;
+    const cudaError_t e = resident_blocks(resident, k_lim2d_fused<T, NV, TC, MINB, UNR>, L::kThreads,
+                                          L::kSmem, &per_sm);
+    if (e != cudaSuccess) return e;
     const long long ntiles = (long long)((a.nx + TC - 1) / TC) * a.ny;
-    const int grid = (int)std::min<long long>(ntiles, (long long)std::max(per_sm, 1) * sm_count);
+    const int grid = (int)std::min<long long>(ntiles, (long long)per_sm * sm_count);
     k_lim2d_fused<T, NV, TC, MINB, UNR><<<grid, L::kThreads, L::kSmem, s>>>(a, k);
     return cudaGetLastError();
 }
@@ -851,20 +845,13 @@ __global__ void __launch_bounds__(LimPacked<NV, TC>::kThreads, MINB)
 template <int NV, int TC, int MINB, int UNR = 4>
 cudaError_t launch_packed_t(const Lim2DArgs& a, int k, int sm_count, cudaStream_t s) {
     using L = LimPacked<NV, TC>;
-    static bool attr = false;
-    static int per_sm = 0;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_lim2d_packed<NV, TC, MINB, UNR>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)L::kSmem);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, k_lim2d_packed<NV, TC, MINB, UNR>, L::kThreads, L::kSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice resident;
+    int per_sm = 0;
+    const cudaError_t e = resident_blocks(resident, k_lim2d_packed<NV, TC, MINB, UNR>, L::kThreads,
+                                          L::kSmem, &per_sm);
+    if (e != cudaSuccess) return e;
     const long long ntiles = (long long)((a.nx + TC - 1) / TC) * a.ny;
-    const int grid = (int)std::min<long long>(ntiles, (long long)std::max(per_sm, 1) * sm_count);
+    const int grid = (int)std::min<long long>(ntiles, (long long)per_sm * sm_count);
     k_lim2d_packed<NV, TC, MINB, UNR><<<grid, L::kThreads, L::kSmem, s>>>(a, k);
     return cudaGetLastError();
 }

@@ -25,9 +25,9 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "lat_internal.h"
+#include "per_device.h"
 #include "step1d_dev.h"
 
 namespace lat {
@@ -240,16 +240,15 @@ template <typename T, bool ONE>
 cudaError_t config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int n_inst, int nv, int w,
                    int nmodes, cudaStream_t s) {
     const size_t smem = line_smem<T>(nv, w, nmodes);
-    static std::atomic<size_t> allowed{0};
-    if (smem > allowed) {
-        cudaError_t e = cudaFuncSetAttribute(
-            k_line1d<T, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_line1d<T, ONE>,
-                                     cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-        allowed = kMaxSmem;
-    }
+    static PerDevice limit, size;
+    cudaError_t e = raise_smem(limit, k_line1d<T, ONE>, kMaxSmem);
+    int done = 0;
+    if (e == cudaSuccess)
+        e = size.get(&done, [](int*) {
+            return cudaFuncSetAttribute(k_line1d<T, ONE>,
+                                        cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        });
+    if (e != cudaSuccess) return e;
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3(n_inst * kCluster);
     cfg->blockDim = dim3(std::min(kCellThreads, (nv * w + 31) / 32 * 32) + 32);

@@ -39,6 +39,7 @@
 #include <algorithm>
 
 #include "lat_internal.h"
+#include "per_device.h"
 #include "step1d_dev.h"
 
 namespace lat {
@@ -460,14 +461,10 @@ namespace {
 template <int NV>
 cudaError_t launch_t(int T, int ntiles, int places, const Step1DArgs& a, const MultiTile* tiles,
                      int kstep, int piped, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(
-            k_multi1d<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kSmemWords);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    cudaError_t e = launch_flow_steps(LAT_F32, a, kstep, T, s);
+    static PerDevice limit;
+    cudaError_t e = raise_smem(limit, k_multi1d<NV>, 4 * kSmemWords);
+    if (e != cudaSuccess) return e;
+    e = launch_flow_steps(LAT_F32, a, kstep, T, s);
     if (e != cudaSuccess) return e;
     const size_t smem = 4 * ((size_t)NV * Shape<NV>::kPitch + side_words(Shape<NV>::J, T, places));
     k_multi1d<NV><<<ntiles, places / 2, smem, s>>>(a, tiles, kstep, T, piped);

@@ -23,6 +23,7 @@
 #include <algorithm>
 
 #include "lat_internal.h"
+#include "per_device.h"
 #include "lat_reduce.h"
 #include "step1d_dev.h"
 
@@ -371,14 +372,9 @@ __global__ void k_advance_step(DevState* st, long long n) { st->step += n; }
 
 template <int NV, int NS, bool MOM, bool LIM>
 cudaError_t launch_pc1_t(int grid, const Step1DArgs& a, int kstep, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_step1d_pc<NV, NS, MOM, LIM>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)pc1d_smem<NV, NS>());
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice limit;
+    const cudaError_t e = raise_smem(limit, k_step1d_pc<NV, NS, MOM, LIM>, pc1d_smem<NV, NS>());
+    if (e != cudaSuccess) return e;
     k_step1d_pc<NV, NS, MOM, LIM><<<grid, PC1_THREADS, pc1d_smem<NV, NS>(), s>>>(a, kstep);
     return cudaGetLastError();
 }
@@ -409,14 +405,9 @@ size_t ring1d_smem() {
 
 template <int NV, int NS, bool LIM>
 cudaError_t launch_ring_t(int grid, const Step1DArgs& a, int kstep, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_step1d_ring<NV, NS, LIM>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)ring1d_smem<NV, NS>());
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice limit;
+    const cudaError_t e = raise_smem(limit, k_step1d_ring<NV, NS, LIM>, ring1d_smem<NV, NS>());
+    if (e != cudaSuccess) return e;
     k_step1d_ring<NV, NS, LIM><<<grid, TW1, ring1d_smem<NV, NS>(), s>>>(a, kstep);
     return cudaGetLastError();
 }

@@ -28,6 +28,7 @@
 #include <map>
 
 #include "lat2d.h"
+#include "per_device.h"
 #include "step2d_dev.h"
 #include "step2d_x2.h"
 #include "step2d_h.h"
@@ -1033,14 +1034,9 @@ cudaError_t launch_plain(int grid, const Step2DArgs& a, int k, cudaStream_t s) {
 
 template <int NV, int C>
 cudaError_t launch_ring(int grid, const Step2DArgs& a, int k, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_step2d_ring<NV, C>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)ring_smem<NV, C>());
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice limit;
+    const cudaError_t e = raise_smem(limit, k_step2d_ring<NV, C>, ring_smem<NV, C>());
+    if (e != cudaSuccess) return e;
     k_step2d_ring<NV, C><<<grid, RingShape<NV, C>::threads, ring_smem<NV, C>(), s>>>(a, k);
     return cudaGetLastError();
 }
@@ -1102,15 +1098,10 @@ int occupancy_ring_c(int chunks) {
 template <int NV, int NS, bool GSM, bool HSM = false, bool MOM = false>
 cudaError_t launch_pc(int grid, const Step2DArgs& a, int k, cudaStream_t s,
                       const Mom2DOut& m = Mom2DOut()) {
-    static bool attr = false;
+    static PerDevice limit;
     const size_t bytes = pc_smem<NV, NS, GSM, HSM>();
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_step2d_pc<NV, NS, GSM, HSM, MOM>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)bytes);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    const cudaError_t e = raise_smem(limit, k_step2d_pc<NV, NS, GSM, HSM, MOM>, bytes);
+    if (e != cudaSuccess) return e;
     k_step2d_pc<NV, NS, GSM, HSM, MOM>
         <<<grid, PCShape<NV, NS, GSM, HSM>::threads, bytes, s>>>(a, k, m, nullptr);
     return cudaGetLastError();
@@ -1121,20 +1112,13 @@ cudaError_t launch_pc(int grid, const Step2DArgs& a, int k, cudaStream_t s,
 template <int NV>
 cudaError_t launch_pc_corr_t(int sm_count, const Step2DArgs& a, const float* G, int k,
                              cudaStream_t s) {
-    static int occ = 0;
+    static PerDevice resident;
     const size_t bytes = pc_smem<NV, 4, false, false, 2 * NV * TW>();
-    if (occ == 0) {
-        cudaError_t e = cudaFuncSetAttribute(k_step2d_pc<NV, 4, false, false, false, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)bytes);
-        if (e != cudaSuccess) return e;
-        int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &nb, k_step2d_pc<NV, 4, false, false, false, true>, PCShape<NV, 4, false, false>::threads,
-            bytes);
-        if (e != cudaSuccess) return e;
-        occ = nb > 0 ? nb : 1;
-    }
+    int occ = 0;
+    const cudaError_t e =
+        resident_blocks(resident, k_step2d_pc<NV, 4, false, false, false, true>,
+                        PCShape<NV, 4, false, false>::threads, bytes, &occ);
+    if (e != cudaSuccess) return e;
     const int grid = std::max(1, std::min(a.ntiles, occ * sm_count));
     k_step2d_pc<NV, 4, false, false, false, true>
         <<<grid, PCShape<NV, 4, false, false>::threads, bytes, s>>>(a, k, Mom2DOut(), G);
@@ -1185,15 +1169,10 @@ cudaError_t launch_pc_mom(int v, int bps, int sm_count, const Step2DArgs& a, int
 
 template <int NV, int NS, bool GSM>
 cudaError_t launch_pc2(int grid, const Step2DArgs& a, int k, cudaStream_t s) {
-    static bool attr = false;
+    static PerDevice limit;
     const size_t bytes = pc2_smem<NV, NS, GSM>();
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_step2d_pc2<NV, NS, GSM>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)bytes);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    const cudaError_t e = raise_smem(limit, k_step2d_pc2<NV, NS, GSM>, bytes);
+    if (e != cudaSuccess) return e;
     k_step2d_pc2<NV, NS, GSM><<<grid, PC2Shape<NV, NS, GSM>::threads, bytes, s>>>(a, k);
     return cudaGetLastError();
 }

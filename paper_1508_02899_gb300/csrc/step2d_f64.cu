@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "lat_internal.h"
+#include "per_device.h"
 #include "step2d_dev.h"
 
 namespace lat {
@@ -158,17 +159,11 @@ __global__ void __launch_bounds__(Tile64<NV>::kThreads) k_step2d_tile64(const St
 template <int NV>
 cudaError_t launch_t(int sm_count, const Step2DArgs& a, int k, cudaStream_t s) {
     using L = Tile64<NV>;
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(
-            k_step2d_tile64<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::kSmem);
-        int n = 0;
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step2d_tile64<NV>, L::kThreads,
-                                                              L::kSmem);
-        if (e != cudaSuccess) return e;
-        per_sm = std::max(n, 1);
-    }
+    static PerDevice resident;
+    int per_sm = 0;
+    const cudaError_t e =
+        resident_blocks(resident, k_step2d_tile64<NV>, L::kThreads, L::kSmem, &per_sm);
+    if (e != cudaSuccess) return e;
     const long long ntiles = (long long)((a.nx + L::TC - 1) / L::TC) * a.ny;
     const int grid = (int)std::min<long long>(ntiles, (long long)per_sm * sm_count);
     k_step2d_tile64<NV><<<grid, L::kThreads, L::kSmem, s>>>(a, k);

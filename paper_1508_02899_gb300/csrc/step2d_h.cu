@@ -34,6 +34,7 @@
 
 #include <algorithm>
 
+#include "per_device.h"
 #include "step2d_h.h"
 
 namespace lat {
@@ -628,14 +629,9 @@ int grid_for(long long n, int per_block) {
 template <typename S, int NV, int NS, bool HSM = false>
 cudaError_t launch_pch(int grid, const Step2DHArgs& a, int k, cudaStream_t s) {
     using Lay = PCHLayout<S, NV, NS, HSM>;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_step2d_pch<S, NV, NS, HSM>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)Lay::total);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static PerDevice limit;
+    const cudaError_t e = raise_smem(limit, k_step2d_pch<S, NV, NS, HSM>, Lay::total);
+    if (e != cudaSuccess) return e;
     k_step2d_pch<S, NV, NS, HSM><<<grid, PCHShape<NV, NS>::threads, Lay::total, s>>>(a, k);
     return cudaGetLastError();
 }
