@@ -51,6 +51,17 @@ __device__ __forceinline__ f2 sub2s(f2 a, f2 b) {
 }
 __device__ __forceinline__ f2 max0(f2 v) { return pk(fmaxf(lo(v), 0.f), fmaxf(hi(v), 0.f)); }
 __device__ __forceinline__ f2 min0(f2 v) { return pk(fminf(lo(v), 0.f), fminf(hi(v), 0.f)); }
+// Minimum and maximum that are NaN where an operand is.
+__device__ __forceinline__ float min_nan(float a, float b) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 // max(0, min(a, b, c)) where a > 0, min(0, max(a, b, c)) where a < 0, zero where a = 0, lane by lane:
 // the limited increment of the sign of a, by three-input instructions.
 __device__ __forceinline__ float lim_min(float a, float b, float c) {

@@ -150,7 +150,7 @@ __device__ __forceinline__ void sweep(const float* p, f2 w2, float g, float r, f
     k.one2 = opaque2(pk(1.f, 1.f));
     k.zero2 = opaque2(0ull);
     // rows up to kp have c a >= 0 in every column of the warp, rows from kn on c a <= 0
-    const float wlo = fminf(lo(w2), hi(w2)), whi = fmaxf(lo(w2), hi(w2));
+    const float wlo = min_nan(lo(w2), hi(w2)), whi = max_nan(lo(w2), hi(w2));
     const bool sane = fabsf(wlo) < 1e6f && fabsf(whi) < 1e6f;  // false for NaN
     const int kp = __reduce_min_sync(0xffffffffu, sane ? (int)floorf(wlo) + J : -1);
     const int kn = __reduce_max_sync(0xffffffffu, sane ? (int)ceilf(whi) + J : NV);

@@ -81,7 +81,8 @@ struct Shape {
 //  * MIXED: some columns' places wrap within the chunk (else one pointer serves both columns);
 //  * the sign of c a = g (w - j) over the chunk's rows and the warp's columns.  Where it is one
 //    sign, one term of the upwind flux (c a_j)^+ f_j + (c a_{j+1})^- f_{j+1} is zero: it is not
-//    formed, nor the minima and maxima (5 of 20 instructions per row).
+//    formed, nor the minima and maxima (5 of 20 instructions per row).  A velocity that is not a
+//    number has no sign: the minima and maxima make both its parts zero.
 // A product that an addition uses is formed as an fma with an opaque zero: the packed product
 // itself would be contracted into the addition (other bits).
 enum { kBoth = 0, kPos = 1, kNeg = 2 };
@@ -199,7 +200,7 @@ __device__ __forceinline__ void sweep2(float* f, const float* U, int c0, int d, 
     const int c = c0 + (threadIdx.x & 31), step = S::kPitch + d;
     float *qa = f + c - J * d, *qb = qa + 32;
     float ua = U[c], ub = U[c + 32];
-    float wlo = fminf(ua, ub), whi = fmaxf(ua, ub);
+    float wlo = min_nan(ua, ub), whi = max_nan(ua, ub);
     Wrap wr{NV + 1, NV + 1, 0.f, 0.f};
     int ma = NV + 1, mb = NV + 1;  // rows from which, and up to which, some columns lose P
     if constexpr (RING) {
@@ -227,8 +228,8 @@ __device__ __forceinline__ void sweep2(float* f, const float* U, int c0, int d, 
         ma = __reduce_min_sync(0xffffffffu, min(wr.ea, wr.eb));
         mb = __reduce_max_sync(0xffffffffu, max(wr.ea, wr.eb));
         if (ma <= NV) {
-            wlo = fminf(fminf(wlo, fminf(ua, ub)), fminf(wr.wa, wr.wb));
-            whi = fmaxf(fmaxf(whi, fmaxf(ua, ub)), fmaxf(wr.wa, wr.wb));
+            wlo = min_nan(min_nan(wlo, min_nan(ua, ub)), min_nan(wr.wa, wr.wb));
+            whi = max_nan(max_nan(whi, max_nan(ua, ub)), max_nan(wr.wa, wr.wb));
         }
     }
     // rows up to kp have c a >= 0 in every column of the warp, rows from kn on c a <= 0

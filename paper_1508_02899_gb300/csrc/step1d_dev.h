@@ -29,12 +29,17 @@ struct Ops<double> {
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 };
 
-// max(v, 0) and min(v, 0).  FP64 by the sign bit: comparisons run on the FP64 pipe, which bounds the
-// FP64 kernels on this part (two operations per clock and SM).
+// max(v, 0) and min(v, 0), zero where v is not a number.  FP64 by the upper word: comparisons run on
+// the FP64 pipe, which bounds the FP64 kernels on this part (two operations per clock and SM).  NaNs
+// (of arithmetic: quiet ones) lie above the infinities.
 __device__ __forceinline__ float pos_part(float v) { return fmaxf(v, 0.f); }
 __device__ __forceinline__ float neg_part(float v) { return fminf(v, 0.f); }
-__device__ __forceinline__ double pos_part(double v) { return __double2hiint(v) < 0 ? 0.0 : v; }
-__device__ __forceinline__ double neg_part(double v) { return __double2hiint(v) < 0 ? v : 0.0; }
+__device__ __forceinline__ double pos_part(double v) {
+    return (unsigned)__double2hiint(v) <= 0x7ff00000u ? v : 0.0;
+}
+__device__ __forceinline__ double neg_part(double v) {
+    return __double2hiint(v) <= (int)0xfff00000u ? v : 0.0;
+}
 
 // c a_j = (dt/dv) * (-(v_j - u)/tau_p) = g (w - j), g = dt/tau_p, w = u/dv
 template <typename T>

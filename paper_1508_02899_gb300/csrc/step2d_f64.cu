@@ -38,6 +38,12 @@ struct Tile64 {
 
 __device__ __forceinline__ bool negative(double v) { return __double2hiint(v) < 0; }
 
+// A c a that is not a number (of such a velocity) counts as zero, as in the other kernels' maxima and
+// minima.
+__device__ __forceinline__ double number(double v) {
+    return ((unsigned)__double2hiint(v) & 0x7fffffffu) <= 0x7ff00000u ? v : 0.0;
+}
+
 // Upwind flux between cells l and r of one axis (c_l >= c_r).
 __device__ __forceinline__ double upwind64(double cl, double fl, double cr, double fr) {
     const bool p = !negative(cl);
@@ -100,9 +106,10 @@ __global__ void __launch_bounds__(Tile64<NV>::kThreads) k_step2d_tile64(const St
         double wx, wy;
         load_w<double>(a, x < nx ? x : 0, y, wx, wy);
         if (jx == 0) cfl_check<double, NV>(a, a.g, wx, wy, in);
-        const double c0 = cacc<double>(a.g, wx, jx - J), cl = cacc<double>(a.g, wx, jx - 1 - J),
-                     cr = cacc<double>(a.g, wx, jx + 1 - J);
-        if (active) cy[jx * TC + c] = cacc<double>(a.g, wy, jx - J);
+        const double c0 = number(cacc<double>(a.g, wx, jx - J)),
+                     cl = number(cacc<double>(a.g, wx, jx - 1 - J)),
+                     cr = number(cacc<double>(a.g, wx, jx + 1 - J));
+        if (active) cy[jx * TC + c] = number(cacc<double>(a.g, wy, jx - J));
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();  // f* and c a_y are there; every warp is done with the last tile's f**
         if (in) {
