@@ -26,7 +26,7 @@ __global__ void k_clear_status(DevState* st) { st->status = 0u; }
 
 // Tiles of columns of an on-chip kernel (none where not built) and their widest places.
 struct TileSet {
-    lat::MultiTile* d = nullptr;
+    const lat::MultiTile* d = nullptr;
     int n = 0, places = 0;
 };
 
@@ -83,12 +83,21 @@ struct lat_ctx {
     bool stalled = false;  // lat_debug_stall
     bool pinned = false;  // a kernel chosen by lat_set_launch: one step per launch
 
+    // Batches of steps (build_plan): what depends on the grids alone, in one block of device memory,
+    // and the rows of u / dv that the flow kernel fills.
+    void* d_plan = nullptr;
     TileSet tiles[2];  // several upwind steps per launch (multi1d.cu); the limited step (lim1d.cu)
-    bool line_ok = false;         // small enough for the cluster kernel (line1d.cu)
-    bool wflow_ok = false;        // the flow kernel's tables and buffer exist
-    void* d_basis = nullptr;      // flow-basis tables, their offsets per instance, and u / dv of a
-    long long* d_basis_off = nullptr;  // launch's steps (multi1d.cu)
+    long long* d_size_off = nullptr;  // [n_inst] columns of the grid sizes before the instance's
+    int* d_sizes = nullptr;           // an instance of every grid size
+    int n_sizes = 0;
+    long long size_cols = 0;          // columns of all grid sizes
     void* d_wflow = nullptr;
+    // Tables of the modes' sines and cosines, one per grid size, for the wavenumbers of basis_k.
+    void* d_basis = nullptr;
+    size_t basis_cap = 0;             // bytes
+    std::vector<int> basis_k;
+    // per number of modes, whether the cluster kernel takes the lattice: 0 not asked, 1 no, 2 yes
+    signed char line_fit[kMaxModes1D + 1] = {};
 
     // cached graphs keyed by the number of steps (buffers are picked by the device step parity)
     std::map<int, cudaGraphExec_t> graphs;
@@ -201,7 +210,7 @@ Step1DArgs step_args(const lat_ctx* c, int k, int dry) {
     a.noise = c->d_noise;
     a.field = c->field;
     a.basis = c->d_basis;
-    a.basis_off = c->d_basis_off;
+    a.size_off = c->d_size_off;
     a.wflow = c->d_wflow;
     a.total_x = c->total_x;
     a.nv = c->nv;
@@ -217,9 +226,7 @@ Step1DArgs step_args(const lat_ctx* c, int k, int dry) {
 constexpr int kMultiT = 5;  // steps per launch of the several-steps kernel
 static_assert(kMultiT <= kFlowSteps, "their flow is formed in one launch");
 
-// Tiles of the several-steps kernel, the flow-basis tables and the flow buffer it reads (beyond
-// kBasisBytes of tables, steps are launched one by one).  Called whenever the flow changes.
-constexpr size_t kBasisBytes = 64u << 20;
+constexpr size_t kBasisBytes = 64u << 20;  // tables of the modes at most: see flow_rows
 constexpr long long kLimRestCells = 8 << 20;  // see enqueue_steps_1d
 constexpr int kMinTile = 64;  // narrower tiles are mostly margin
 
@@ -244,11 +251,12 @@ int tile_cut(int nx, int w, int wmax) {
 // (0.7 + k), P the places of a tile (the parts are of its sweep and of its latencies); the widest of
 // equals.  Upwind, N_v = 33, 64 instances of 200 to 1500 columns, 50 steps: two tiles per SM 268 us,
 // one 303 us, one step per launch 435 us.
-int build_tiles(lat_ctx* c, bool lim) {
-    TileSet& t = c->tiles[lim];
+std::vector<MultiTile> make_tiles(const lat_ctx* c, bool lim, int* widest_places) {
     int places = 0, margin = 0;
-    if (!(lim ? lim1d_shape(c->nv, &places) : multi1d_shape(c->nv, kMultiT, &places, &margin)))
-        return LAT_OK;
+    std::vector<MultiTile> tiles;
+    if (c->dtype != LAT_F32 ||
+        !(lim ? lim1d_shape(c->nv, &places) : multi1d_shape(c->nv, kMultiT, &places, &margin)))
+        return tiles;
     const int wmax = (places - 2 * margin) / 8 * 8;
     const int held = lim ? 3 : 2;
     std::map<int, int> sizes;  // N_x -> instances
@@ -275,71 +283,108 @@ int build_tiles(lat_ctx* c, bool lim) {
             wtile = w;
         }
     }
-    std::vector<MultiTile> tiles;
+    *widest_places = 0;
     for (int i = 0; i < c->n_inst; ++i) {
         const Inst1D& in = c->h_inst[i];
         const int w = tile_cut(in.nx, wtile, wmax);
         for (int x0 = 0; x0 < in.nx; x0 += w) {
             const int cols = std::min(w, in.nx - x0);
             tiles.push_back({in.off, in.xoff, in.nx, x0, cols, (float)in.g, (float)in.r});
-            t.places = std::max(t.places, tile_places(c, lim, cols));
+            *widest_places = std::max(*widest_places, tile_places(c, lim, cols));
         }
     }
-    if (cudaMalloc(&t.d, sizeof(MultiTile) * tiles.size()) != cudaSuccess) {
+    return tiles;
+}
+
+// Whether the cluster kernel takes the lattice, asked once per number of modes.
+void fit_line(lat_ctx* c) {
+    signed char& fit = c->line_fit[c->nmodes];
+    if (!fit) fit = line1d_fits(c->dtype, c->n_inst, max_nx(c), c->nv, c->nmodes) ? 2 : 1;
+}
+
+// What batches of steps need of the grids: the tiles of the two on-chip kernels, the distinct grid
+// sizes, and the rows of the flow.  Once per context; without room for it steps are launched one by
+// one, with the flow inside.
+int build_plan(lat_ctx* c) {
+    fit_line(c);
+    std::vector<MultiTile> tiles[2];
+    for (int q = 0; q < 2; ++q) tiles[q] = make_tiles(c, q == 1, &c->tiles[q].places);
+    std::map<int, long long> at;  // N_x -> columns before it
+    std::vector<long long> off(c->n_inst);
+    std::vector<int> sizes;
+    for (int i = 0; i < c->n_inst; ++i) {
+        const int nx = c->h_inst[i].nx;
+        const auto e = at.emplace(nx, c->size_cols);
+        if (e.second) {
+            sizes.push_back(i);
+            c->size_cols += nx;
+        }
+        off[i] = e.first->second;
+    }
+    const size_t bt0 = sizeof(MultiTile) * tiles[0].size(), bt1 = sizeof(MultiTile) * tiles[1].size(),
+                 bo = sizeof(long long) * off.size(), bs = sizeof(int) * sizes.size();
+    const size_t elem = c->dtype == LAT_F64 ? sizeof(double) : sizeof(float);
+    if (cudaMalloc(&c->d_plan, bt0 + bt1 + bo + bs) != cudaSuccess ||
+        cudaMalloc(&c->d_wflow, elem * kFlowSteps * c->total_x) != cudaSuccess) {
         cudaGetLastError();
+        c->d_wflow = nullptr;
         return LAT_OK;
     }
-    CK(upload(t.d, tiles.data(), sizeof(MultiTile) * tiles.size(), c->stream));
-    t.n = (int)tiles.size();
+    static_assert(sizeof(MultiTile) % sizeof(long long) == 0, "what follows the tiles is aligned");
+    std::vector<char> image(bt0 + bt1 + bo + bs);
+    char* const dev = static_cast<char*>(c->d_plan);
+    size_t p = 0;
+    auto put = [&](const void* src, size_t bytes) {
+        if (bytes) memcpy(image.data() + p, src, bytes);
+        p += bytes;
+        return dev + p - bytes;
+    };
+    for (int q = 0; q < 2; ++q) {
+        c->tiles[q].n = (int)tiles[q].size();
+        c->tiles[q].d = reinterpret_cast<const MultiTile*>(
+            put(tiles[q].data(), sizeof(MultiTile) * tiles[q].size()));
+    }
+    c->d_size_off = reinterpret_cast<long long*>(put(off.data(), bo));
+    c->d_sizes = reinterpret_cast<int*>(put(sizes.data(), bs));
+    c->n_sizes = (int)sizes.size();
+    CK(upload(c->d_plan, image.data(), image.size(), c->stream));
     return LAT_OK;
 }
 
-int build_multi(lat_ctx* c) {
-    c->line_ok = line1d_fits(c->dtype, c->n_inst, max_nx(c), c->nv, c->nmodes);
-    for (TileSet& t : c->tiles) {
-        cudaFree(t.d);
-        t = TileSet{};
+// The tables of the modes for the flow kernel, where they are not those of the present wavenumbers
+// (beyond kBasisBytes, or without room, there are none).  Fields and no flow need none.
+int build_basis(lat_ctx* c) {
+    const std::vector<int> k(c->k1d, c->k1d + c->nmodes);
+    if (c->flow_kind != LAT_FLOW_MODES || !c->d_wflow || k == c->basis_k) return LAT_OK;
+    const size_t need = 2 * (c->dtype == LAT_F64 ? sizeof(double) : sizeof(float)) * c->size_cols *
+                        (size_t)c->nmodes;
+    c->basis_k.clear();
+    if (need > kBasisBytes) return LAT_OK;
+    if (need > c->basis_cap) {
+        cudaFree(c->d_basis);
+        c->basis_cap = 0;
+        if (cudaMalloc(&c->d_basis, need) != cudaSuccess) {
+            cudaGetLastError();
+            c->d_basis = nullptr;
+            return LAT_OK;
+        }
+        c->basis_cap = need;
     }
-    cudaFree(c->d_basis);
-    cudaFree(c->d_basis_off);
-    c->d_basis = nullptr;
-    c->d_basis_off = nullptr;
-    c->wflow_ok = false;
-    const size_t elem = c->dtype == LAT_F64 ? sizeof(double) : sizeof(float);
-    std::map<int, std::pair<int, long long>> sizes;  // N_x -> (an instance, table offset)
-    std::vector<long long> off(c->n_inst);
-    long long total = 0;
-    for (int i = 0; i < c->n_inst; ++i) {
-        const int nx = c->h_inst[i].nx;
-        const auto at = sizes.emplace(nx, std::make_pair(i, total));
-        if (at.second) total += (long long)nx * c->nmodes;
-        off[i] = at.first->second.second;
-    }
-    if (2 * elem * (size_t)total > kBasisBytes) return LAT_OK;
-    if (cudaMalloc(&c->d_basis_off, sizeof(long long) * c->n_inst) != cudaSuccess ||
-        (total > 0 && cudaMalloc(&c->d_basis, 2 * elem * total) != cudaSuccess) ||
-        (!c->d_wflow &&
-         cudaMalloc(&c->d_wflow, elem * kFlowSteps * c->total_x) != cudaSuccess)) {
-        cudaGetLastError();  // no room for them: steps are launched one by one
-        return LAT_OK;
-    }
-    CK(upload(c->d_basis_off, off.data(), sizeof(long long) * c->n_inst, c->stream));
-    if (total > 0) {
-        const Step1DArgs a = step_args(c, 0, 0);
-        for (const auto& e : sizes)
-            CK(launch_flow_basis(c->dtype, a, e.second.first, e.first, c->d_basis, e.second.second,
-                                 c->stream));
-    }
-    c->wflow_ok = true;
-    if (c->dtype != LAT_F32) return LAT_OK;
-    int rc = build_tiles(c, false);
-    return rc != LAT_OK ? rc : build_tiles(c, true);
+    CK(launch_flow_basis(c->dtype, step_args(c, 0, 0), c->d_sizes, c->n_sizes, max_nx(c), c->d_basis,
+                         c->stream));
+    c->basis_k = k;
+    return LAT_OK;
+}
+
+// Whether the flow kernel can form the rows of u / dv.
+bool flow_rows(const lat_ctx* c) {
+    return c->d_wflow && (c->flow_kind != LAT_FLOW_MODES || !c->basis_k.empty());
 }
 
 // Whether batches of steps run on the cluster kernel of small lattices.
 bool line_1d(const lat_ctx* c) {
     return c->d == 1 && !c->pinned && c->mode != 1 && c->scheme == LAT_SCHEME_UPWIND &&
-           c->line_ok && !c->stalled;
+           c->line_fit[c->nmodes] == 2 && !c->stalled;
 }
 
 // Enqueue n steps of a 1D context on stream s (used directly and under capture).  Where no launch
@@ -353,15 +398,16 @@ int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
         if (c->n_inst > 1) CK(launch_advance_step(c->d_state, n, s));
         return LAT_OK;
     }
-    const bool multi = on_chip && c->tiles[0].n;
-    const bool lim = !chosen && c->scheme == LAT_SCHEME_KOREN && c->tiles[1].n;
+    const bool rows = flow_rows(c);
+    const bool multi = on_chip && rows && c->tiles[0].n;
+    const bool lim = !chosen && rows && c->scheme == LAT_SCHEME_KOREN && c->tiles[1].n;
     // The plain-load and the limited kernels take the flow from the flow kernel, kFlowSteps steps at
     // a time (evaluating the basis costs an FP64 column as much as half its sweep).  The launch is
     // not worth it for fewer FP32 steps (1000 instances of 601 columns, N_v = 33, one upwind step:
     // 52 us, with the launch 58 us) unless the limited step is long (1200 instances of 1024 columns,
     // one step: N_v = 65 175 us, one column per thread 303 us; N_v = 17 89 and 82 us; 48 instances of
     // 4096 columns, N_v = 33: 28 and 25 us).
-    const bool pre = lim || (!chosen && c->variant == STEP1D_PLAIN && c->wflow_ok &&
+    const bool pre = lim || (!chosen && c->variant == STEP1D_PLAIN && rows &&
                              c->flow_kind == LAT_FLOW_MODES);
     const bool rest = c->dtype == LAT_F64 ||
                       (lim && c->nv >= 33 && c->total_x * c->nv >= kLimRestCells);
@@ -523,7 +569,7 @@ int lat_ensemble_init(lat_ctx** out, int n_inst, const lat_instance* inst, int n
             }
         }
         rc = build_items(c);
-        if (rc == LAT_OK) rc = build_multi(c);
+        if (rc == LAT_OK) rc = build_plan(c);
     }
     if (rc != LAT_OK) {
         lat_free(c);
@@ -630,7 +676,8 @@ int lat_set_flow(lat_ctx* c, const lat_flow* fl) {
     k_set_noise_window<<<1, 1, 0, c->stream>>>(c->d_state, c->h_step, 0);
     CK(cudaGetLastError());
     drop_graphs(c);
-    return build_multi(c);
+    fit_line(c);
+    return build_basis(c);
 }
 
 int lat_set_noise(lat_ctx* c, const double* noise, long long rows) {
@@ -1432,9 +1479,8 @@ void lat_free(lat_ctx* c) {
     cudaFree(c->d_items);
     cudaFree(c->d_inst_begin);
     cudaFree(c->d_partials);
-    for (TileSet& t : c->tiles) cudaFree(t.d);
+    cudaFree(c->d_plan);
     cudaFree(c->d_basis);
-    cudaFree(c->d_basis_off);
     cudaFree(c->d_wflow);
     cudaFree(c->d_glob);
     cudaFree(c->d_amp);

@@ -85,7 +85,7 @@ struct Step1DArgs {
     const void* field;       // FIELD flow, per-cell array over all instances
     // several steps per launch (multi1d.cu)
     const void* basis;           // (sin, cos) tables of the modes, one per grid size
-    const long long* basis_off;  // [n_inst] offset of the instance's table
+    const long long* size_off;   // [n_inst] columns of the tables before the instance's
     void* wflow;                 // [T][total_x] u / dv of the steps
     const void* wpre;            // u / dv of this step's columns (a row of wflow), or null
     long long total_x;
@@ -126,10 +126,10 @@ cudaError_t launch_lim1d(int nv, int ntiles, int places, const Step1DArgs& a, co
 bool line1d_fits(int dtype, int n_inst, int nx_max, int nv, int nmodes);
 cudaError_t launch_line1d(int dtype, int n_inst, int nx_max, int nv, const Step1DArgs& a, int kstep,
                           int n, cudaStream_t s);
-// Table of the flow's basis for instance inst's grid size, at entry `at` of the table:
-// (sin, cos) of 2 pi k_m x / N_x, [m][x].
-cudaError_t launch_flow_basis(int dtype, const Step1DArgs& a, int inst, int nx, void* table,
-                              long long at, cudaStream_t s);
+// Tables of the flow's basis, one per grid size (sizes: an instance of each; nx_max the largest):
+// (sin, cos) of 2 pi k_m x / N_x, [m][x], from entry M size_off on.
+cudaError_t launch_flow_basis(int dtype, const Step1DArgs& a, const int* sizes, int n_sizes,
+                              int nx_max, void* table, cudaStream_t s);
 // u / dv of steps kstep .. kstep + T - 1 into wflow (T <= kFlowSteps, odd: the amplitudes move to the
 // step after them, in the parity that no block reads).  One block per item.
 constexpr int kFlowSteps = 5;

@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kste
     const F cf = a.scheme == LAT_SCHEME_KOREN ? F(1) + F(a.mu) : F(1);  // Eq. (cfl) of the scheme
     bool cfl = false;
     for (int x = item.y + tid; x < min(nx, item.y + a.tile); x += blockDim.x) {
-        const F2* basis = static_cast<const F2*>(a.basis) + a.basis_off[item.x] + x;
+        const F2* basis = static_cast<const F2*>(a.basis) + M * a.size_off[item.x] + x;
         F* w = static_cast<F*>(a.wflow) + in.xoff + x;
 #pragma unroll 1
         for (int s0 = 0; s0 < T; s0 += kFlowGroup) {

@@ -356,15 +356,18 @@ __global__ void __launch_bounds__(PC1_THREADS) k_step1d_pc(const Step1DArgs a, c
     }
 }
 
-// The flow's basis of one grid size: sin and cos of 2 pi k_m x / N_x, [m][x].
+// The flow's basis of every grid size: sin and cos of 2 pi k_m x / N_x, [m][x].
 template <typename T, typename T2>
-__global__ void k_flow_basis(const Step1DArgs a, int inst, T2* out) {
-    const Inst1D in = a.inst[inst];
-    const T two_over_nx = T(in.two_over_nx);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.nmodes * in.nx;
-         i += gridDim.x * blockDim.x) {
-        const int m = i / in.nx;
-        flow_basis<T>(a.k[m], in, two_over_nx, i - m * in.nx, &out[i].x, &out[i].y);
+__global__ void k_flow_basis(const Step1DArgs a, const int* sizes, int n_sizes, T2* table) {
+    for (int q = blockIdx.y; q < n_sizes; q += gridDim.y) {
+        const Inst1D in = a.inst[sizes[q]];
+        const T two_over_nx = T(in.two_over_nx);
+        T2* out = table + a.nmodes * a.size_off[sizes[q]];
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.nmodes * in.nx;
+             i += gridDim.x * blockDim.x) {
+            const int m = i / in.nx;
+            flow_basis<T>(a.k[m], in, two_over_nx, i - m * in.nx, &out[i].x, &out[i].y);
+        }
     }
 }
 
@@ -560,12 +563,13 @@ cudaError_t launch_step1d(int dtype, int nv, int variant, int block, int slots, 
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_flow_basis(int dtype, const Step1DArgs& a, int inst, int nx, void* table,
-                              long long at, cudaStream_t s) {
-    const int grid = (a.nmodes * nx + 255) / 256;
+cudaError_t launch_flow_basis(int dtype, const Step1DArgs& a, const int* sizes, int n_sizes,
+                              int nx_max, void* table, cudaStream_t s) {
+    const dim3 grid((a.nmodes * nx_max + 255) / 256, std::min(n_sizes, 65535));
     if (dtype == LAT_F64)
-        k_flow_basis<double><<<grid, 256, 0, s>>>(a, inst, static_cast<double2*>(table) + at);
-    else k_flow_basis<float><<<grid, 256, 0, s>>>(a, inst, static_cast<float2*>(table) + at);
+        k_flow_basis<double><<<grid, 256, 0, s>>>(a, sizes, n_sizes, static_cast<double2*>(table));
+    else
+        k_flow_basis<float><<<grid, 256, 0, s>>>(a, sizes, n_sizes, static_cast<float2*>(table));
     return cudaGetLastError();
 }
 
