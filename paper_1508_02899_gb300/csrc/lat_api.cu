@@ -991,7 +991,7 @@ int lat_s1(lat_ctx* c, int ns, const int* seps, double* num, double* den) {
         if (seps[q] < 0 || seps[q] >= nmin) return LAT_EINVAL;
     const int nout = c->n_inst * ns;
     int rc = obs_scratch(c, (size_t)c->total_x + 2 * (size_t)nout + (ns + 1) / 2 +
-                                s1_scratch(c->n_inst, max_nx(c), c->total_x, c->sm_count));
+                                s1_scratch(c->n_inst, c->total_x, c->sm_count));
     if (rc != LAT_OK) return rc;
     double* rho = c->d_obs;
     double* d_num = rho + c->total_x;
@@ -1001,8 +1001,8 @@ int lat_s1(lat_ctx* c, int ns, const int* seps, double* num, double* den) {
     rc = lat_moments(c, rho, nullptr, nullptr, nullptr);
     if (rc != LAT_OK) return rc;
     CK(cudaMemcpyAsync(d_s, seps, sizeof(int) * ns, cudaMemcpyHostToDevice, c->stream));
-    CK(launch_s1_1d(c->dtype, c->f[c->cur], c->d_inst, c->n_inst, max_nx(c), c->total_x, c->nv, rho,
-                    d_s, ns, d_part, d_num, d_den, c->sm_count, c->stream));
+    CK(launch_s1_1d(c->dtype, c->f[c->cur], c->d_inst, c->n_inst, c->total_x, c->nv, rho, d_s,
+                    ns, d_part, d_num, d_den, c->sm_count, c->stream));
     CK(cudaMemcpyAsync(num, d_num, sizeof(double) * nout, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(den, d_den, sizeof(double) * nout, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));

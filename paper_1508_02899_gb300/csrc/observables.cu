@@ -199,18 +199,24 @@ __global__ void __launch_bounds__(kObsThreads)
 // then times dv^3; the denominator rho_i rho_{i+s}.  T = float for FP32 states (errors about
 // N_v u of the positive sums), double for FP64 states.
 //
-// A block takes a run of columns of one instance, a thread cpt cells of it, and kS1Group separations
-// in one pair of sweeps: a_j is loaded for all of them, and what remains per separation and velocity
-// cell is one load and three operations in either direction (1024 instances, N_v = 65, eight
-// separations: 2.4 ms; a block per instance and separation 6.5 ms).  The cells' sums are FP64 Neumaier
-// sums per thread; the 2 kS1Group sums of a warp's lanes are folded by halving (every lane ends with
-// one of them) rather than by as many butterflies, which took longer than the sweeps.  The blocks'
-// sums go to part[instance][chunk][num, den of each][sum, compensation], folded in order.
+// A block takes a run of columns of one instance (a slot: see s1_slot), a thread cpt cells of it, and
+// kS1Group separations in one pair of sweeps: a_j is loaded for all of them, and what remains per
+// separation and velocity cell is one load and three operations in either direction (1024 instances,
+// N_v = 65, eight separations: 2.4 ms; a block per instance and separation 6.5 ms).  The cells' sums
+// are FP64 Neumaier sums per thread; the 2 kS1Group sums of a warp's lanes are folded by halving (every
+// lane ends with one of them) rather than by as many butterflies, which took longer than the sweeps.
+// The blocks' sums go to part[slot][num, den of each][sum, compensation], folded in slot order.
 constexpr int kS1Group = 8;
 constexpr int kS1Threads = 128;
 
 __device__ __forceinline__ Comp shfl_xor(const Comp& a, int m) {
     return Comp{__shfl_xor_sync(0xffffffffu, a.s, m), __shfl_xor_sync(0xffffffffu, a.c, m)};
+}
+
+// First slot of instance k: its runs of `per` columns take the slots from here on, at most
+// floor((xoff + N_x) / per) - floor(xoff / per) + 1 of them, so instances do not share any.
+__host__ __device__ __forceinline__ long long s1_slot(const Inst1D& in, int k, int per) {
+    return in.xoff / per + k;
 }
 
 template <typename T>
@@ -220,96 +226,101 @@ __global__ void __launch_bounds__(kS1Threads)
     constexpr int NS = 2 * kS1Group;  // sums: 2 q the numerator, 2 q + 1 the denominator
     __shared__ Comp wsum[kS1Threads / 32][NS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = blockIdx.y; k < n_inst; k += gridDim.y) {
-        const Inst1D& in = inst[k];
-        const int n = in.nx, x0 = blockIdx.x * kS1Threads * cpt;
-        if (x0 >= n) continue;
-        const T* fk = f + in.off;
-        Comp t[NS];
+    const int per = kS1Threads * cpt;
+    int k = 0;  // the last instance whose first slot is not beyond this one
+    for (int hi = n_inst; hi - k > 1;) {
+        const int mid = (k + hi) / 2;
+        if (s1_slot(inst[mid], mid, per) <= (long long)blockIdx.x) k = mid;
+        else hi = mid;
+    }
+    const Inst1D& in = inst[k];
+    const int n = in.nx;
+    const long long first = ((long long)blockIdx.x - s1_slot(in, k, per)) * per;
+    if (first >= n) return;  // a slot without columns
+    const int x0 = (int)first;
+    const T* fk = f + in.off;
+    Comp t[NS];
 #pragma unroll
-        for (int q = 0; q < NS; ++q) t[q] = Comp{0, 0};
-        for (int e = 0; e < cpt; ++e) {
-            const int i = x0 + e * kS1Threads + threadIdx.x;
-            if (i >= n) break;
-            int i2[kS1Group];
-            T acc[kS1Group], B[kS1Group], run[kS1Group];
+    for (int q = 0; q < NS; ++q) t[q] = Comp{0, 0};
+    for (int e = 0; e < cpt; ++e) {
+        const int i = x0 + e * kS1Threads + threadIdx.x;
+        if (i >= n) break;
+        int i2[kS1Group];
+        T acc[kS1Group], B[kS1Group], run[kS1Group];
+#pragma unroll
+        for (int q = 0; q < kS1Group; ++q) {
+            const int s = q < nq ? seps[q0 + q] : 0;
+            i2[q] = i + s < n ? i + s : i + s - n;
+            acc[q] = B[q] = run[q] = T(0);
+        }
+        const T* row = fk;
+#pragma unroll 2
+        for (int j = 0; j < nv; ++j) {
+            const T a = row[i];
 #pragma unroll
             for (int q = 0; q < kS1Group; ++q) {
-                const int s = q < nq ? seps[q0 + q] : 0;
-                i2[q] = i + s < n ? i + s : i + s - n;
-                acc[q] = B[q] = run[q] = T(0);
+                acc[q] += a * run[q];
+                B[q] += row[i2[q]];
+                run[q] += B[q];
             }
-            const T* row = fk;
+            row += n;
+        }
+#pragma unroll
+        for (int q = 0; q < kS1Group; ++q) B[q] = run[q] = T(0);
 #pragma unroll 2
-            for (int j = 0; j < nv; ++j) {
-                const T a = row[i];
-#pragma unroll
-                for (int q = 0; q < kS1Group; ++q) {
-                    acc[q] += a * run[q];
-                    B[q] += row[i2[q]];
-                    run[q] += B[q];
-                }
-                row += n;
-            }
-#pragma unroll
-            for (int q = 0; q < kS1Group; ++q) B[q] = run[q] = T(0);
-#pragma unroll 2
-            for (int j = nv - 1; j >= 0; --j) {
-                row -= n;
-                const T a = row[i];
-#pragma unroll
-                for (int q = 0; q < kS1Group; ++q) {
-                    acc[q] += a * run[q];
-                    B[q] += row[i2[q]];
-                    run[q] += B[q];
-                }
-            }
-            const double* rk = rho + in.xoff;
-            const double ri = rk[i];
+        for (int j = nv - 1; j >= 0; --j) {
+            row -= n;
+            const T a = row[i];
 #pragma unroll
             for (int q = 0; q < kS1Group; ++q) {
-                nadd(t[2 * q], (double)acc[q]);
-                nadd(t[2 * q + 1], ri * rk[i2[q]]);
+                acc[q] += a * run[q];
+                B[q] += row[i2[q]];
+                run[q] += B[q];
             }
         }
-        // halve the sums a lane holds, level by level: after it lane l holds sum l / 2 over the
-        // lanes of its parity, then over all
+        const double* rk = rho + in.xoff;
+        const double ri = rk[i];
 #pragma unroll
-        for (int h = NS / 2, m = 16; h >= 1; h >>= 1, m >>= 1) {
-            const bool up = (lane & m) != 0;
+        for (int q = 0; q < kS1Group; ++q) {
+            nadd(t[2 * q], (double)acc[q]);
+            nadd(t[2 * q + 1], ri * rk[i2[q]]);
+        }
+    }
+    // halve the sums a lane holds, level by level: after it lane l holds sum l / 2 over the
+    // lanes of its parity, then over all
 #pragma unroll
-            for (int q = 0; q < h; ++q) {
-                const Comp keep = up ? t[q + h] : t[q], give = up ? t[q] : t[q + h];
-                t[q] = keep;
-                nmerge(t[q], shfl_xor(give, m));
-            }
+    for (int h = NS / 2, m = 16; h >= 1; h >>= 1, m >>= 1) {
+        const bool up = (lane & m) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const Comp keep = up ? t[q + h] : t[q], give = up ? t[q] : t[q + h];
+            t[q] = keep;
+            nmerge(t[q], shfl_xor(give, m));
         }
-        nmerge(t[0], shfl_xor(t[0], 1));
-        if ((lane & 1) == 0) wsum[warp][lane / 2] = t[0];
-        __syncthreads();
-        if (threadIdx.x < NS) {
-            Comp z{0, 0};
-            for (int w = 0; w < kS1Threads / 32; ++w) nmerge(z, wsum[w][threadIdx.x]);
-            double* p = part + (((size_t)k * gridDim.x + blockIdx.x) * NS + threadIdx.x) * 2;
-            p[0] = z.s;
-            p[1] = z.c;
-        }
-        __syncthreads();
+    }
+    nmerge(t[0], shfl_xor(t[0], 1));
+    if ((lane & 1) == 0) wsum[warp][lane / 2] = t[0];
+    __syncthreads();
+    if (threadIdx.x < NS) {
+        Comp z{0, 0};
+        for (int w = 0; w < kS1Threads / 32; ++w) nmerge(z, wsum[w][threadIdx.x]);
+        double* p = part + ((size_t)blockIdx.x * NS + threadIdx.x) * 2;
+        p[0] = z.s;
+        p[1] = z.c;
     }
 }
 
 // One half-warp per instance folds its chunks' sums in order.
-__global__ void k_s1_fold(const double* part, int nchunk, int cpt, const Inst1D* inst, int n_inst,
+__global__ void k_s1_fold(const double* part, int cpt, const Inst1D* inst, int n_inst,
                           int q0, int nq, int ns, double* num, double* den) {
     constexpr int NS = 2 * kS1Group;
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) / NS, q = threadIdx.x % NS;
     if (k >= n_inst || q >= 2 * nq) return;
     const Inst1D& in = inst[k];
     Comp z{0, 0};
-    for (int c = 0; c * kS1Threads * cpt < in.nx; ++c) {
-        const double* p = part + (((size_t)k * nchunk + c) * NS + q) * 2;
-        nmerge(z, Comp{p[0], p[1]});
-    }
+    const int per = kS1Threads * cpt;
+    const double* p = part + (s1_slot(in, k, per) * NS + q) * 2;
+    for (long long x0 = 0; x0 < in.nx; x0 += per, p += 2 * NS) nmerge(z, Comp{p[0], p[1]});
     const size_t o = (size_t)k * ns + q0 + q / 2;
     if (q % 2 == 0) num[o] = nval(z) * in.dv * in.dv * in.dv / in.nx;
     else den[o] = nval(z) / in.nx;
@@ -355,17 +366,22 @@ cudaError_t launch_coarse2d(const double* rho, int nx, int ny, double dx, const 
     return cudaGetLastError();
 }
 
-size_t s1_scratch(int n_inst, int nx_max, long long total_x, int sm_count) {
-    const int per = kS1Threads * s1_cells(total_x, sm_count);
-    return (size_t)n_inst * ((nx_max + per - 1) / per) * 4 * kS1Group;
+namespace {
+long long s1_slots(int n_inst, long long total_x, int sm_count) {
+    return total_x / (kS1Threads * s1_cells(total_x, sm_count)) + n_inst;
+}
+}  // namespace
+
+size_t s1_scratch(int n_inst, long long total_x, int sm_count) {
+    return (size_t)s1_slots(n_inst, total_x, sm_count) * 4 * kS1Group;
 }
 
-cudaError_t launch_s1_1d(int dtype, const void* f, const Inst1D* inst, int n_inst, int nx_max,
+cudaError_t launch_s1_1d(int dtype, const void* f, const Inst1D* inst, int n_inst,
                          long long total_x, int nv, const double* rho, const int* seps, int ns,
                          double* part, double* num, double* den, int sm_count, cudaStream_t s) {
     if (dtype != LAT_F32 && dtype != LAT_F64) return cudaErrorInvalidValue;
-    const int cpt = s1_cells(total_x, sm_count), per = kS1Threads * cpt;
-    const dim3 grid((nx_max + per - 1) / per, std::min(n_inst, 65535));
+    const int cpt = s1_cells(total_x, sm_count);
+    const unsigned grid = (unsigned)s1_slots(n_inst, total_x, sm_count);
     for (int q0 = 0; q0 < ns; q0 += kS1Group) {
         const int nq = std::min(kS1Group, ns - q0);
         if (dtype == LAT_F32)
@@ -374,7 +390,7 @@ cudaError_t launch_s1_1d(int dtype, const void* f, const Inst1D* inst, int n_ins
         else
             k_s1_1d<double><<<grid, kS1Threads, 0, s>>>(static_cast<const double*>(f), inst, n_inst,
                                                         cpt, nv, rho, seps, q0, nq, part);
-        k_s1_fold<<<(n_inst + 7) / 8, 16 * kS1Group, 0, s>>>(part, grid.x, cpt, inst, n_inst, q0, nq,
+        k_s1_fold<<<(n_inst + 7) / 8, 16 * kS1Group, 0, s>>>(part, cpt, inst, n_inst, q0, nq,
                                                              ns, num, den);
     }
     return cudaGetLastError();
