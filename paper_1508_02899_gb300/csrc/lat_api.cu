@@ -991,7 +991,7 @@ int lat_s1(lat_ctx* c, int ns, const int* seps, double* num, double* den) {
         if (seps[q] < 0 || seps[q] >= nmin) return LAT_EINVAL;
     const int nout = c->n_inst * ns;
     int rc = obs_scratch(c, (size_t)c->total_x + 2 * (size_t)nout + (ns + 1) / 2 +
-                                s1_scratch(c->n_inst, c->total_x, c->sm_count));
+                                s1_scratch(c->n_inst, c->total_x, ns, c->sm_count));
     if (rc != LAT_OK) return rc;
     double* rho = c->d_obs;
     double* d_num = rho + c->total_x;

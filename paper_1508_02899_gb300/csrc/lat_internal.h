@@ -177,7 +177,7 @@ cudaError_t launch_coarse1d(const double* rho, const Inst1D* inst, int n_inst, l
 cudaError_t launch_coarse2d(const double* rho, int nx, int ny, double dx, const int* widths,
                             int nw, double* S, double* out, int sm_count, cudaStream_t s);
 // part: s1_scratch() doubles.
-size_t s1_scratch(int n_inst, long long total_x, int sm_count);
+size_t s1_scratch(int n_inst, long long total_x, int ns, int sm_count);
 cudaError_t launch_s1_1d(int dtype, const void* f, const Inst1D* inst, int n_inst,
                          long long total_x, int nv, const double* rho, const int* seps, int ns,
                          double* part, double* num, double* den, int sm_count, cudaStream_t s);

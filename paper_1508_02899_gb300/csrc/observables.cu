@@ -199,14 +199,14 @@ __global__ void __launch_bounds__(kObsThreads)
 // then times dv^3; the denominator rho_i rho_{i+s}.  T = float for FP32 states (errors about
 // N_v u of the positive sums), double for FP64 states.
 //
-// A block takes a run of columns of one instance (a slot: see s1_slot), a thread cpt cells of it, and
-// kS1Group separations in one pair of sweeps: a_j is loaded for all of them, and what remains per
-// separation and velocity cell is one load and three operations in either direction (1024 instances,
-// N_v = 65, eight separations: 2.4 ms; a block per instance and separation 6.5 ms).  The cells' sums
-// are FP64 Neumaier sums per thread; the 2 kS1Group sums of a warp's lanes are folded by halving (every
-// lane ends with one of them) rather than by as many butterflies, which took longer than the sweeps.
-// The blocks' sums go to part[slot][num, den of each][sum, compensation], folded in slot order.
-constexpr int kS1Group = 8;
+// A block takes a run of columns of one instance (a slot: see s1_slot), a thread cpt cells of it, and G
+// separations in one pair of sweeps: a_j is loaded for all of them, and what remains per separation
+// and velocity cell is one load and three operations in either direction (1024 instances, N_v = 65,
+// eight separations: 2.4 ms; a block per instance and separation 6.5 ms).  The cells' sums are FP64
+// Neumaier sums per thread; the 2 G sums of a warp's lanes are folded by halving (every lane ends with
+// one of them) rather than by as many butterflies, which took longer than the sweeps.  The blocks'
+// sums go to part[group][slot][num, den of each][sum, compensation], folded in slot order.
+constexpr int kS1Group = 8;  // separations of a pair of sweeps at most
 constexpr int kS1Threads = 128;
 
 __device__ __forceinline__ Comp shfl_xor(const Comp& a, int m) {
@@ -219,11 +219,11 @@ __host__ __device__ __forceinline__ long long s1_slot(const Inst1D& in, int k, i
     return in.xoff / per + k;
 }
 
-template <typename T>
+template <typename T, int G>
 __global__ void __launch_bounds__(kS1Threads)
     k_s1_1d(const T* f, const Inst1D* inst, int n_inst, int cpt, int nv, const double* rho,
-            const int* seps, int q0, int nq, double* part) {
-    constexpr int NS = 2 * kS1Group;  // sums: 2 q the numerator, 2 q + 1 the denominator
+            const int* seps, double* part) {
+    constexpr int NS = 2 * G;  // sums: 2 q the numerator, 2 q + 1 the denominator
     __shared__ Comp wsum[kS1Threads / 32][NS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per = kS1Threads * cpt;
@@ -239,18 +239,18 @@ __global__ void __launch_bounds__(kS1Threads)
     if (first >= n) return;  // a slot without columns
     const int x0 = (int)first;
     const T* fk = f + in.off;
+    seps += blockIdx.y * G;
     Comp t[NS];
 #pragma unroll
     for (int q = 0; q < NS; ++q) t[q] = Comp{0, 0};
     for (int e = 0; e < cpt; ++e) {
         const int i = x0 + e * kS1Threads + threadIdx.x;
         if (i >= n) break;
-        int i2[kS1Group];
-        T acc[kS1Group], B[kS1Group], run[kS1Group];
+        int i2[G];
+        T acc[G], B[G], run[G];
 #pragma unroll
-        for (int q = 0; q < kS1Group; ++q) {
-            const int s = q < nq ? seps[q0 + q] : 0;
-            i2[q] = i + s < n ? i + s : i + s - n;
+        for (int q = 0; q < G; ++q) {
+            i2[q] = i < n - seps[q] ? i + seps[q] : i - (n - seps[q]);
             acc[q] = B[q] = run[q] = T(0);
         }
         const T* row = fk;
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kS1Threads)
         for (int j = 0; j < nv; ++j) {
             const T a = row[i];
 #pragma unroll
-            for (int q = 0; q < kS1Group; ++q) {
+            for (int q = 0; q < G; ++q) {
                 acc[q] += a * run[q];
                 B[q] += row[i2[q]];
                 run[q] += B[q];
@@ -266,13 +266,13 @@ __global__ void __launch_bounds__(kS1Threads)
             row += n;
         }
 #pragma unroll
-        for (int q = 0; q < kS1Group; ++q) B[q] = run[q] = T(0);
+        for (int q = 0; q < G; ++q) B[q] = run[q] = T(0);
 #pragma unroll 2
         for (int j = nv - 1; j >= 0; --j) {
             row -= n;
             const T a = row[i];
 #pragma unroll
-            for (int q = 0; q < kS1Group; ++q) {
+            for (int q = 0; q < G; ++q) {
                 acc[q] += a * run[q];
                 B[q] += row[i2[q]];
                 run[q] += B[q];
@@ -281,48 +281,52 @@ __global__ void __launch_bounds__(kS1Threads)
         const double* rk = rho + in.xoff;
         const double ri = rk[i];
 #pragma unroll
-        for (int q = 0; q < kS1Group; ++q) {
+        for (int q = 0; q < G; ++q) {
             nadd(t[2 * q], (double)acc[q]);
             nadd(t[2 * q + 1], ri * rk[i2[q]]);
         }
     }
-    // halve the sums a lane holds, level by level: after it lane l holds sum l / 2 over the
-    // lanes of its parity, then over all
+    // halve the sums a lane holds, level by level, until it holds one (of index lane / (32 / NS));
+    // the lanes left with the same one add theirs
 #pragma unroll
-    for (int h = NS / 2, m = 16; h >= 1; h >>= 1, m >>= 1) {
-        const bool up = (lane & m) != 0;
+    for (int m = 16, h = G; m >= 1; m >>= 1, h >>= 1) {
+        if (h >= 1) {
+            const bool up = (lane & m) != 0;
 #pragma unroll
-        for (int q = 0; q < h; ++q) {
-            const Comp keep = up ? t[q + h] : t[q], give = up ? t[q] : t[q + h];
-            t[q] = keep;
-            nmerge(t[q], shfl_xor(give, m));
+            for (int q = 0; q < h; ++q) {
+                const Comp keep = up ? t[q + h] : t[q], give = up ? t[q] : t[q + h];
+                t[q] = keep;
+                nmerge(t[q], shfl_xor(give, m));
+            }
+        } else {
+            nmerge(t[0], shfl_xor(t[0], m));
         }
     }
-    nmerge(t[0], shfl_xor(t[0], 1));
-    if ((lane & 1) == 0) wsum[warp][lane / 2] = t[0];
+    if (lane % (32 / NS) == 0) wsum[warp][lane / (32 / NS)] = t[0];
     __syncthreads();
     if (threadIdx.x < NS) {
         Comp z{0, 0};
         for (int w = 0; w < kS1Threads / 32; ++w) nmerge(z, wsum[w][threadIdx.x]);
-        double* p = part + ((size_t)blockIdx.x * NS + threadIdx.x) * 2;
+        double* p = part + (((size_t)blockIdx.y * gridDim.x + blockIdx.x) * NS + threadIdx.x) * 2;
         p[0] = z.s;
         p[1] = z.c;
     }
 }
 
-// One half-warp per instance folds its chunks' sums in order.
-__global__ void k_s1_fold(const double* part, int cpt, const Inst1D* inst, int n_inst,
-                          int q0, int nq, int ns, double* num, double* den) {
-    constexpr int NS = 2 * kS1Group;
-    const int k = (blockIdx.x * blockDim.x + threadIdx.x) / NS, q = threadIdx.x % NS;
-    if (k >= n_inst || q >= 2 * nq) return;
+// One thread per sum of an instance folds its slots' sums in order: groups of G separations, the
+// first one seps[q0].
+__global__ void k_s1_fold(const double* part, long long slots, int cpt, const Inst1D* inst,
+                          int n_inst, int G, int groups, int q0, int ns, double* num, double* den) {
+    const int NS = 2 * G, per = kS1Threads * cpt;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = (int)(i / (groups * NS)), r = (int)(i % (groups * NS));
+    if (k >= n_inst) return;
     const Inst1D& in = inst[k];
+    const double* p = part + (((r / NS) * slots + s1_slot(in, k, per)) * NS + r % NS) * 2;
     Comp z{0, 0};
-    const int per = kS1Threads * cpt;
-    const double* p = part + (s1_slot(in, k, per) * NS + q) * 2;
     for (long long x0 = 0; x0 < in.nx; x0 += per, p += 2 * NS) nmerge(z, Comp{p[0], p[1]});
-    const size_t o = (size_t)k * ns + q0 + q / 2;
-    if (q % 2 == 0) num[o] = nval(z) * in.dv * in.dv * in.dv / in.nx;
+    const size_t o = (size_t)k * ns + q0 + r / 2;
+    if (r % 2 == 0) num[o] = nval(z) * in.dv * in.dv * in.dv / in.nx;
     else den[o] = nval(z) / in.nx;
 }
 
@@ -330,6 +334,52 @@ __global__ void k_s1_fold(const double* part, int cpt, const Inst1D* inst, int n
 int s1_cells(long long total_x, int sm_count) {
     const long long c = total_x / ((long long)kS1Threads * 16 * sm_count);
     return (int)std::max(1ll, std::min(8ll, c));
+}
+
+// How ns separations of a state are dealt out: groups of G, `batch` of them per launch, then the rest in
+// groups of the smaller powers of two, so that no sweep is made for a separation that was not asked
+// for (each costs its own sums).  G is the largest that leaves four blocks per SM: few columns in large
+// groups would leave the SMs idle.  The call with the density, 512 instances of 1024 .. 4096 columns,
+// N_v = 9, FP32: one separation 190 us, nine 638 us (a block per instance and separation 216 and 629,
+// whole groups of eight 552 and 996); 9 instances of 256, N_v = 65, FP64, one 157 us (210, 253).
+struct S1Split {
+    int cpt, G, batch;
+    long long slots;
+};
+
+int pow2_from(int n) {
+    int p = 1;
+    while (p < n) p *= 2;
+    return p;
+}
+
+S1Split s1_split(int n_inst, long long total_x, int ns, int sm_count) {
+    S1Split q;
+    q.cpt = s1_cells(total_x, sm_count);
+    q.slots = total_x / (kS1Threads * q.cpt) + n_inst;
+    q.G = std::min(kS1Group, pow2_from(ns));
+    while (q.G > 1 && q.slots * ((ns + q.G - 1) / q.G) < 4ll * sm_count) q.G /= 2;
+    // groups together while their blocks would not fill sixteen per SM
+    const long long most = 16ll * sm_count / q.slots;
+    q.batch = (int)std::max(1ll, std::min<long long>(most, (ns + q.G - 1) / q.G));
+    return q;
+}
+
+template <typename T>
+cudaError_t launch_s1_group(int G, int groups, const S1Split& sp, const void* f, const Inst1D* inst,
+                            int n_inst, int nv, const double* rho, const int* seps, double* part,
+                            cudaStream_t s) {
+    const dim3 grid((unsigned)sp.slots, groups);
+    switch (G) {
+#define X(g) \
+    case g:  \
+        k_s1_1d<T, g><<<grid, kS1Threads, 0, s>>>(static_cast<const T*>(f), inst, n_inst, sp.cpt, \
+                                                  nv, rho, seps, part);                           \
+        return cudaGetLastError();
+        X(1) X(2) X(4) X(8)
+#undef X
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 int obs_grid(long long blocks, int sm_count) {
@@ -366,32 +416,31 @@ cudaError_t launch_coarse2d(const double* rho, int nx, int ny, double dx, const 
     return cudaGetLastError();
 }
 
-namespace {
-long long s1_slots(int n_inst, long long total_x, int sm_count) {
-    return total_x / (kS1Threads * s1_cells(total_x, sm_count)) + n_inst;
-}
-}  // namespace
-
-size_t s1_scratch(int n_inst, long long total_x, int sm_count) {
-    return (size_t)s1_slots(n_inst, total_x, sm_count) * 4 * kS1Group;
+size_t s1_scratch(int n_inst, long long total_x, int ns, int sm_count) {
+    const S1Split sp = s1_split(n_inst, total_x, ns, sm_count);
+    return (size_t)sp.slots * 4 * sp.batch * sp.G;
 }
 
 cudaError_t launch_s1_1d(int dtype, const void* f, const Inst1D* inst, int n_inst,
                          long long total_x, int nv, const double* rho, const int* seps, int ns,
                          double* part, double* num, double* den, int sm_count, cudaStream_t s) {
     if (dtype != LAT_F32 && dtype != LAT_F64) return cudaErrorInvalidValue;
-    const int cpt = s1_cells(total_x, sm_count);
-    const unsigned grid = (unsigned)s1_slots(n_inst, total_x, sm_count);
-    for (int q0 = 0; q0 < ns; q0 += kS1Group) {
-        const int nq = std::min(kS1Group, ns - q0);
-        if (dtype == LAT_F32)
-            k_s1_1d<float><<<grid, kS1Threads, 0, s>>>(static_cast<const float*>(f), inst, n_inst,
-                                                       cpt, nv, rho, seps, q0, nq, part);
-        else
-            k_s1_1d<double><<<grid, kS1Threads, 0, s>>>(static_cast<const double*>(f), inst, n_inst,
-                                                        cpt, nv, rho, seps, q0, nq, part);
-        k_s1_fold<<<(n_inst + 7) / 8, 16 * kS1Group, 0, s>>>(part, cpt, inst, n_inst, q0, nq,
-                                                             ns, num, den);
+    const S1Split sp = s1_split(n_inst, total_x, ns, sm_count);
+    for (int q0 = 0; q0 < ns;) {
+        int G = sp.G, groups = std::min(sp.batch, (ns - q0) / sp.G);
+        if (groups == 0) {
+            groups = 1;
+            while (G > ns - q0) G /= 2;
+        }
+        const cudaError_t e =
+            dtype == LAT_F32
+                ? launch_s1_group<float>(G, groups, sp, f, inst, n_inst, nv, rho, seps + q0, part, s)
+                : launch_s1_group<double>(G, groups, sp, f, inst, n_inst, nv, rho, seps + q0, part, s);
+        if (e != cudaSuccess) return e;
+        const long long sums = (long long)n_inst * groups * 2 * G;
+        k_s1_fold<<<(unsigned)((sums + 127) / 128), 128, 0, s>>>(part, sp.slots, sp.cpt, inst, n_inst,
+                                                                 G, groups, q0, ns, num, den);
+        q0 += groups * G;
     }
     return cudaGetLastError();
 }

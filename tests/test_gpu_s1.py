@@ -1,6 +1,7 @@
-"""S1 over groups of separations: any number of them (one group of eight and more), instances
+"""S1 over groups of separations: any number of them (groups of eight, four, two and one), instances
 of one and of many runs of columns, several cells per thread, against the oracle; scratch that grows
-with the columns, not with instances times the longest one."""
+with the columns, not with instances times the longest one; and a single separation that does not
+pay for eight."""
 import math
 
 import numpy as np
@@ -68,4 +69,24 @@ def test_scratch_follows_the_columns(lat):
     free = torch.cuda.mem_get_info()[0]
     check(ens, dv, 3, torch.float32, [1, 2, 3, 4, 5, 6, 7, 8], [0, 1, 5000, 10000])
     assert free - torch.cuda.mem_get_info()[0] < 256 << 20  # 11 MB of densities, the blocks' sums
+    ens.close()
+
+
+def test_one_separation_does_not_pay_for_eight(lat):
+    rng = np.random.default_rng(4)
+    ens, _ = ensemble(lat, list(map(int, rng.choice([1024, 2048, 4096], 512))), 9, torch.float32)
+
+    def best(seps):
+        out = math.inf
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        for _ in range(12):
+            a.record()
+            ens.s1(seps)
+            b.record()
+            b.synchronize()
+            out = min(out, a.elapsed_time(b))
+        return out
+
+    one, eight = best([1]), best(list(range(1, 9)))
+    assert one < 0.75 * eight, (one, eight)
     ens.close()
