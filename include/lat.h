@@ -138,8 +138,9 @@ int lat_set_noise(lat_ctx* c, const double* noise, long long rows);
 /* Enqueue n time steps (Section 2: stream, drag, diffuse) on the context's stream.  In the
  * default launch mode the n steps are one CUDA-graph launch; the graph is captured on first use
  * of that n and cached (see lat_prepare).  With the upwind drag and unless lat_set_launch chose a
- * kernel, up to eight small 1D lattices take all n steps in one launch, and other FP32 ones with
- * N_v in {9, 17, 33, 65} five per launch on chip while as many remain (the same bits). */
+ * kernel, up to eight small 1D lattices take all n steps in one launch where that is estimated to be
+ * faster, and other FP32 ones with N_v in {9, 17, 33, 65} five per launch on chip while as many
+ * remain (the same bits). */
 int lat_step(lat_ctx* c, int n);
 
 /* Capture and instantiate the graph for n steps now, without running it, so that a later

@@ -96,8 +96,9 @@ struct lat_ctx {
     void* d_basis = nullptr;
     size_t basis_cap = 0;             // bytes
     std::vector<int> basis_k;
-    // per number of modes, whether the cluster kernel takes the lattice: 0 not asked, 1 no, 2 yes
-    signed char line_fit[kMaxModes1D + 1] = {};
+    // per number of modes, the clusters of the small-lattice kernel that run at a time (line1d.cu),
+    // plus one; 0 not asked yet
+    int line_clusters[kMaxModes1D + 1] = {};
 
     // cached graphs keyed by the number of steps (buffers are picked by the device step parity)
     std::map<int, cudaGraphExec_t> graphs;
@@ -296,10 +297,10 @@ std::vector<MultiTile> make_tiles(const lat_ctx* c, bool lim, int* widest_places
     return tiles;
 }
 
-// Whether the cluster kernel takes the lattice, asked once per number of modes.
+// Asks whether the cluster kernel can take the lattice, once per number of modes.
 void fit_line(lat_ctx* c) {
-    signed char& fit = c->line_fit[c->nmodes];
-    if (!fit) fit = line1d_fits(c->dtype, c->n_inst, max_nx(c), c->nv, c->nmodes) ? 2 : 1;
+    int& q = c->line_clusters[c->nmodes];
+    if (!q) q = 1 + line1d_clusters(c->dtype, c->n_inst, max_nx(c), c->nv, c->nmodes);
 }
 
 // What batches of steps need of the grids: the tiles of the two on-chip kernels, the distinct grid
@@ -381,10 +382,30 @@ bool flow_rows(const lat_ctx* c) {
     return c->d_wflow && (c->flow_kind != LAT_FLOW_MODES || !c->basis_k.empty());
 }
 
-// Whether batches of steps run on the cluster kernel of small lattices.
-bool line_1d(const lat_ctx* c) {
-    return c->d == 1 && !c->pinned && c->mode != 1 && c->scheme == LAT_SCHEME_UPWIND &&
-           c->line_fit[c->nmodes] == 2 && !c->stalled;
+// About how long n upwind steps of a few small lattices take on the other kernels (us, a graph of n
+// steps): a launch per step is bound by the latency of a column's sweep (compiled N_v, or any), in FP64
+// by its pipe where the columns are many.  Measured per step: FP32 N_v = 5 3.2, 33 4.7, 65 6.5, 13
+// 6.6, 129 44 us; five steps on chip N_v = 9 9.0, 33 12.4, 65 21.6 us; FP64 N_v = 5 4.5, 33 14.4, 65
+// 26.1, 13 10.5, 129 79 us, 24,000 columns of 33 22 us.
+double launches_us(const lat_ctx* c, int n) {
+    const bool compiled = c->nv == 3 || c->nv == 5 || c->nv == 9 || c->nv == 17 || c->nv == 33 ||
+                          c->nv == 65;
+    if (c->dtype == LAT_F64)
+        return 8.0 + n * (2.7 + (compiled ? 0.36 : 0.58) * c->nv + 1.2e-5 * c->total_x * c->nv);
+    const double step = compiled ? 2.7 + 0.06 * c->nv : 1.9 + 0.36 * c->nv;
+    if (!(flow_rows(c) && c->tiles[0].n)) return 3.0 + n * step;
+    return 4.0 + n / kMultiT * (6.5 + 0.23 * c->nv) + n % kMultiT * step;
+}
+
+// Whether a batch of n steps runs on the cluster kernel of small lattices: where it is faster.  Ten steps
+// on the cluster against the launches: FP32 256 x 9 16 us and 21, 4096 x 5 47 and 35, 8888 x 3 86 and 37;
+// FP64 256 x 33 41 and 152, 1001 x 33 123 and 152, 4096 x 5 172 and 55.
+bool line_1d(const lat_ctx* c, int n) {
+    const int clusters = c->line_clusters[c->nmodes] - 1;
+    return n > 1 && c->d == 1 && !c->pinned && c->mode != 1 && c->scheme == LAT_SCHEME_UPWIND &&
+           !c->stalled && clusters > 0 &&
+           line1d_us(c->dtype, c->n_inst, max_nx(c), c->nv, c->nmodes, clusters, n) <
+               launches_us(c, n);
 }
 
 // Enqueue n steps of a 1D context on stream s (used directly and under capture).  Where no launch
@@ -393,7 +414,7 @@ bool line_1d(const lat_ctx* c) {
 int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
     const bool chosen = c->pinned || c->mode == 1;
     const bool on_chip = !chosen && c->scheme == LAT_SCHEME_UPWIND;
-    if (n > 1 && line_1d(c)) {
+    if (line_1d(c, n)) {
         CK(launch_line1d(c->dtype, c->n_inst, max_nx(c), c->nv, step_args(c, 0, 0), 0, n, s));
         if (c->n_inst > 1) CK(launch_advance_step(c->d_state, n, s));
         return LAT_OK;
@@ -827,7 +848,7 @@ int enqueue_step_moments(lat_ctx* c, int n, double* rho, double* mean_v, double*
         return LAT_OK;
     }
     const bool fused = c->d == 1 && c->variant == STEP1D_PC && c->mode != 1 &&
-                       step1d_moments_supported(c->dtype, c->nv) && !(n > 1 && line_1d(c));
+                       step1d_moments_supported(c->dtype, c->nv) && !line_1d(c, n);
     if (!fused) {
         int rc = lat_step(c, n);
         if (rc != LAT_OK) return rc;

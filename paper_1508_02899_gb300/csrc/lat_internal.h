@@ -123,7 +123,10 @@ cudaError_t launch_lim1d(int nv, int ntiles, int places, const Step1DArgs& a, co
                          int kstep, const float* wrow, int piped, cudaStream_t s);
 // Steps kstep .. kstep + n - 1 of small 1D lattices (upwind drag), one cluster per lattice with the
 // state in shared memory throughout (line1d.cu).
-bool line1d_fits(int dtype, int n_inst, int nx_max, int nv, int nmodes);
+// line1d_clusters: clusters that run at a time, 0 where there is no kernel; line1d_us: about how long n
+// steps take.
+int line1d_clusters(int dtype, int n_inst, int nx_max, int nv, int nmodes);
+double line1d_us(int dtype, int n_inst, int nx_max, int nv, int nmodes, int clusters, int n);
 cudaError_t launch_line1d(int dtype, int n_inst, int nx_max, int nv, const Step1DArgs& a, int kstep,
                           int n, cudaStream_t s);
 // Tables of the flow's basis, one per grid size (sizes: an instance of each; nx_max the largest):

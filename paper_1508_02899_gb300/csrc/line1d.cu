@@ -40,7 +40,7 @@ constexpr int kCluster = 16;
 constexpr int kCellThreads = 992;  // at most; 32 more for the flow
 constexpr size_t kMaxSmem = 220 * 1024;
 constexpr int kMaxInst = 8;
-constexpr long long kMaxCells64 = 80000, kMaxCells32 = 30000;
+constexpr long long kMaxCells64 = 80000, kMaxCells32 = 30000;  // larger ones: not measured
 
 template <typename T>
 size_t line_smem(int nv, int w, int nmodes) {
@@ -263,14 +263,14 @@ cudaError_t config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int n_inst,
 }
 
 template <typename T, bool ONE>
-bool runs(int nv, int w, int nmodes) {
+int runs(int nv, int w, int nmodes) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
     int nclusters = 0;
-    return line_smem<T>(nv, w, nmodes) <= kMaxSmem &&
-           config<T, ONE>(&cfg, &at, 1, nv, w, nmodes, nullptr) == cudaSuccess &&
-           cudaOccupancyMaxActiveClusters(&nclusters, k_line1d<T, ONE>, &cfg) == cudaSuccess &&
-           nclusters > 0;
+    const bool ok = line_smem<T>(nv, w, nmodes) <= kMaxSmem &&
+                    config<T, ONE>(&cfg, &at, 1, nv, w, nmodes, nullptr) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&nclusters, k_line1d<T, ONE>, &cfg) == cudaSuccess;
+    return ok ? nclusters : 0;
 }
 
 template <typename T, bool ONE>
@@ -288,20 +288,30 @@ int columns(int nx_max) { return (nx_max + kCluster - 1) / kCluster; }
 
 }  // namespace
 
-// FP32 up to 30,000 cells (39,600 cells of N_v = 33: 3.05 us here, 2.69 on multi1d.cu's tiles; 19,500 of
-// N_v = 65: 1.95 against 4.36); FP64 up to 80,000 (0.32 us per 1000 cells, where a launch per step
-// in narrow blocks takes 23 us at N_v = 33 and 34 at 65 whatever the columns), as far as shared
-// memory holds them; at most eight lattices, one cluster each.
-bool line1d_fits(int dtype, int n_inst, int nx_max, int nv, int nmodes) {
+// At most eight lattices, one cluster each, as far as shared memory holds them.
+int line1d_clusters(int dtype, int n_inst, int nx_max, int nv, int nmodes) {
     const long long cells = (long long)nx_max * nv;
-    if (n_inst > kMaxInst || cells > (dtype == LAT_F64 ? kMaxCells64 : kMaxCells32)) return false;
+    if (n_inst > kMaxInst || cells > (dtype == LAT_F64 ? kMaxCells64 : kMaxCells32)) return 0;
     const int w = columns(nx_max);
     const bool one = nv * w <= kCellThreads;
-    const bool ok = dtype == LAT_F64
-                        ? (one ? runs<double, true>(nv, w, nmodes) : runs<double, false>(nv, w, nmodes))
-                        : (one ? runs<float, true>(nv, w, nmodes) : runs<float, false>(nv, w, nmodes));
-    if (!ok) cudaGetLastError();
-    return ok;
+    const int n = dtype == LAT_F64
+                      ? (one ? runs<double, true>(nv, w, nmodes) : runs<double, false>(nv, w, nmodes))
+                      : (one ? runs<float, true>(nv, w, nmodes) : runs<float, false>(nv, w, nmodes));
+    if (n == 0) cudaGetLastError();
+    return n;
+}
+
+// A step is bound by the flow warp, which takes a block's columns 32 at a time, or by the cells; more
+// clusters than run at a time take turns.  Measured per step (and a launch's fixed part), eight modes:
+// FP64 N_x = 256, N_v = 9 2.0 us (6.3); 1001, 33 11.1 us (11.8); 4096, 5 14.9 us (23); FP32 256, 9
+// 0.9 us (5.7); 1001, 21 2.0 us (6.3); 8888, 3 7.9 us (7).
+double line1d_us(int dtype, int n_inst, int nx_max, int nv, int nmodes, int clusters, int n) {
+    const int rounds = (columns(nx_max) + 31) / 32;
+    const double modes = rounds * (nmodes / 8.0), kcells = 1e-3 * nx_max * nv;
+    const int turns = (n_inst + clusters - 1) / clusters;
+    if (dtype == LAT_F64)
+        return 5.0 + turns * (2.2 * modes + n * (0.4 + 0.1 * rounds + 1.2 * modes + 0.25 * kcells));
+    return 5.5 + turns * (0.3 * modes + n * (0.4 + 0.05 * rounds + 0.38 * modes + 0.03 * kcells));
 }
 
 cudaError_t launch_line1d(int dtype, int n_inst, int nx_max, int nv, const Step1DArgs& a, int kstep,
