@@ -12,8 +12,8 @@
 // mbarrier) into a 4-slot ring, two rows ahead of the sweep: the streaming shift is applied by
 // the copy's source address (x window rounded down to 16 bytes, split in two at the periodic
 // wrap; y wraps by choosing the source row).  A plain-load variant with the same arithmetic
-// serves grids the copy path does not cover (N_x not a multiple of 4, or < 132); FP64 lattices have
-// their own kernel (step2d_f64.cu).
+// serves grids the copy path does not cover (N_x not a multiple of 4, or < 132) and FP64 grids that
+// fill the SMs with a thread per cell; the others have their own kernel (step2d_f64.cu).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
@@ -67,7 +67,7 @@ struct Flow2DArgs {
     int frozen, dry;
 };
 
-// ---- plain-load kernel (any N_x, N_y) -------------------------------------------------------
+// ---- plain-load kernel (any N_x, N_y; FP32 or FP64) -----------------------------------------
 template <typename T, int NV>
 __global__ void __launch_bounds__(TW) k_step2d_plain(const Step2DArgs a, int kstep) {
     const long long step = a.st->step + kstep;
@@ -1228,11 +1228,12 @@ bool pc_supported(int nv) {
     }
 }
 
-cudaError_t launch_step2d(int nv, bool ring, int chunks, int pcv, int grid,
+cudaError_t launch_step2d(int dtype, int nv, bool ring, int chunks, int pcv, int grid,
                           const Step2DArgs& a, int k, cudaStream_t s) {
     switch (nv) {
 #define X(n)                                                                   \
     case n:                                                                    \
+        if (dtype == LAT_F64) return launch_plain<double, n>(grid, a, k, s);   \
         if (ring && pcv) return launch_pc_v<n>(pcv, grid, a, k, s);            \
         if (ring) return launch_ring_c<n>(chunks, grid, a, k, s);              \
         return launch_plain<float, n>(grid, a, k, s);
@@ -1502,10 +1503,10 @@ int enqueue2d(Ctx2D* c, void* const f[2], int n, cudaStream_t s, int dry) {
             const Step2DHArgs ha = half_args(c, a);
             CK2(launch_scale2d(c->nv, c->ny, ha, k, s));
             CK2(launch_step2d_h(c->dtype, c->nv, c->ring ? c->pcv : 0, grid, ha, k, s));
-        } else if (c->dtype == LAT_F64) {
+        } else if (c->dtype == LAT_F64 && step2d_f64_tiles(c->nv, c->nx, c->ny, c->sm_count)) {
             CK2(launch_step2d_f64(c->nv, c->sm_count, a, k, s));
         } else {
-            CK2(launch_step2d(c->nv, c->ring, c->chunks, c->pcv, grid, a, k, s));
+            CK2(launch_step2d(c->dtype, c->nv, c->ring, c->chunks, c->pcv, grid, a, k, s));
         }
     }
     if (!dry) {

@@ -291,7 +291,9 @@ cudaError_t launch_step2d_limited(int dtype, const k2d::Step2DArgs& s2, int nv, 
                                   cudaStream_t s);
 bool limiter2d_fused_supported(int nv);
 
-// FP64 step with the upwind drag (step2d_f64.cu), every N_v of the 2D kernels.
+// FP64 step with the upwind drag on tiles (step2d_f64.cu), every N_v of the 2D kernels; where it is
+// faster than the plain kernel's thread per cell.
+bool step2d_f64_tiles(int nv, int nx, int ny, int sm_count);
 cudaError_t launch_step2d_f64(int nv, int sm_count, const k2d::Step2DArgs& a, int k, cudaStream_t s);
 
 }  // namespace lat

@@ -14,8 +14,8 @@
 //  * the diffusion is one fma with the sum of the differences of f** (rounded as differences, not as
 //    four scaled fluxes).
 //
-// Measured (128^2 x 33^2): 0.87 ms per step, the FP64 pipe 75 % active, against 0.97 with a thread
-// per cell.
+// A thread per cell and column sweep (step2d.cu's plain kernel) issues fewer instructions beside the FP64
+// ones and is faster where its 128-cell blocks fill the SMs evenly: step2d_f64_tiles chooses.
 #include <algorithm>
 
 #include "lat_internal.h"
@@ -178,6 +178,22 @@ cudaError_t launch_t(int sm_count, const Step2DArgs& a, int k, cudaStream_t s) {
 }
 
 }  // namespace
+
+// Time in units of an SM that gets one 128-cell block of the plain kernel, which is what this one takes
+// for 128 cells per SM; the plain kernel takes `plain` of it.  Blocks land on the SMs in pairs: 300 to
+// 304 of them (152 SMs) take two units, 320 take four.  Measured per step (us), tiles against plain:
+// N_v = 33 128 x 128 874 and 917, 160 x 160 1360 and 3198, 256 x 150 1987 and 1615; N_v = 17 160 x 160
+// 330 and 860, 256 x 150 509 and 438, 512 x 256 1621 and 1720; N_v = 9 160 x 160 99 and 185, 512 x 300
+// 503 and 544, 512 x 512 856 and 843.
+bool step2d_f64_tiles(int nv, int nx, int ny, int sm_count) {
+    const double plain = nv >= 33 ? 0.81 : nv >= 19 ? 0.915 : nv >= 17 ? 0.88 : nv >= 13 ? 0.97
+                       : nv >= 9 ? 1.1 : nv >= 5 ? 0.92 : nv >= 3 ? 1.0 : 0.7;
+    const int TC = nv >= 33 ? 8 : nv >= 17 ? 16 : 32;  // Tile64<NV>::TC
+    const long long blocks = (long long)((nx + TW - 1) / TW) * ny, pair = 2ll * sm_count;
+    const double units = blocks <= sm_count ? 1.13 : 2.0 * ((blocks + pair - 1) / pair);
+    const double cells = (double)((nx + TC - 1) / TC * TC) * ny / (128.0 * sm_count);
+    return cells < plain * units;
+}
 
 cudaError_t launch_step2d_f64(int nv, int sm_count, const k2d::Step2DArgs& a, int k, cudaStream_t s) {
     switch (nv) {
