@@ -810,13 +810,10 @@ __device__ __forceinline__ double to_d(T v) { return (double)v; }
 
 constexpr int kMom2DWarps = 8;  // warps per moment block (256 threads)
 
-// f of one cell (both lanes the same) or of two neighbouring cells.
-template <typename T, bool PAIR>
+// f of two neighbouring cells.
+template <typename T>
 __device__ __forceinline__ f2 load_cells(const T* p) {
-    if constexpr (!PAIR) {
-        const float v = (float)*p;
-        return pk(v, v);
-    } else if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 4) {
         return *reinterpret_cast<const f2*>(p);
     } else {
         T h[2];
@@ -845,32 +842,98 @@ __device__ __forceinline__ void two_sum_merge(f2& s, f2& c, f2 os, f2 oc) {
 //   FP64 storage: Neumaier FP64 throughout.
 //   FP32 / FP16 / BF16 storage: FP32 Kahan sums per cell and across a thread's cells and the
 //   warp (exact integer weights); FP64 from the warp partials on (FP64 is slow on this GPU).
-template <typename T, bool PAIR = false>
-__global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* scales, int nv,
-                                                   int nx, int ny, double dv, double* rho,
-                                                   double* mv, double* mv2, double* partials,
-                                                   DevState* st) {
+// Forms: a thread per cell; FP64 also a block per 32 cells (kMomTile), for grids of few cells; the others
+// also two neighbouring cells per thread in the lanes of f32x2 pairs, for grids of many.  Velocity rows
+// unrolled by four or eight, or with the loads of eight (the rest one by one) or seven (the rest
+// masked) ahead of their sums; mom2d_form chooses.  Four blocks per SM: with 70 registers the 16-bit
+// forms held three, and 362 x 362 cells took two waves (N_v = 33, FP16: 399 us, now 188).
+enum MomForm { kMomCell, kMomCell8, kMomTile, kMomPair4, kMomPair7, kMomPair8 };
+
+// take(jx, load(jx)) for a velocity row.
+template <MomForm FORM, class Load, class Take>
+__device__ __forceinline__ void mom_row(int nv, const Load& load, const Take& take) {
+    if constexpr (FORM == kMomCell8 || FORM == kMomPair7) {
+        constexpr bool whole = FORM == kMomCell8;
+        constexpr int W = whole ? 8 : 7;
+        int jx = 0;
+#pragma unroll 1
+        for (; whole ? jx + W <= nv : jx < nv; jx += W) {
+            decltype(load(0)) v[W];
+#pragma unroll
+            for (int e = 0; e < W; ++e) v[e] = whole || jx + e < nv ? load(jx + e) : 0;
+#pragma unroll
+            for (int e = 0; e < W; ++e)
+                if (whole || jx + e < nv) take(jx + e, v[e]);
+        }
+#pragma unroll 1
+        for (; jx < nv; ++jx) take(jx, load(jx));
+    } else {
+        constexpr int U = FORM == kMomPair8 ? 8 : 4;
+#pragma unroll(U)
+        for (int jx = 0; jx < nv; ++jx) take(jx, load(jx));
+    }
+}
+
+template <typename T, MomForm FORM>
+__global__ void __launch_bounds__(256, FORM == kMomCell && sizeof(T) == sizeof(double) ? 3 : 4)
+    k_moments2d(const void* fv, const float* scales, int nv, int nx, int ny, double dv, double* rho,
+                double* mv, double* mv2, double* partials, DevState* st) {
     const T* f = static_cast<const T*>(fv);
     const int J = (nv - 1) / 2;
     const long long ncell = (long long)nx * ny;
     const double dv2 = __dmul_rn(dv, dv);
-    const f2 zero2 = opaque2(0ull);  // keeps a packed product from fusing with an addition
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double* p = partials + (size_t)blockIdx.x * 8;  // one partial per block
     bool bad = false;
     if constexpr (sizeof(T) == sizeof(double)) {
-        // A block takes 32 cells at a time, warp w their velocity rows w, w + 8, ..; warp 0 merges
-        // the warps in order (128^2 cells with a thread each are 64 blocks: 2.35 ms).
-        __shared__ Comp part[kMom2DWarps - 1][4][32];
         Comp t[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-        for (long long c0 = (long long)blockIdx.x * 32; c0 < ncell; c0 += (long long)gridDim.x * 32) {
-            const long long c = c0 + lane;
-            Comp s[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-            if (c < ncell) {
-                for (int jy = warp; jy < nv; jy += kMom2DWarps) {
-                    const double vy = __dmul_rn((double)(jy - J), dv);
-                    const double vy2 = __dmul_rn(vy, vy);
+        if constexpr (FORM == kMomTile) {
+            // A block takes 32 cells at a time, warp w their velocity rows w, w + 8, ..; warp 0 merges
+            // the warps in order (128^2 cells with a thread each are 64 blocks: 2.35 ms).
+            __shared__ Comp part[kMom2DWarps - 1][4][32];
+            for (long long c0 = (long long)blockIdx.x * 32; c0 < ncell; c0 += (long long)gridDim.x * 32) {
+                const long long c = c0 + lane;
+                Comp s[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+                if (c < ncell) {
+                    for (int jy = warp; jy < nv; jy += kMom2DWarps) {
+                        const double vy = __dmul_rn((double)(jy - J), dv);
+                        const double vy2 = __dmul_rn(vy, vy);
 #pragma unroll 4
+                        for (int jx = 0; jx < nv; ++jx) {
+                            const double vx = __dmul_rn((double)(jx - J), dv);
+                            const size_t plane = (size_t)jy * nv + jx;
+                            const double fvv = to_d(f[plane * ncell + c]);
+                            bad |= !isfinite(fvv);
+                            nadd(s[0], fvv);
+                            nadd(s[1], __dmul_rn(vx, fvv));
+                            nadd(s[2], __dmul_rn(vy, fvv));
+                            nadd(s[3], __dmul_rn(__dadd_rn(__dmul_rn(vx, vx), vy2), fvv));
+                        }
+                    }
+                    if (warp > 0)
+                        for (int q = 0; q < 4; ++q) part[warp - 1][q][lane] = s[q];
+                }
+                __syncthreads();
+                if (warp == 0 && c < ncell) {
+                    for (int w = 0; w < kMom2DWarps - 1; ++w)
+                        for (int q = 0; q < 4; ++q) nmerge(s[q], part[w][q][lane]);
+                    const double m0 = nval(s[0]);
+                    if (rho) rho[c] = m0 * dv * dv;
+                    if (mv) {
+                        mv[c] = m0 != 0.0 ? nval(s[1]) / m0 : 0.0;
+                        mv[ncell + c] = m0 != 0.0 ? nval(s[2]) / m0 : 0.0;
+                    }
+                    if (mv2) mv2[c] = m0 != 0.0 ? nval(s[3]) / m0 : 0.0;
+                    for (int q = 0; q < 4; ++q) nmerge(t[q], s[q]);
+                }
+                __syncthreads();
+            }
+        } else {
+            for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < ncell;
+                 c += (long long)gridDim.x * blockDim.x) {
+                Comp s[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+                for (int jy = 0; jy < nv; ++jy) {
+                    const double vy = __dmul_rn((double)(jy - J), dv);
                     for (int jx = 0; jx < nv; ++jx) {
                         const double vx = __dmul_rn((double)(jx - J), dv);
                         const size_t plane = (size_t)jy * nv + jx;
@@ -879,16 +942,9 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
                         nadd(s[0], fvv);
                         nadd(s[1], __dmul_rn(vx, fvv));
                         nadd(s[2], __dmul_rn(vy, fvv));
-                        nadd(s[3], __dmul_rn(__dadd_rn(__dmul_rn(vx, vx), vy2), fvv));
+                        nadd(s[3], __dmul_rn(__dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy)), fvv));
                     }
                 }
-                if (warp > 0)
-                    for (int q = 0; q < 4; ++q) part[warp - 1][q][lane] = s[q];
-            }
-            __syncthreads();
-            if (warp == 0 && c < ncell) {
-                for (int w = 0; w < kMom2DWarps - 1; ++w)
-                    for (int q = 0; q < 4; ++q) nmerge(s[q], part[w][q][lane]);
                 const double m0 = nval(s[0]);
                 if (rho) rho[c] = m0 * dv * dv;
                 if (mv) {
@@ -898,7 +954,6 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
                 if (mv2) mv2[c] = m0 != 0.0 ? nval(s[3]) / m0 : 0.0;
                 for (int q = 0; q < 4; ++q) nmerge(t[q], s[q]);
             }
-            __syncthreads();
         }
         for (int q = 0; q < 4; ++q) warp_reduce(t[q]);
         __shared__ Comp wsum[kMom2DWarps][4];
@@ -916,10 +971,26 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
         // per cell: the mass exact up to the roundings of its compensation (TwoSum per velocity
         // row, rows merged); the weighted sums one FMA per value (the integer weights exact, the
         // product exact inside the FMA), error at most (N_v^2 - 1) u of the sum of
-        // |weight f|, u = 2^-24.  PAIR: two neighbouring cells per thread in the lanes of f32x2
-        // pairs, one load for both (1024^2 x 33^2: FP16 1.34 -> 0.60 ms, a scalar thread per cell
-        // is bound by its instructions).
+        // |weight f|, u = 2^-24
         FComp t[4];
+        // the sums of cell c: mass; sum jx f, jy f, (jx^2 + jy^2) f
+        auto done = [&](long long c, const FComp& s0, float s1, float s2, float s3) {
+            bad |= !isfinite(s0.s) || !isfinite(s3);
+            if (rho || mv || mv2) {  // FP64 per cell only when asked for (FP64 is slow here)
+                const double m0 = nval(s0.to_comp(1.0));
+                if (rho) rho[c] = m0 * dv2;
+                if (mv) {
+                    mv[c] = m0 != 0.0 ? __dmul_rn((double)s1, dv) / m0 : 0.0;
+                    mv[ncell + c] = m0 != 0.0 ? __dmul_rn((double)s2, dv) / m0 : 0.0;
+                }
+                if (mv2) mv2[c] = m0 != 0.0 ? __dmul_rn((double)s3, dv2) / m0 : 0.0;
+            }
+            t[0].merge(s0);
+            t[1].merge(FComp{s1, 0.f});
+            t[2].merge(FComp{s2, 0.f});
+            t[3].merge(FComp{s3, 0.f});
+        };
+        constexpr bool PAIR = FORM >= kMomPair4;
         const long long nunit = PAIR ? ncell / 2 : ncell;
         for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nunit;
              q += (long long)gridDim.x * blockDim.x) {
@@ -927,48 +998,57 @@ __global__ void __launch_bounds__(256) k_moments2d(const void* fv, const float* 
             // scales of this cell's row: [jy][jx padded]
             const float* sc_c =
                 sizeof(T) == 2 ? scales + (size_t)(c / nx) * nv * nv_padded(nv) : nullptr;
-            f2 S = 0ull, C = 0ull, s1 = 0ull, s2 = 0ull, s3 = 0ull;  // mass (sum, -error); weighted
-            for (int jy = 0; jy < nv; ++jy) {
-                const float fy = (float)(jy - J);
-                const float fy2 = fy * fy;
-                f2 rs = 0ull, rc = 0ull, ex = 0ull;  // the velocity row: mass, sum jx f
-                const T* fr = f + (size_t)jy * nv * ncell + c;
-#pragma unroll 8
-                for (int jx = 0; jx < nv; ++jx) {
-                    const float fx = (float)(jx - J);
-                    f2 v = load_cells<T, PAIR>(fr + (size_t)jx * ncell);
-                    if constexpr (sizeof(T) == 2) {  // exact: powers of two
-                        const float sv = sc_c[jy * nv_padded(nv) + jx];
-                        v = fma2(v, pk(sv, sv), zero2);
-                    }
-                    two_sum_add(rs, rc, v);
-                    ex = fma2(pk(fx, fx), v, ex);
-                    const float w3 = __fmaf_rn(fx, fx, fy2);
-                    s3 = fma2(pk(w3, w3), v, s3);
+            if constexpr (PAIR) {
+                const f2 zero2 = opaque2(0ull);  // keeps a packed product from fusing with an addition
+                f2 S = 0ull, C = 0ull, s1 = 0ull, s2 = 0ull, s3 = 0ull;
+                for (int jy = 0; jy < nv; ++jy) {
+                    const float fy = (float)(jy - J);
+                    const float fy2 = fy * fy;
+                    f2 rs = 0ull, rc = 0ull, ex = 0ull;  // the velocity row: mass, sum jx f
+                    const T* fr = f + (size_t)jy * nv * ncell + c;
+                    mom_row<FORM>(
+                        nv, [&](int jx) { return load_cells<T>(fr + (size_t)jx * ncell); },
+                        [&](int jx, f2 v) {
+                            const float fx = (float)(jx - J);
+                            if constexpr (sizeof(T) == 2) {  // exact: powers of two
+                                const float sv = sc_c[jy * nv_padded(nv) + jx];
+                                v = fma2(v, pk(sv, sv), zero2);
+                            }
+                            two_sum_add(rs, rc, v);
+                            ex = fma2(pk(fx, fx), v, ex);
+                            const float w3 = __fmaf_rn(fx, fx, fy2);
+                            s3 = fma2(pk(w3, w3), v, s3);
+                        });
+                    two_sum_merge(S, C, rs, rc);
+                    s1 = add2(s1, ex);
+                    s2 = fma2(pk(fy, fy), sub2(rs, rc), s2);
                 }
-                two_sum_merge(S, C, rs, rc);
-                s1 = add2(s1, ex);
-                s2 = fma2(pk(fy, fy), sub2(rs, rc), s2);
-            }
-#pragma unroll
-            for (int e = 0; e < (PAIR ? 2 : 1); ++e) {
-                const FComp s0{e ? hi(S) : lo(S), e ? hi(C) : lo(C)};
-                const float m1 = e ? hi(s1) : lo(s1), m2 = e ? hi(s2) : lo(s2),
-                            m3 = e ? hi(s3) : lo(s3);
-                bad |= !isfinite(s0.s) || !isfinite(m3);
-                if (rho || mv || mv2) {  // FP64 per cell only when asked for (FP64 is slow here)
-                    const double m0 = nval(s0.to_comp(1.0));
-                    if (rho) rho[c + e] = m0 * dv2;
-                    if (mv) {
-                        mv[c + e] = m0 != 0.0 ? __dmul_rn((double)m1, dv) / m0 : 0.0;
-                        mv[ncell + c + e] = m0 != 0.0 ? __dmul_rn((double)m2, dv) / m0 : 0.0;
-                    }
-                    if (mv2) mv2[c + e] = m0 != 0.0 ? __dmul_rn((double)m3, dv2) / m0 : 0.0;
+                done(c, FComp{lo(S), lo(C)}, lo(s1), lo(s2), lo(s3));
+                done(c + 1, FComp{hi(S), hi(C)}, hi(s1), hi(s2), hi(s3));
+            } else {
+                FComp s0;
+                float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+                for (int jy = 0; jy < nv; ++jy) {
+                    const float fy = (float)(jy - J);
+                    const float fy2 = fy * fy;
+                    FComp ey;        // sum f of the velocity row
+                    float ex = 0.f;  // sum jx f of the velocity row
+                    const T* fr = f + (size_t)jy * nv * ncell + c;
+                    mom_row<FORM>(
+                        nv, [&](int jx) { return (float)fr[(size_t)jx * ncell]; },
+                        [&](int jx, float v) {
+                            const float fx = (float)(jx - J);
+                            if constexpr (sizeof(T) == 2)  // exact: powers of two
+                                v = v * sc_c[jy * nv_padded(nv) + jx];
+                            ey.add_exact(v);
+                            ex = __fmaf_rn(fx, v, ex);
+                            s3 = __fmaf_rn(__fmaf_rn(fx, fx, fy2), v, s3);
+                        });
+                    s0.merge(ey);
+                    s1 = __fadd_rn(s1, ex);
+                    s2 = __fmaf_rn(fy, __fsub_rn(ey.s, ey.c), s2);
                 }
-                t[0].merge(s0);
-                t[1].merge(FComp{m1, 0.f});
-                t[2].merge(FComp{m2, 0.f});
-                t[3].merge(FComp{m3, 0.f});
+                done(c, s0, s1, s2, s3);
             }
         }
         for (int q = 0; q < 4; ++q) warp_reduce(t[q]);
@@ -1321,7 +1401,6 @@ struct Ctx2D {
     double* d_partials = nullptr;
     double* d_glob = nullptr;
     double* h_glob = nullptr;
-    int mom_blocks = 0;
     std::map<int, cudaGraphExec_t> graphs;
 };
 
@@ -1572,12 +1651,8 @@ int ctx2d_create(Ctx2D** out, const lat_grid* g, DevState* st, int sm_count, cud
     c->chunks = chunks_supported(c->nv, 3) ? 3 : 1;
     c->pcv = c->ring && pc_ok(c) ? (half ? 6 : 9) : 0;
     if (half && !c->pcv) c->ring = false;
-    const long long ncell = (long long)c->nx * c->ny;
-    // a thread per cell, or (FP64) a block per 32 cells
-    const int mom_cells = c->dtype == LAT_F64 ? 32 : 256;
-    c->mom_blocks = (int)std::min<long long>((ncell + mom_cells - 1) / mom_cells, 8LL * sm_count);
-    // room for the moment kernel's block partials or the fused step's warp partials
-    const size_t npart = std::max<size_t>(c->mom_blocks, (size_t)8 * sm_count * (TW / 32));
+    // room for the fused step's warp partials, more than the moment kernel's blocks
+    const size_t npart = (size_t)8 * sm_count * (TW / 32);
     if (cudaMalloc(&c->d_partials, sizeof(double) * 8 * npart) != cudaSuccess ||
         cudaMalloc(&c->d_glob, sizeof(double) * 4) != cudaSuccess ||
         cudaMallocHost(&c->h_glob, sizeof(double) * 4) != cudaSuccess) {
@@ -1795,31 +1870,58 @@ int copy_globals(Ctx2D* c, double* globals, bool wait, cudaStream_t s) {
     return LAT_OK;
 }
 
-// Cells from which the moments take two per thread: a smaller grid does not fill the SMs with a thread
-// per cell (one step and moments, pair against single: 456 x 213, N_v = 19 253 and 235 us; 64^2, 17
-// 140 and 127 us; 512 x 400, 19 325 and 377 us).
-constexpr long long kPairCells = 1 << 17;
+// Form of the moment kernel.
+//  * FP64: both forms are bound by the FP64 pipe, u = N_v^2 units per 256 cells of an SM.  A thread per
+//    cell takes whole blocks of 256 cells; a block per 32 cells takes 23 units more per 256 and
+//    9 + u / 8 for its serial parts.  N_v = 33, 128 x 128: 1.26 against 2.34 ms (a thread per cell), N_v = 9,
+//    512 x 300 920 against 796 us, N_v = 3, 256 x 150 192 against 89 us.
+//  * Others: pairs of cells, where a pair lies in one grid row and is aligned, for more cells than four
+//    blocks per SM of threads with one (FP16, N_v = 33: 362 x 362 188 us and 234 in pairs, 512 x 512 312
+//    and 264); per-cell outputs of up to five velocities want the threads for their FP64 divisions
+//    (N_v = 5, 512 x 400: 95 and 104 us).  Rows by fours or eights as they divide: one cell, FP32, 300 x 200
+//    N_v = 33 226 and 166 us, 13 66 and 70; pairs, 1024 x 600, FP16 N_v = 17 194 and 182 us, 13 144 and 166,
+//    FP32 21 326 by fours, 263 by masked sevens (16-bit 256 and 327: their scales are masked too).
+MomForm mom2d_form(const Ctx2D* c, const void* f, bool per_cell) {
+    const long long ncell = (long long)c->nx * c->ny;
+    if (c->dtype == LAT_F64) {
+        const double u = (double)c->nv * c->nv, blocks = (ncell + 255) / 256;
+        return (u + 23.0) * blocks / c->sm_count + 9.0 + u / 8 < u * ceil(blocks / c->sm_count)
+                   ? kMomTile : kMomCell;
+    }
+    const int nv = c->nv, rest = nv % 8;
+    if (c->nx % 2 != 0 || (uintptr_t)f % 8 != 0 || ncell <= 4 * 256 * c->sm_count ||
+        (per_cell && nv <= 5))
+        return nv >= 9 && (rest == 1 || rest == 3) ? kMomCell8 : kMomCell;
+    if (rest == 1) return kMomPair8;
+    return c->dtype == LAT_F32 && nv > 8 ? kMomPair7 : kMomPair4;
+}
 
 int ctx2d_moments(Ctx2D* c, const void* f, int cur, double* rho, double* mean_v,
                   double* mean_v2, double* globals, bool wait, cudaStream_t s) {
     const float* sc = c->half ? c->d_sc + (size_t)cur * c->nlines : nullptr;
+    const MomForm form = mom2d_form(c, f, rho || mean_v || mean_v2);
+    const long long cells = form == kMomTile ? 32 : 256;  // of a block
+    const int blocks = (int)std::min<long long>(((long long)c->nx * c->ny + cells - 1) / cells,
+                                                8LL * c->sm_count);
     auto run = [&](auto kernel) {
-        kernel<<<c->mom_blocks, 32 * kMom2DWarps, 0, s>>>(f, sc, c->nv, c->nx, c->ny, c->dv, rho,
-                                                         mean_v, mean_v2, c->d_partials, c->st);
+        kernel<<<blocks, 32 * kMom2DWarps, 0, s>>>(f, sc, c->nv, c->nx, c->ny, c->dv, rho, mean_v,
+                                                   mean_v2, c->d_partials, c->st);
     };
-    // pairs of cells where a pair lies in one grid row and is aligned, on grids that fill the SMs
-    const bool pair = c->nx % 2 == 0 && (uintptr_t)f % 8 == 0 &&
-                      (long long)c->nx * c->ny >= kPairCells;
-    if (c->dtype == LAT_F16)
-        pair ? run(k_moments2d<__half, true>) : run(k_moments2d<__half>);
-    else if (c->dtype == LAT_BF16)
-        pair ? run(k_moments2d<__nv_bfloat16, true>) : run(k_moments2d<__nv_bfloat16>);
-    else if (c->dtype == LAT_F64)
-        run(k_moments2d<double>);
-    else
-        pair ? run(k_moments2d<float, true>) : run(k_moments2d<float>);
+    auto run_t = [&](auto t) {
+        using T = decltype(t);
+        if (form == kMomPair4) run(k_moments2d<T, kMomPair4>);
+        else if (form == kMomPair8) run(k_moments2d<T, kMomPair8>);
+        else if (form == kMomCell8) run(k_moments2d<T, kMomCell8>);
+        else run(k_moments2d<T, kMomCell>);
+    };
+    if (c->dtype == LAT_F16) run_t(__half());
+    else if (c->dtype == LAT_BF16) run_t(__nv_bfloat16());
+    else if (c->dtype == LAT_F32 && form == kMomPair7) run(k_moments2d<float, kMomPair7>);
+    else if (c->dtype == LAT_F32) run_t(float());
+    else if (form == kMomTile) run(k_moments2d<double, kMomTile>);
+    else run(k_moments2d<double, kMomCell>);
     CK2(cudaGetLastError());
-    k_finalize2d<<<1, kFin2DThreads, 0, s>>>(c->d_partials, c->mom_blocks,
+    k_finalize2d<<<1, kFin2DThreads, 0, s>>>(c->d_partials, blocks,
                                              c->dx * c->dx * c->dv * c->dv, c->d_glob);
     CK2(cudaGetLastError());
     return copy_globals(c, globals, wait, s);
