@@ -228,7 +228,7 @@ constexpr int kMultiT = 5;  // steps per launch of the several-steps kernel
 static_assert(kMultiT <= kFlowSteps, "their flow is formed in one launch");
 
 constexpr size_t kBasisBytes = 64u << 20;  // tables of the modes at most: see flow_rows
-constexpr long long kLimRestCells = 8 << 20;  // see enqueue_steps_1d
+constexpr long long kLimRestCells = 8 << 20, kLim17Cells = 300000;  // see enqueue_steps_1d
 constexpr int kMinTile = 64;  // narrower tiles are mostly margin
 
 int max_nx(const lat_ctx* c) {
@@ -421,7 +421,10 @@ int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
     }
     const bool rows = flow_rows(c);
     const bool multi = on_chip && rows && c->tiles[0].n;
-    const bool lim = !chosen && rows && c->scheme == LAT_SCHEME_KOREN && c->tiles[1].n;
+    // Few cells of N_v = 17 on the copy pipeline wait as long there as on the tiles, and need no flow
+    // launch (ten steps: 4096 columns 45 us, on the tiles 49; eight lattices of 3000 56 and 51).
+    const bool lim = !chosen && rows && c->scheme == LAT_SCHEME_KOREN && c->tiles[1].n &&
+                     !(c->nv == 17 && c->variant != STEP1D_PLAIN && c->total_x * c->nv < kLim17Cells);
     // The plain-load and the limited kernels take the flow from the flow kernel, kFlowSteps steps at
     // a time (evaluating the basis costs an FP64 column as much as half its sweep).  The launch is
     // not worth it for fewer FP32 steps (1000 instances of 601 columns, N_v = 33, one upwind step:
