@@ -42,10 +42,10 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
-// a - b lane by lane with scalar instructions (same rounding as sub2).  The packed 1D sweep
-// uses it for the difference of consecutive diffusion fluxes: with sub.rn.f32x2 there, the
-// kernels built by this toolchain differed from the scalar sweep by one unit in the last
-// place in a few cells, while every packed instruction on its own rounds exactly.
+// a - b lane by lane with scalar instructions (same rounding as sub2), for the difference of
+// consecutive diffusion fluxes of the packed 1D sweep: the toolchain contracts a packed product into
+// the packed add or subtract that takes it (one rounding less, other bits than the scalar sweep's).
+// Later kernels form such products as fma2(a, b, an opaque zero) instead, which costs nothing.
 __device__ __forceinline__ f2 sub2s(f2 a, f2 b) {
     return pk(__fsub_rn(lo(a), lo(b)), __fsub_rn(hi(a), hi(b)));
 }
@@ -77,6 +77,19 @@ __device__ __forceinline__ f2 lim_min2(f2 a, f2 b, f2 c) {
 __device__ __forceinline__ f2 opaque2(f2 v) {
     asm volatile("mov.b64 %0, %0;" : "+l"(v));
     return v;
+}
+// Koren's limiter in two lanes (lim_inc's value up to the sign of a zero).  zero2 is an opaque zero: a
+// product that only feeds a packed add or subtract is formed as fma2(a, b, zero2), which keeps the
+// toolchain from contracting it into that instruction (the scalar kernels round it).
+struct LimPair {
+    f2 mu2, third2, sixth2, zero2;
+};
+__device__ __forceinline__ LimPair lim_pair(float mu) {
+    return LimPair{pk(mu, mu), pk(float(1.0 / 3.0), float(1.0 / 3.0)),
+                   pk(float(1.0 / 6.0), float(1.0 / 6.0)), opaque2(0ull)};
+}
+__device__ __forceinline__ f2 lim_inc_x2(f2 dp, f2 dm, const LimPair& k) {
+    return lim_min2(dp, fma2(dm, k.sixth2, mul2(dp, k.third2)), mul2(k.mu2, dm));
 }
 
 }  // namespace lat

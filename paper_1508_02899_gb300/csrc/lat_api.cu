@@ -224,8 +224,6 @@ Step1DArgs step_args(const lat_ctx* c, int k, int dry) {
     return a;
 }
 
-constexpr int kMultiT = 5;  // steps per launch of the several-steps kernel
-static_assert(kMultiT <= kFlowSteps, "their flow is formed in one launch");
 
 constexpr size_t kBasisBytes = 64u << 20;  // tables of the modes at most: see flow_rows
 constexpr long long kLimRestCells = 8 << 20, kLim17Cells = 300000;  // see enqueue_steps_1d
@@ -238,7 +236,7 @@ int max_nx(const lat_ctx* c) {
 }
 
 int tile_places(const lat_ctx* c, bool lim, int w) {
-    return lim ? lim1d_places(w) : multi1d_places(c->nv, kMultiT, w);
+    return lim ? lim1d_places(w) : multi1d_places(c->nv, w);
 }
 
 // Instances are cut into equal tiles of at most w columns.
@@ -256,7 +254,7 @@ std::vector<MultiTile> make_tiles(const lat_ctx* c, bool lim, int* widest_places
     int places = 0, margin = 0;
     std::vector<MultiTile> tiles;
     if (c->dtype != LAT_F32 ||
-        !(lim ? lim1d_shape(c->nv, &places) : multi1d_shape(c->nv, kMultiT, &places, &margin)))
+        !(lim ? lim1d_shape(c->nv, &places) : multi1d_shape(c->nv, &places, &margin)))
         return tiles;
     const int wmax = (places - 2 * margin) / 8 * 8;
     const int held = lim ? 3 : 2;
@@ -394,7 +392,7 @@ double launches_us(const lat_ctx* c, int n) {
         return 8.0 + n * (2.7 + (compiled ? 0.36 : 0.58) * c->nv + 1.2e-5 * c->total_x * c->nv);
     const double step = compiled ? 2.7 + 0.06 * c->nv : 1.9 + 0.36 * c->nv;
     if (!(flow_rows(c) && c->tiles[0].n)) return 3.0 + n * step;
-    return 4.0 + n / kMultiT * (6.5 + 0.23 * c->nv) + n % kMultiT * step;
+    return 4.0 + n / kFlowSteps * (6.5 + 0.23 * c->nv) + n % kFlowSteps * step;
 }
 
 // Whether a batch of n steps runs on the cluster kernel of small lattices: where it is faster.  Ten steps
@@ -409,7 +407,7 @@ bool line_1d(const lat_ctx* c, int n) {
 }
 
 // Enqueue n steps of a 1D context on stream s (used directly and under capture).  Where no launch
-// shape was chosen: all of them in one launch for small lattices, kMultiT per launch where that
+// shape was chosen: all of them in one launch for small lattices, kFlowSteps per launch where that
 // kernel is built; else one by one.
 int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
     const bool chosen = c->pinned || c->mode == 1;
@@ -439,9 +437,9 @@ int enqueue_steps_1d(lat_ctx* c, int n, cudaStream_t s) {
     int formed = 0, first = 0;  // steps whose flow is formed, from step `first` on
     for (int k = 0, t; k < n; k += t) {
         Step1DArgs a = step_args(c, k, 0);
-        t = multi && n - k >= kMultiT ? kMultiT : 1;
+        t = multi && n - k >= kFlowSteps ? kFlowSteps : 1;
         if (t > 1) {
-            CK(launch_multi1d(c->nv, t, c->tiles[0].n, c->tiles[0].places, a, c->tiles[0].d, k,
+            CK(launch_multi1d(c->nv, c->tiles[0].n, c->tiles[0].places, a, c->tiles[0].d, k,
                               c->ring_ok ? 1 : 0, s));
             continue;
         }
@@ -823,8 +821,7 @@ int enqueue_moments(lat_ctx* c, double* rho, double* mean_v, double* mean_v2, do
     a.mean_v2 = mean_v2;
     a.partials = c->d_partials;
     a.st = c->d_state;
-    const int grid = std::max(1, c->nitems);
-    CK(launch_moments1d(c->dtype, tile_of(c), 1, grid, a, c->stream));
+    CK(launch_moments1d(c->dtype, tile_of(c), a, c->stream));
     return finalize_1d(c, tile_of(c) / 32, gdst, wait);
 }
 

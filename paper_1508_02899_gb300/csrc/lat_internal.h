@@ -86,7 +86,7 @@ struct Step1DArgs {
     // several steps per launch (multi1d.cu)
     const void* basis;           // (sin, cos) tables of the modes, one per grid size
     const long long* size_off;   // [n_inst] columns of the tables before the instance's
-    void* wflow;                 // [T][total_x] u / dv of the steps
+    void* wflow;                 // [kFlowSteps][total_x] u / dv of the steps
     const void* wpre;            // u / dv of this step's columns (a row of wflow), or null
     long long total_x;
     int nv, tile;                // N_v; columns per item
@@ -112,9 +112,11 @@ struct MultiTile {
     int nx, x0, w;
     float g, r;
 };
-// T = 5, 9, 13 .. steps per launch for the N_v it is built for: the places a tile may take with its
-// margins (w + 2 margin <= max_places); false where there is no kernel.
-bool multi1d_shape(int nv, int T, int* max_places, int* margin);
+// Steps of a launch of the several-steps kernel, and of the flow kernel at most.
+constexpr int kFlowSteps = 5;
+// For the N_v the several-steps kernel is built for: the places a tile may take with its margins
+// (w + 2 margin <= max_places); false where there is no kernel.
+bool multi1d_shape(int nv, int* max_places, int* margin);
 // One flux-limited step of every tile (lim1d.cu, FP32): columns of a tile at most, places (threads x 2)
 // of a tile of w columns; wrow the step's row of wflow.
 bool lim1d_shape(int nv, int* max_places);
@@ -133,15 +135,14 @@ cudaError_t launch_line1d(int dtype, int n_inst, int nx_max, int nv, const Step1
 // (sin, cos) of 2 pi k_m x / N_x, [m][x], from entry M size_off on.
 cudaError_t launch_flow_basis(int dtype, const Step1DArgs& a, const int* sizes, int n_sizes,
                               int nx_max, void* table, cudaStream_t s);
-// u / dv of steps kstep .. kstep + T - 1 into wflow (T <= kFlowSteps, odd: the amplitudes move to the
+// u / dv of steps kstep .. kstep + n - 1 into wflow (n <= kFlowSteps, odd: the amplitudes move to the
 // step after them, in the parity that no block reads).  One block per item.
-constexpr int kFlowSteps = 5;
-cudaError_t launch_flow_steps(int dtype, const Step1DArgs& a, int kstep, int T, cudaStream_t s);
+cudaError_t launch_flow_steps(int dtype, const Step1DArgs& a, int kstep, int n, cudaStream_t s);
 // Places of a tile of w columns.
-int multi1d_places(int nv, int T, int w);
-// Steps kstep .. kstep + T - 1 of every tile, each on `places` (the widest tile's).  piped: N_x and x0
+int multi1d_places(int nv, int w);
+// Steps kstep .. kstep + kFlowSteps - 1 of every tile, each on `places` (the widest tile's).  piped: N_x and x0
 // multiples of 4 throughout.
-cudaError_t launch_multi1d(int nv, int T, int ntiles, int places, const Step1DArgs& a,
+cudaError_t launch_multi1d(int nv, int ntiles, int places, const Step1DArgs& a,
                            const MultiTile* tiles, int kstep, int piped, cudaStream_t s);
 
 // Arguments of the moment kernels (1D).
@@ -170,8 +171,7 @@ int step1d_ring_occupancy(int nv, int slots, int variant);
 // One producer/consumer step (2 slots) that also writes the moments of the new state.
 cudaError_t launch_step1d_moments(int nv, int grid, const Step1DArgs& a, cudaStream_t s);
 bool step1d_moments_supported(int dtype, int nv);
-cudaError_t launch_moments1d(int dtype, int block, int tile_xpt, int grid, const Mom1DArgs& a,
-                             cudaStream_t s);
+cudaError_t launch_moments1d(int dtype, int block, const Mom1DArgs& a, cudaStream_t s);
 // Fold per-instance partials: instance i owns partials [per_item begin[i], per_item begin[i+1]).
 // Observables (observables.cu): <rho_r^2> and the Eulerian S1 from per-cell rho (FP64).
 cudaError_t launch_coarse1d(const double* rho, const Inst1D* inst, int n_inst, long long total_x,

@@ -33,14 +33,9 @@ constexpr int kChunk = 8;       // rows per pass of the loop
 constexpr int kPlaces = 256;    // columns of a tile at most
 constexpr int kPitch = kPlaces + 4;
 
-struct LimConst {
-    f2 g2, r2, mu2, third2, sixth2, half2, one2, zero2;
+struct LimConst : LimPair {
+    f2 g2, r2, half2, one2;
 };
-
-// psi(theta) dp in two lanes (lim_inc)
-__device__ __forceinline__ f2 inc2(f2 dp, f2 dm, const LimConst& k) {
-    return lim_min2(dp, fma2(dm, k.sixth2, mul2(dp, k.third2)), mul2(k.mu2, dm));
-}
 
 enum { kBoth = 0, kPos = 1, kNeg = 2 };
 
@@ -57,7 +52,7 @@ __device__ __forceinline__ f2 face(Split& s, f2 ca, f2 v, const LimConst& k) {
     f2 F = 0ull;
     if (SIGN != kNeg) {
         const f2 d = sub2(s.P2, s.P1);
-        F = add2(s.P1, inc2(d, s.dP, k));
+        F = add2(s.P1, lim_inc_x2(d, s.dP, k));
         s.P1 = s.P2;
         s.dP = d;
         s.P2 = fma2(SIGN == kPos ? ca : max0(ca), v, k.zero2);
@@ -65,7 +60,7 @@ __device__ __forceinline__ f2 face(Split& s, f2 ca, f2 v, const LimConst& k) {
     if (SIGN != kPos) {
         const f2 M3 = fma2(SIGN == kNeg ? ca : min0(ca), v, k.zero2);
         const f2 d = sub2(s.M2, M3);
-        const f2 n = add2(s.M2, inc2(s.dM, d, k));
+        const f2 n = add2(s.M2, lim_inc_x2(s.dM, d, k));
         F = SIGN == kNeg ? n : add2(F, n);
         s.M2 = M3;
         s.dM = d;
@@ -143,12 +138,9 @@ __device__ __forceinline__ void sweep(const float* p, f2 w2, float g, float r, f
     LimConst k;
     k.g2 = pk(g, g);
     k.r2 = pk(r, r);
-    k.mu2 = pk(mu, mu);
-    k.third2 = pk(float(1.0 / 3.0), float(1.0 / 3.0));
-    k.sixth2 = pk(float(1.0 / 6.0), float(1.0 / 6.0));
+    static_cast<LimPair&>(k) = lim_pair(mu);
     k.half2 = pk(0.5f, 0.5f);
     k.one2 = opaque2(pk(1.f, 1.f));
-    k.zero2 = opaque2(0ull);
     // rows up to kp have c a >= 0 in every column of the warp, rows from kn on c a <= 0
     const float wlo = min_nan(lo(w2), hi(w2)), whi = max_nan(lo(w2), hi(w2));
     const bool sane = fabsf(wlo) < 1e6f && fabsf(whi) < 1e6f;  // false for NaN

@@ -599,22 +599,11 @@ __device__ __forceinline__ f2 ld2s(const float* p) { return *reinterpret_cast<co
 __device__ __forceinline__ void st2s(float* p, f2 v) { *reinterpret_cast<f2*>(p) = v; }
 __device__ __forceinline__ f2 splat(float a) { return pk(a, a); }
 
-// Limiter constants of a pair; zero2 is an opaque zero: a product that only feeds a packed add or
-// subtract is formed as fma2(a, b, zero2), which keeps it from being contracted into that
-// instruction (the scalar kernel rounds it).
-struct LimPair {
-    f2 mu2, third2, sixth2, zero2;
-};
-
-// lim_inc2<float> lane by lane (up to the sign of a zero)
-__device__ __forceinline__ f2 lim_inc2_x2(f2 dp, f2 dm, const LimPair& k) {
-    return lim_min2(dp, fma2(dm, k.sixth2, mul2(dp, k.third2)), mul2(k.mu2, dm));
-}
 __device__ __forceinline__ f2 pos_part_x2(f2 P0, f2 P1, f2 P2, const LimPair& k) {
-    return add2(P1, lim_inc2_x2(sub2(P2, P1), sub2(P1, P0), k));
+    return add2(P1, lim_inc_x2(sub2(P2, P1), sub2(P1, P0), k));
 }
 __device__ __forceinline__ f2 neg_part_x2(f2 M1, f2 M2, f2 M3, const LimPair& k) {
-    return add2(M2, lim_inc2_x2(sub2(M1, M2), sub2(M2, M3), k));
+    return add2(M2, lim_inc_x2(sub2(M1, M2), sub2(M2, M3), k));
 }
 __device__ __forceinline__ f2 face_parts_x2(int kind, f2 P0, f2 P1, f2 P2, f2 M1, f2 M2, f2 M3,
                                             const LimPair& k) {
@@ -762,7 +751,7 @@ __global__ void __launch_bounds__(LimPacked<NV, TC>::kThreads, MINB)
     const float g = (float)a.g, mu = (float)a.mu, inv_dv = (float)a.inv_dv;
     const float cflf = O::mul(g, O::add(1.f, mu));
     const f2 g2 = splat(g), r2 = splat((float)a.r);
-    const LimPair lk{splat(mu), splat((float)(1.0 / 3.0)), splat((float)(1.0 / 6.0)), opaque2(0ull)};
+    const LimPair lk = lim_pair(mu);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = 2 * (lane % L::LPC);
     const int jx_raw = warp * L::CPW + lane / L::LPC;

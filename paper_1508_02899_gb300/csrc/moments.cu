@@ -20,8 +20,7 @@ using namespace cs;
 
 constexpr int kMomRows = 8;
 
-// One block (one thread per column of a work item's tile, blockDim = tile width) per item,
-// grid-stride over items.  Every warp writes one partial per item: partials[item][warp][6].
+// One block (one thread per column of a work item's tile, blockDim = tile width) per item.  Every warp writes one partial per item: partials[item][warp][6].
 //  FP32 storage: column sums in FP32 (ColumnSums: mass compensated, weights j, j^2 by FMA),
 //    cross-column sums per warp in FP32 compensated form, FP64 from the warp partials on (FP64
 //    is slow here).
@@ -31,106 +30,104 @@ constexpr int kMomRows = 8;
 // with loads paired with their sums, eight blocks per SM walking the items and lane 0 scaling all
 // three sums.
 template <typename T>
-__global__ void __launch_bounds__(1024) k_moments1d(const Mom1DArgs a, const int xpt) {
+__global__ void __launch_bounds__(1024) k_moments1d(const Mom1DArgs a) {
     const int nv = a.nv;
     const int J = (nv - 1) / 2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
-    for (int it = blockIdx.x; it < a.nitems; it += gridDim.x) {
-        const int2 item = a.items[it];
-        const Inst1D in = a.inst[item.x];
-        const T* f = static_cast<const T*>(a.f) + in.off;
-        const int x = item.y + threadIdx.x;
-        const bool on = x < in.nx;
-        bool bad = false;
-        double* p = a.partials + ((size_t)it * nwarps + warp) * 6;
-        (void)xpt;
-        if (sizeof(T) == sizeof(double)) {
-            Comp s0{0, 0}, s1{0, 0}, s2{0, 0};
-            if (on) {
+    const int it = blockIdx.x;
+    const int2 item = a.items[it];
+    const Inst1D in = a.inst[item.x];
+    const T* f = static_cast<const T*>(a.f) + in.off;
+    const int x = item.y + threadIdx.x;
+    const bool on = x < in.nx;
+    bool bad = false;
+    double* p = a.partials + ((size_t)it * nwarps + warp) * 6;
+    if (sizeof(T) == sizeof(double)) {
+        Comp s0{0, 0}, s1{0, 0}, s2{0, 0};
+        if (on) {
 #pragma unroll 4
-                for (int jj = 0; jj < nv; ++jj) {
-                    const double v = __dmul_rn((double)(jj - J), in.dv);
-                    const double fv = (double)f[(size_t)jj * in.nx + x];
-                    bad |= !isfinite(fv);
-                    nadd(s0, fv);
-                    nadd(s1, __dmul_rn(v, fv));
-                    nadd(s2, __dmul_rn(__dmul_rn(v, v), fv));
-                }
-                const double m0 = nval(s0), m1 = nval(s1), m2 = nval(s2);
-                const long long cell = in.xoff + x;
-                if (a.rho) a.rho[cell] = m0 * in.dv;
-                if (a.mean_v) a.mean_v[cell] = (m0 != 0.0) ? m1 / m0 : 0.0;
-                if (a.mean_v2) a.mean_v2[cell] = (m0 != 0.0) ? m2 / m0 : 0.0;
+            for (int jj = 0; jj < nv; ++jj) {
+                const double v = __dmul_rn((double)(jj - J), in.dv);
+                const double fv = (double)f[(size_t)jj * in.nx + x];
+                bad |= !isfinite(fv);
+                nadd(s0, fv);
+                nadd(s1, __dmul_rn(v, fv));
+                nadd(s2, __dmul_rn(__dmul_rn(v, v), fv));
             }
-            warp_reduce3(s0, s1, s2);
-            if (lane == 0) {
-                p[0] = s0.s; p[1] = s0.c;
-                p[2] = s1.s; p[3] = s1.c;
-                p[4] = s2.s; p[5] = s2.c;
-            }
-        } else {
-            ColumnSums sums;
-            if (on && nv >= 5) {
-                // two half-columns, as the fused step epilogue sums them (ColumnSums2)
-                // kMomRows pairs of rows are read before the first is summed: as many loads are
-                // in flight as a column's sums leave registers for.  A value that is not finite
-                // makes z NaN.
-                ColumnSums2 s2;
-                const f2 one2 = pk(1.f, 1.f), zero2 = opaque2(0ull);
-                f2 jv = pk((float)-J, 0.f), z = zero2;
-                const float* r0 = reinterpret_cast<const float*>(f) + x;
-                const float* r1 = r0 + (size_t)J * in.nx;
-                auto add = [&](f2 v) {
-                    z = fma2(v, zero2, z);
-                    s2.add(jv, mul2(jv, jv), v);
-                    jv = add2(jv, one2);
-                };
-                int p = 0;
-                for (; p + kMomRows <= J; p += kMomRows) {
-                    float v0[kMomRows], v1[kMomRows];
+            const double m0 = nval(s0), m1 = nval(s1), m2 = nval(s2);
+            const long long cell = in.xoff + x;
+            if (a.rho) a.rho[cell] = m0 * in.dv;
+            if (a.mean_v) a.mean_v[cell] = (m0 != 0.0) ? m1 / m0 : 0.0;
+            if (a.mean_v2) a.mean_v2[cell] = (m0 != 0.0) ? m2 / m0 : 0.0;
+        }
+        warp_reduce3(s0, s1, s2);
+        if (lane == 0) {
+            p[0] = s0.s; p[1] = s0.c;
+            p[2] = s1.s; p[3] = s1.c;
+            p[4] = s2.s; p[5] = s2.c;
+        }
+    } else {
+        ColumnSums sums;
+        if (on && nv >= 5) {
+            // two half-columns, as the fused step epilogue sums them (ColumnSums2)
+            // kMomRows pairs of rows are read before the first is summed: as many loads are
+            // in flight as a column's sums leave registers for.  A value that is not finite
+            // makes z NaN.
+            ColumnSums2 s2;
+            const f2 one2 = pk(1.f, 1.f), zero2 = opaque2(0ull);
+            f2 jv = pk((float)-J, 0.f), z = zero2;
+            const float* r0 = reinterpret_cast<const float*>(f) + x;
+            const float* r1 = r0 + (size_t)J * in.nx;
+            auto add = [&](f2 v) {
+                z = fma2(v, zero2, z);
+                s2.add(jv, mul2(jv, jv), v);
+                jv = add2(jv, one2);
+            };
+            int p = 0;
+            for (; p + kMomRows <= J; p += kMomRows) {
+                float v0[kMomRows], v1[kMomRows];
 #pragma unroll
-                    for (int q = 0; q < kMomRows; ++q) {
-                        v0[q] = __ldg(r0);
-                        v1[q] = __ldg(r1);
-                        r0 += in.nx;
-                        r1 += in.nx;
-                    }
-#pragma unroll
-                    for (int q = 0; q < kMomRows; ++q) add(pk(v0[q], v1[q]));
-                }
-                const float fl = __ldg(r0 + (size_t)(nv - 1 - p) * in.nx);
-#pragma unroll 4
-                for (; p < J; ++p) {
-                    add(pk(__ldg(r0), __ldg(r1)));
+                for (int q = 0; q < kMomRows; ++q) {
+                    v0[q] = __ldg(r0);
+                    v1[q] = __ldg(r1);
                     r0 += in.nx;
                     r1 += in.nx;
                 }
-                bad = !isfinite(fl) || lo(z) != 0.f || hi(z) != 0.f;
-                s2.add_hi((float)J, fl);
-                sums = s2.collapse();
-            } else if (on) {
-                for (int jj = 0; jj < nv; ++jj) {
-                    const float fv = (float)f[(size_t)jj * in.nx + x];
-                    bad |= !isfinite(fv);
-                    sums.add((float)(jj - J), fv);
-                }
+#pragma unroll
+                for (int q = 0; q < kMomRows; ++q) add(pk(v0[q], v1[q]));
             }
-            if (on) {
-                if (a.rho || a.mean_v || a.mean_v2) {  // FP64 per cell only when asked for
-                    Comp s0, s1, s2;
-                    sums.result(in.dv, s0, s1, s2);
-                    const double m0 = nval(s0);
-                    const long long cell = in.xoff + x;
-                    if (a.rho) a.rho[cell] = m0 * in.dv;
-                    if (a.mean_v) a.mean_v[cell] = (m0 != 0.0) ? s1.s / m0 : 0.0;
-                    if (a.mean_v2) a.mean_v2[cell] = (m0 != 0.0) ? s2.s / m0 : 0.0;
-                }
+            const float fl = __ldg(r0 + (size_t)(nv - 1 - p) * in.nx);
+#pragma unroll 4
+            for (; p < J; ++p) {
+                add(pk(__ldg(r0), __ldg(r1)));
+                r0 += in.nx;
+                r1 += in.nx;
             }
-            warp_partial_1d(sums, in.dv, p);
+            bad = !isfinite(fl) || lo(z) != 0.f || hi(z) != 0.f;
+            s2.add_hi((float)J, fl);
+            sums = s2.collapse();
+        } else if (on) {
+            for (int jj = 0; jj < nv; ++jj) {
+                const float fv = (float)f[(size_t)jj * in.nx + x];
+                bad |= !isfinite(fv);
+                sums.add((float)(jj - J), fv);
+            }
         }
-        if (bad) atomicOr(&a.st->status, ST_NUMERIC);
+        if (on) {
+            if (a.rho || a.mean_v || a.mean_v2) {  // FP64 per cell only when asked for
+                Comp s0, s1, s2;
+                sums.result(in.dv, s0, s1, s2);
+                const double m0 = nval(s0);
+                const long long cell = in.xoff + x;
+                if (a.rho) a.rho[cell] = m0 * in.dv;
+                if (a.mean_v) a.mean_v[cell] = (m0 != 0.0) ? s1.s / m0 : 0.0;
+                if (a.mean_v2) a.mean_v2[cell] = (m0 != 0.0) ? s2.s / m0 : 0.0;
+            }
+        }
+        warp_partial_1d(sums, in.dv, p);
     }
+    if (bad) atomicOr(&a.st->status, ST_NUMERIC);
 }
 
 // Eight lanes per instance (four instances per warp) fold that instance's partials (per_item
@@ -261,11 +258,10 @@ int noalloc_scratch(double** out) {
 
 }  // namespace
 
-cudaError_t launch_moments1d(int dtype, int block, int xpt, int grid, const Mom1DArgs& a,
-                             cudaStream_t s) {
-    if (grid <= 0) return cudaSuccess;
-    if (dtype == LAT_F32) k_moments1d<float><<<grid, block, 0, s>>>(a, xpt);
-    else if (dtype == LAT_F64) k_moments1d<double><<<grid, block, 0, s>>>(a, xpt);
+cudaError_t launch_moments1d(int dtype, int block, const Mom1DArgs& a, cudaStream_t s) {
+    if (a.nitems <= 0) return cudaSuccess;
+    if (dtype == LAT_F32) k_moments1d<float><<<a.nitems, block, 0, s>>>(a);
+    else if (dtype == LAT_F64) k_moments1d<double><<<a.nitems, block, 0, s>>>(a);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }

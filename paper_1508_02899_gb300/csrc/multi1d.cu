@@ -52,26 +52,26 @@ constexpr int kCols = 64;   // columns of a warp: lane l takes c0 + l and c0 + 3
 constexpr int kChunk = 8;   // velocity rows per pass of the sweep's loop
 constexpr int kSmemWords = 113 * 1024 / 4;
 constexpr int kMaxPlaces = 512;
+constexpr int T = kFlowSteps;  // steps per launch
+static_assert(T % 4 == 1, "odd: from one buffer to the other; and the shifts of Shape");
 constexpr int round_up(int v, int n) { return (v + n - 1) / n * n; }
-constexpr int margin_of(int T) { return round_up(kReach * T * (T - 1) / 2, 4); }
+constexpr int kMargin = round_up(kReach * T * (T - 1) / 2, 4);
 // Words besides the planes: the copies' mbarrier and u / dv of every step's columns.
-constexpr int side_words(int J, int T, int P) { return 4 + T * P + J * T * (T - 1); }
+constexpr int side_words(int J, int P) { return 4 + T * P + J * T * (T - 1); }
 
 // Shape of the kernel for N_v.  Two blocks per SM (one loads while the other computes), so at most
-// about 113 KB each; the pitch of the plane rows is the largest for T = 5.
+// about 113 KB each.
 template <int NV>
 struct Shape {
     static constexpr int J = (NV - 1) / 2;
-    static constexpr int kFit = (kSmemWords - 4 * NV - side_words(J, 5, 0)) / (NV + 5) / kCols * kCols;
+    static constexpr int kFit = (kSmemWords - 4 * NV - side_words(J, 0)) / (NV + T) / kCols * kCols;
     static constexpr int kPitch = (kFit < kMaxPlaces ? kFit : kMaxPlaces) + 4;
     static_assert((NV - 1) % kChunk == 0 && J % 4 == 0, "whole chunks, one pattern of shifts");
     // offset of plane row jj's window in its row: the 16-byte rounding of column x0 - m - j T
     // (T = 1 modulo 4)
     __host__ __device__ static constexpr int shift(int jj) { return (J - jj) & 3; }
-    static constexpr int max_places(int T) {
-        const int p = (kSmemWords - NV * kPitch - side_words(J, T, 0)) / T;
-        return (p < kPitch - 4 ? p : kPitch - 4) / kCols * kCols;
-    }
+    static constexpr int kPlaces = kPitch - 4;  // of a tile at most
+    static_assert(NV * kPitch + side_words(J, kPlaces) <= kSmemWords, "two blocks per SM");
 };
 
 // ---- the sweep of two columns ------------------------------------------------------------------
@@ -271,16 +271,15 @@ __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
 
 template <int NV>
 __global__ void __launch_bounds__(kMaxPlaces / 2, 2)
-    k_multi1d(const Step1DArgs a, const MultiTile* tiles, int kstep, int T, int piped) {
+    k_multi1d(const Step1DArgs a, const MultiTile* tiles, int kstep, int piped) {
     using S = Shape<NV>;
     constexpr int J = S::J, PT = S::kPitch;
     extern __shared__ __align__(128) unsigned char smem[];
-    const int margin = margin_of(T);
     float* f = reinterpret_cast<float*>(smem);
     float* U = f + (size_t)NV * PT;  // rows of P + 2 J d: the columns -J d .. P + J d - 1 of a step
     uint64_t* bar = reinterpret_cast<uint64_t*>(U + T * 2 * blockDim.x + J * T * (T - 1));
     const MultiTile tile = tiles[blockIdx.x];
-    const int nx = tile.nx, P = 2 * blockDim.x, first = tile.x0 - margin;
+    const int nx = tile.nx, P = 2 * blockDim.x, first = tile.x0 - kMargin;
     const long long step = a.st->step + kstep;
     const int par = (int)(step & 1);
     const float* fin = static_cast<const float*>(par ? a.f[1] : a.f[0]) + tile.off;
@@ -346,6 +345,7 @@ __global__ void __launch_bounds__(kMaxPlaces / 2, 2)
     // all steps but the last, in place
     const float* Us = U;
     const int c0 = (tid >> 5) * kCols;
+#pragma unroll 1
     for (int d = T - 1; d > 0; --d) {
         Us += J * d;
         const Put<false> put{nullptr, 0, true, true};
@@ -354,27 +354,25 @@ __global__ void __launch_bounds__(kMaxPlaces / 2, 2)
         __syncthreads();
     }
     // the last step: every place is its column, and the outputs go to the other buffer
-    const int c = c0 + (tid & 31) - margin;
+    const int c = c0 + (tid & 31) - kMargin;
     sweep2<NV, false>(f, Us, c0, 0, P, tile.g, tile.r,
                       Put<true>{fout + tile.x0 + c, nx, c >= 0 && c < tile.w,
                                 c + 32 >= 0 && c + 32 < tile.w});
 }
 
-// u / dv of every column at the T steps, W[step][column], one block per tile of columns; the
+// u / dv of every column at the n <= T steps, W[step][column], one block per tile of columns; the
 // instance's first tile also advances the amplitudes to the step after them.  The basis comes from
 // tables (one per grid size, flow_basis's values): evaluated per column and step, as the one-step
 // kernels do, the eight sincospi would cost as much as a fifth of the sweeps.
-constexpr int kFlowGroup = 5;  // steps formed together
 template <typename F> struct Pair;
 template <> struct Pair<float> { using type = float2; };
 template <> struct Pair<double> { using type = double2; };
 
 template <typename F>
-__global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kstep, int T) {
+__global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kstep, int n) {
     using F2 = typename Pair<F>::type;
     extern __shared__ double2 amp_raw[];
-    F* amp = reinterpret_cast<F*>(amp_raw);  // [M][2 T], T in whole groups: A, B of each step
-    const int Tg = round_up(T, kFlowGroup);
+    F* amp = reinterpret_cast<F*>(amp_raw);  // [M][T][A, B]
     const int2 item = a.items[blockIdx.x];
     const Inst1D& in = a.inst[item.x];
     const int nx = in.nx, tid = threadIdx.x;
@@ -384,25 +382,22 @@ __global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kste
     if (tid < 2 * M) {
         const long long at = (long long)item.x * 2 * M + tid;
         double v = a.amp[par * a.amp_stride + at];
-        F* row_q = amp + (tid < M ? tid : tid - M) * 2 * Tg + (tid < M ? 0 : 1);
+        F* row_q = amp + (tid < M ? tid : tid - M) * 2 * T + (tid < M ? 0 : 1);
         const long long row0 = step - a.st->noise_base, rows = a.st->noise_rows;
         const double e = in.ou_e, sg = in.ou_s;
         bool missing = false;
-#pragma unroll 1
-        for (int s0 = 0; s0 < T; s0 += kFlowGroup) {
-            double xi[kFlowGroup];
+        double xi[T];
 #pragma unroll
-            for (int s = 0; s < kFlowGroup; ++s) {
-                const long long row = row0 + s0 + s;
-                const bool have = !a.frozen && s0 + s < T && row >= 0 && row < rows;
-                missing |= !have && s0 + s < T;
-                xi[s] = have ? a.noise[row * a.amp_stride + at] : 0.0;
-            }
+        for (int s = 0; s < T; ++s) {
+            const long long row = row0 + s;
+            const bool have = !a.frozen && s < n && row >= 0 && row < rows;
+            missing |= !have && s < n;
+            xi[s] = have ? a.noise[row * a.amp_stride + at] : 0.0;
+        }
 #pragma unroll
-            for (int s = 0; s < kFlowGroup; ++s) {
-                row_q[2 * (s0 + s)] = F(v);
-                if (!a.frozen && s0 + s < T) v = __dadd_rn(__dmul_rn(v, e), __dmul_rn(sg, xi[s]));
-            }
+        for (int s = 0; s < T; ++s) {
+            row_q[2 * s] = F(v);
+            if (!a.frozen && s < n) v = __dadd_rn(__dmul_rn(v, e), __dmul_rn(sg, xi[s]));
         }
         if (!a.frozen && item.y == 0) {
             a.amp_w[(1 - par) * a.amp_stride + at] = v;
@@ -418,57 +413,39 @@ __global__ void __launch_bounds__(256) k_flow_steps(const Step1DArgs a, int kste
     for (int x = item.y + tid; x < min(nx, item.y + a.tile); x += blockDim.x) {
         const F2* basis = static_cast<const F2*>(a.basis) + M * a.size_off[item.x] + x;
         F* w = static_cast<F*>(a.wflow) + in.xoff + x;
-#pragma unroll 1
-        for (int s0 = 0; s0 < T; s0 += kFlowGroup) {
-            F u[kFlowGroup];
-            const F v = a.flow_kind == LAT_FLOW_FIELD
-                                ? static_cast<const F*>(a.field)[in.xoff + x]
-                            : F(0);
+        F u[T];
+        const F v =
+            a.flow_kind == LAT_FLOW_FIELD ? static_cast<const F*>(a.field)[in.xoff + x] : F(0);
 #pragma unroll
-            for (int s = 0; s < kFlowGroup; ++s) u[s] = v;
+        for (int s = 0; s < T; ++s) u[s] = v;
 #pragma unroll 8
-            for (int m = 0; m < M; ++m) {
-                const F2 sc = __ldg(basis + (size_t)m * nx);
-                const F2* ab = reinterpret_cast<const F2*>(amp + m * 2 * Tg) + s0;
+        for (int m = 0; m < M; ++m) {
+            const F2 sc = __ldg(basis + (size_t)m * nx);
+            const F2* ab = reinterpret_cast<const F2*>(amp + m * 2 * T);
 #pragma unroll
-                for (int s = 0; s < kFlowGroup; ++s)
-                    u[s] = flow_add<F>(u[s], ab[s].x, ab[s].y, sc.x, sc.y);
-            }
+            for (int s = 0; s < T; ++s) u[s] = flow_add<F>(u[s], ab[s].x, ab[s].y, sc.x, sc.y);
+        }
 #pragma unroll
-            for (int s = 0; s < kFlowGroup; ++s) {
-                if (s0 + s >= T) break;
-                const F ws = u[s] * inv_dv;
-                w[(s0 + s) * a.total_x] = ws;
-                cfl |= cf * (g * (J + fabs(ws))) > F(1);
-            }
+        for (int s = 0; s < T; ++s) {
+            if (s >= n) break;
+            const F ws = u[s] * inv_dv;
+            w[s * a.total_x] = ws;
+            cfl |= cf * (g * (J + fabs(ws))) > F(1);
         }
     }
     if (cfl) atomicOr(&a.st->status, ST_CFL);
 }
 
-}  // namespace
-
-cudaError_t launch_flow_steps(int dtype, const Step1DArgs& a, int kstep, int T, cudaStream_t s) {
-    const int M = a.flow_kind == LAT_FLOW_MODES ? a.nmodes : 0;
-    const int words = 2 * M * round_up(T, kFlowGroup), threads = std::min(256, a.tile);
-    if (dtype == LAT_F64)
-        k_flow_steps<double><<<a.item_end, threads, sizeof(double) * words, s>>>(a, kstep, T);
-    else k_flow_steps<float><<<a.item_end, threads, sizeof(float) * words, s>>>(a, kstep, T);
-    return cudaGetLastError();
-}
-
-namespace {
-
 template <int NV>
-cudaError_t launch_t(int T, int ntiles, int places, const Step1DArgs& a, const MultiTile* tiles,
-                     int kstep, int piped, cudaStream_t s) {
+cudaError_t launch_t(int ntiles, int places, const Step1DArgs& a, const MultiTile* tiles, int kstep,
+                     int piped, cudaStream_t s) {
     static PerDevice limit;
     cudaError_t e = raise_smem(limit, k_multi1d<NV>, 4 * kSmemWords);
     if (e != cudaSuccess) return e;
     e = launch_flow_steps(LAT_F32, a, kstep, T, s);
     if (e != cudaSuccess) return e;
-    const size_t smem = 4 * ((size_t)NV * Shape<NV>::kPitch + side_words(Shape<NV>::J, T, places));
-    k_multi1d<NV><<<ntiles, places / 2, smem, s>>>(a, tiles, kstep, T, piped);
+    const size_t smem = 4 * ((size_t)NV * Shape<NV>::kPitch + side_words(Shape<NV>::J, places));
+    k_multi1d<NV><<<ntiles, places / 2, smem, s>>>(a, tiles, kstep, piped);
     return cudaGetLastError();
 }
 
@@ -476,25 +453,33 @@ cudaError_t launch_t(int T, int ntiles, int places, const Step1DArgs& a, const M
 
 }  // namespace
 
-bool multi1d_shape(int nv, int T, int* max_places, int* margin) {
-    if (T < 5 || T % 4 != 1) return false;
-    *margin = margin_of(T);
+cudaError_t launch_flow_steps(int dtype, const Step1DArgs& a, int kstep, int n, cudaStream_t s) {
+    const int M = a.flow_kind == LAT_FLOW_MODES ? a.nmodes : 0;
+    const int words = 2 * M * T, threads = std::min(256, a.tile);
+    if (dtype == LAT_F64)
+        k_flow_steps<double><<<a.item_end, threads, sizeof(double) * words, s>>>(a, kstep, n);
+    else k_flow_steps<float><<<a.item_end, threads, sizeof(float) * words, s>>>(a, kstep, n);
+    return cudaGetLastError();
+}
+
+bool multi1d_shape(int nv, int* max_places, int* margin) {
+    *margin = kMargin;
     switch (nv) {
-#define X(n)     case n: *max_places = Shape<n>::max_places(T); return true;
+#define X(n)     case n: *max_places = Shape<n>::kPlaces; return true;
         MULTI_NV_LIST(X)
 #undef X
         default: return false;
     }
 }
 
-int multi1d_places(int nv, int T, int w) {
-    return round_up(std::max(w + 2 * margin_of(T), (nv - 1) * (T - 1) + kCols), kCols);
+int multi1d_places(int nv, int w) {
+    return round_up(std::max(w + 2 * kMargin, (nv - 1) * (T - 1) + kCols), kCols);
 }
 
-cudaError_t launch_multi1d(int nv, int T, int ntiles, int places, const Step1DArgs& a,
+cudaError_t launch_multi1d(int nv, int ntiles, int places, const Step1DArgs& a,
                            const MultiTile* tiles, int kstep, int piped, cudaStream_t s) {
     switch (nv) {
-#define X(n)     case n: return launch_t<n>(T, ntiles, places, a, tiles, kstep, piped, s);
+#define X(n)     case n: return launch_t<n>(ntiles, places, a, tiles, kstep, piped, s);
         MULTI_NV_LIST(X)
 #undef X
         default: return cudaErrorInvalidValue;

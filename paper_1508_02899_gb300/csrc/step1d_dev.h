@@ -1,4 +1,4 @@
-// Device code shared by the 1D step kernels (included by step1d.cu and multi1d.cu only): the column
+// Device code shared by the 1D step kernels (step1d.cu, multi1d.cu, lim1d.cu, line1d.cu): the column
 // arithmetic of both drag schemes, the flow evaluation and the amplitude update, and PTX wrappers
 // for mbarriers and bulk asynchronous copies.
 #pragma once

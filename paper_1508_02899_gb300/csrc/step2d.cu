@@ -2034,6 +2034,8 @@ int ctx2d_autotune(Ctx2D* c, void* const f[2], int reps, double* best, cudaStrea
             const int occ = c->half ? occupancy_step2d_h(c->dtype, c->nv, c->pcv)
                                     : occupancy_ring(c->nv, c->chunks, c->pcv);
             if (c->ring && bps > occ) continue;
+            if (bps > 1 && c->dtype == LAT_F64 && step2d_f64_tiles(c->nv, c->nx, c->ny, c->sm_count))
+                break;  // one launch shape
             int rc = enqueue2d(c, f, 1, s, 1);
             if (rc != LAT_OK) return rc;
             CK2(cudaEventRecord(e0, s));
