@@ -33,6 +33,7 @@ struct TileSet {
 }  // namespace
 
 struct lat_ctx {
+    Uploads up;
     int d = 1;
     int dtype = LAT_F32;
     int nv = 0;
@@ -162,9 +163,9 @@ int build_items(lat_ctx* c) {
                    sizeof(double) * 6 * std::max(kPcConsumerWarps, tile / 32) * items.size()) !=
             cudaSuccess)
         return LAT_ENOMEM;
-    CK(upload(c->d_items, items.data(), sizeof(int2) * items.size(), c->stream));
-    CK(upload(c->d_inst_begin, c->h_inst_begin.data(), sizeof(int) * (c->n_inst + 1),
-              c->stream));
+    CK(c->up.copy(c->d_items, items.data(), sizeof(int2) * items.size(), c->stream));
+    CK(c->up.copy(c->d_inst_begin, c->h_inst_begin.data(), sizeof(int) * (c->n_inst + 1),
+                  c->stream));
     drop_graphs(c);
     return LAT_OK;
 }
@@ -346,7 +347,7 @@ int build_plan(lat_ctx* c) {
     c->d_size_off = reinterpret_cast<long long*>(put(off.data(), bo));
     c->d_sizes = reinterpret_cast<int*>(put(sizes.data(), bs));
     c->n_sizes = (int)sizes.size();
-    CK(upload(c->d_plan, image.data(), image.size(), c->stream));
+    CK(c->up.copy(c->d_plan, image.data(), image.size(), c->stream));
     return LAT_OK;
 }
 
@@ -566,7 +567,7 @@ int lat_ensemble_init(lat_ctx** out, int n_inst, const lat_instance* inst, int n
     if (rc == LAT_OK && cudaMallocHost(&c->h_glob, sizeof(double) * 4 * n_inst) != cudaSuccess)
         rc = LAT_ENOMEM;
     if (rc == LAT_OK &&
-        upload(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * n_inst, c->stream) != cudaSuccess)
+        c->up.copy(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * n_inst, c->stream) != cudaSuccess)
         rc = LAT_ECUDA;
     if (rc == LAT_OK) {
         // default launch shape: the producer/consumer bulk-copy pipeline where every instance
@@ -666,10 +667,10 @@ int lat_set_flow(lat_ctx* c, const lat_flow* fl) {
         }
         // both parities start from amp0 so that a frozen flow reads the same values every step
         std::vector<float> a32(fl->amp0, fl->amp0 + stride);
-        CK(upload(amp, fl->amp0, sizeof(double) * stride, c->stream));
-        CK(upload(amp + stride, fl->amp0, sizeof(double) * stride, c->stream));
-        CK(upload(ampf, a32.data(), sizeof(float) * stride, c->stream));
-        CK(upload(ampf + stride, a32.data(), sizeof(float) * stride, c->stream));
+        CK(c->up.copy(amp, fl->amp0, sizeof(double) * stride, c->stream));
+        CK(c->up.copy(amp + stride, fl->amp0, sizeof(double) * stride, c->stream));
+        CK(c->up.copy(ampf, a32.data(), sizeof(float) * stride, c->stream));
+        CK(c->up.copy(ampf + stride, a32.data(), sizeof(float) * stride, c->stream));
         if (c->d_amp) cudaFree(c->d_amp);
         if (c->d_ampf) cudaFree(c->d_ampf);
         c->d_amp = amp;
@@ -690,7 +691,7 @@ int lat_set_flow(lat_ctx* c, const lat_flow* fl) {
                 q.ou_s = fl->sigma * sqrt(1.0 - q.ou_e * q.ou_e);
             }
         }
-        CK(upload(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * c->n_inst, c->stream));
+        CK(c->up.copy(c->d_inst, c->h_inst.data(), sizeof(Inst1D) * c->n_inst, c->stream));
     } else {
         return LAT_EINVAL;
     }

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <list>
 #include <map>
 #include <vector>
 
@@ -18,13 +19,30 @@
 
 namespace lat {
 
-// A host array into a device table that kernels of stream s read, done on return.  Always on the
-// context's own stream: a copy from pageable memory on the default stream may return before its last
-// transfer is done, and a non-blocking stream (such as PyTorch's) does not wait for that one.
-inline cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t s) {
-    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
-    return e != cudaSuccess ? e : cudaStreamSynchronize(s);
-}
+// Host arrays into device tables that kernels of a context's stream read, without waiting.  Always on
+// that stream: a copy from pageable memory on the default stream may return before its last transfer is
+// done, and a non-blocking stream (such as PyTorch's) does not wait for that one.  The arrays are copied
+// here and held, as the transfers may read them later: at most kHeld bytes and the latest array,
+// then the stream is waited for.  lat_free does before it lets them go.
+class Uploads {
+    static constexpr size_t kHeld = 16u << 20;
+    std::list<std::vector<char>> held_;
+    size_t bytes_ = 0;
+
+public:
+    cudaError_t copy(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+        if (bytes_ + bytes > kHeld && !held_.empty()) {
+            const cudaError_t e = cudaStreamSynchronize(s);
+            if (e != cudaSuccess) return e;
+            held_.clear();
+            bytes_ = 0;
+        }
+        const char* p = static_cast<const char*>(src);
+        held_.emplace_back(p, p + bytes);
+        bytes_ += bytes;
+        return cudaMemcpyAsync(dst, held_.back().data(), bytes, cudaMemcpyHostToDevice, s);
+    }
+};
 
 // Device status bits; translated to LAT_E* codes by the host.
 enum : unsigned {

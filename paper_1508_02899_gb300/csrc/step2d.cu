@@ -1348,6 +1348,7 @@ int occupancy_ring(int nv, int chunks, int pcv) {
 
 // ---- context ----------------------------------------------------------------------------------
 struct Ctx2D {
+    Uploads up;
     int nx, ny, nv, dtype;
     double L, dx, dv, g, r, dt;
     DevState* st;
@@ -1713,7 +1714,7 @@ int ctx2d_set_flow(Ctx2D* c, const lat_flow* fl, bool frozen, cudaStream_t s) {
         cudaFree(c->d_perm);
         c->d_perm = nullptr;
         if (cudaMalloc(&c->d_perm, sizeof(int) * M) != cudaSuccess) return LAT_ENOMEM;
-        CK2(upload(c->d_perm, perm.data(), sizeof(int) * M, s));
+        CK2(c->up.copy(c->d_perm, perm.data(), sizeof(int) * M, s));
         // runs of equal kx: [first mode, kx] per run, then [M, 0]
         std::vector<int> runs;
         for (int m = 0; m < M; ++m)
@@ -1727,16 +1728,16 @@ int ctx2d_set_flow(Ctx2D* c, const lat_flow* fl, bool frozen, cudaStream_t s) {
         cudaFree(c->d_runs);
         c->d_runs = nullptr;
         if (cudaMalloc(&c->d_runs, sizeof(int) * runs.size()) != cudaSuccess) return LAT_ENOMEM;
-        CK2(upload(c->d_runs, runs.data(), sizeof(int) * runs.size(), s));
+        CK2(c->up.copy(c->d_runs, runs.data(), sizeof(int) * runs.size(), s));
         if (cudaMalloc(&c->d_k, sizeof(int2) * M) != cudaSuccess ||
             cudaMalloc(&c->d_cx, sizeof(double) * M) != cudaSuccess ||
             cudaMalloc(&c->d_cy, sizeof(double) * M) != cudaSuccess ||
             cudaMalloc(&c->d_phase, sizeof(double) * 2 * M) != cudaSuccess)
             return LAT_ENOMEM;
-        CK2(upload(c->d_k, k.data(), sizeof(int2) * M, s));
-        CK2(upload(c->d_cx, cx.data(), sizeof(double) * M, s));
-        CK2(upload(c->d_cy, cy.data(), sizeof(double) * M, s));
-        CK2(upload(c->d_phase, ph.data(), sizeof(double) * 2 * M, s));
+        CK2(c->up.copy(c->d_k, k.data(), sizeof(int2) * M, s));
+        CK2(c->up.copy(c->d_cx, cx.data(), sizeof(double) * M, s));
+        CK2(c->up.copy(c->d_cy, cy.data(), sizeof(double) * M, s));
+        CK2(c->up.copy(c->d_phase, ph.data(), sizeof(double) * 2 * M, s));
         const size_t es = c->dtype == LAT_F64 ? sizeof(double) : sizeof(float);
         if (!c->d_u) {
             if (cudaMalloc(&c->d_u, es * 2 * (size_t)c->nx * c->ny) != cudaSuccess)
@@ -1761,10 +1762,10 @@ int ctx2d_set_flow(Ctx2D* c, const lat_flow* fl, bool frozen, cudaStream_t s) {
             *dst = nullptr;
             if (cudaMalloc(dst, es * cnt) != cudaSuccess) return LAT_ENOMEM;
             if (es == sizeof(double)) {
-                CK2(upload(*dst, t.data(), es * cnt, s));
+                CK2(c->up.copy(*dst, t.data(), es * cnt, s));
             } else {
                 std::vector<float> tf(t.begin(), t.end());
-                CK2(upload(*dst, tf.data(), es * cnt, s));
+                CK2(c->up.copy(*dst, tf.data(), es * cnt, s));
             }
             return LAT_OK;
         };
