@@ -668,9 +668,11 @@ int lat_set_flow(lat_ctx* c, const lat_flow* fl) {
         // both parities start from amp0 so that a frozen flow reads the same values every step
         std::vector<float> a32(fl->amp0, fl->amp0 + stride);
         CK(c->up.copy(amp, fl->amp0, sizeof(double) * stride, c->stream));
-        CK(c->up.copy(amp + stride, fl->amp0, sizeof(double) * stride, c->stream));
+        CK(cudaMemcpyAsync(amp + stride, amp, sizeof(double) * stride, cudaMemcpyDeviceToDevice,
+                           c->stream));
         CK(c->up.copy(ampf, a32.data(), sizeof(float) * stride, c->stream));
-        CK(c->up.copy(ampf + stride, a32.data(), sizeof(float) * stride, c->stream));
+        CK(cudaMemcpyAsync(ampf + stride, ampf, sizeof(float) * stride, cudaMemcpyDeviceToDevice,
+                           c->stream));
         if (c->d_amp) cudaFree(c->d_amp);
         if (c->d_ampf) cudaFree(c->d_ampf);
         c->d_amp = amp;

@@ -1874,7 +1874,7 @@ int copy_globals(Ctx2D* c, double* globals, bool wait, cudaStream_t s) {
 // Form of the moment kernel.
 //  * FP64: both forms are bound by the FP64 pipe, u = N_v^2 units per 256 cells of an SM.  A thread per
 //    cell takes whole blocks of 256 cells; a block per 32 cells takes 23 units more per 256 and
-//    9 + u / 8 for its serial parts.  N_v = 33, 128 x 128: 1.26 against 2.34 ms (a thread per cell), N_v = 9,
+//    7 + u / 8 for its serial parts.  N_v = 33, 128 x 128: 1.26 against 2.34 ms (a thread per cell), N_v = 9,
 //    512 x 300 920 against 796 us, N_v = 3, 256 x 150 192 against 89 us.
 //  * Others: pairs of cells, where a pair lies in one grid row and is aligned, for more cells than four
 //    blocks per SM of threads with one (FP16, N_v = 33: 362 x 362 188 us and 234 in pairs, 512 x 512 312
@@ -1886,7 +1886,7 @@ MomForm mom2d_form(const Ctx2D* c, const void* f, bool per_cell) {
     const long long ncell = (long long)c->nx * c->ny;
     if (c->dtype == LAT_F64) {
         const double u = (double)c->nv * c->nv, blocks = (ncell + 255) / 256;
-        return (u + 23.0) * blocks / c->sm_count + 9.0 + u / 8 < u * ceil(blocks / c->sm_count)
+        return (u + 23.0) * blocks / c->sm_count + 7.0 + u / 8 < u * ceil(blocks / c->sm_count)
                    ? kMomTile : kMomCell;
     }
     const int nv = c->nv, rest = nv % 8;
