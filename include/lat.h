@@ -127,7 +127,9 @@ int lat_init(lat_ctx** out, const lat_grid* g, void* f_a, void* f_b, void* strea
 int lat_ensemble_init(lat_ctx** out, int n_inst, const lat_instance* inst, int nv, int dtype,
                       void* f_a, void* f_b, void* stream);
 
-/* Set the carrier flow (see lat_flow).  Resets the noise table. */
+/* Set the carrier flow (see lat_flow).  Resets the noise table.  For d = 1 a FIELD or NONE is enqueued
+ * without waiting or allocating; MODES allocates and may wait for the device, and forms tables of the
+ * modes (at most 64 MiB per context) where the wavenumbers are others than before. */
 int lat_set_flow(lat_ctx* c, const lat_flow* flow);
 
 /* Copy `rows` steps of standard normal draws from host memory into the context's noise table;
@@ -157,7 +159,8 @@ int lat_prepare(lat_ctx* c, int n);
 int lat_moments(lat_ctx* c, double* rho, double* mean_v, double* mean_v2, double* globals);
 
 /* lat_step(c, n) followed by lat_moments(c, ...), with the moments of the final state computed
- * inside the last step (no second pass over f) when the 1D producer/consumer kernel is in use,
+ * inside the last step (no second pass over f) when the 1D producer/consumer kernel is in use
+ * (not where n > 1 steps of small lattices go in one launch, see lat_step),
  * or, in 2D, FP32 storage with the upwind drag on launch kernel 4, 5 or 8-10; otherwise exactly
  * the two calls.  Same arguments, outputs, synchronisation and status as
  * lat_moments.  The per-cell outputs equal lat_moments' bit for bit; the globals agree to the
@@ -259,10 +262,15 @@ int lat_adam(float* params, float* m, float* v, const float* grad, int n, int t,
 /* Steps taken since init. */
 long long lat_steps_done(const lat_ctx* c);
 
-/* Launch shape of the step kernel.  Every variant gives the same bits.
+/* Launch shape of the step kernel.  Every variant gives the same bits for a finite state (values that
+ * are not finite reach other cells in some variants than in others; a flow velocity that is not a
+ * number counts as no drag in all).  Of the flux-limited scheme the variants, and batches of five or
+ * more FP32 1D steps against single ones, agree up to the sign of zero values.
  *  kernel: 0 keep; a kernel of 1D lattices takes one step per launch (lat_autotune does not choose
- *          in this sense: it sets the shape of the steps that are launched one by one);
- *          1 plain coalesced loads (any size, FP32 or FP64).  The others bring the
+ *          in this sense: it sets the shape of the steps that are launched one by one, and gives
+ *          batches of them back to the kernels of several steps);
+ *          1 plain coalesced loads (any size, FP32 or FP64; FP64 2D upwind lattices take it or
+ *          tiles of cells in shared memory by their size, whatever is set here).  The others bring the
  *          shifted plane windows into shared memory with bulk asynchronous copies (FP32; every
  *          N_x a multiple of 4 and >= 132):
  *          d = 1: 2..4 ring of that many item slots refilled after a block barrier;
@@ -286,7 +294,8 @@ long long lat_steps_done(const lat_ctx* c);
  *                 in storage order.  Same bits.
  *  block:  threads per block (= x cells per tile) for kernel 1; the copy pipelines fix a 128-cell
  *          tile (2D kernel 2: 128 C threads); 0 keeps.
- *  blocks_per_sm: resident blocks per SM of the persistent grid; 0 keeps.  The fused
+ *  blocks_per_sm: resident blocks per SM of the persistent grid; 0 keeps (FP64 2D tiles ignore
+ *          it).  The fused
  *          flux-limited kernel takes 1 or 2 (FP32, N_v = 17 and 19: the register budget it is
  *          compiled for; 2 by default) and ignores it otherwise.
  *  mode:   -1 keep; 0 one persistent launch per step, n steps captured in one CUDA graph;
@@ -340,7 +349,9 @@ int lat_s1(lat_ctx* c, int ns, const int* seps, double* num, double* den);
 
 /* Time candidate launch shapes on the current state without advancing it (reads the current
  * buffer, writes the other; the flow state is not advanced) and keep the fastest.  best[4]
- * (host, may be NULL) receives {kernel, block, blocks_per_sm, microseconds per step}. */
+ * (host, may be NULL) receives {kernel, block, blocks_per_sm, microseconds per step}.  For d = 1
+ * the time is that of a step launched by itself (batches may take several per launch, which is not
+ * timed), and a kernel chosen by lat_set_launch is no longer chosen afterwards. */
 int lat_autotune(lat_ctx* c, int reps, double* best);
 
 /* ---- host density I/O and checkpoints ------------------------------------------------------ */

@@ -12,8 +12,9 @@
 //
 // Measured (1024 instances, N_x 1024 .. 8192, N_v = 65): 385 us per step at 5.4 TB/s, issue slots 57 %
 // busy, 12 warps per SM (three tiles' planes fill the shared memory); one column per thread 945 us;
-// ten steps, moments and globals 9.96 -> 4.65 ms.  Tiles of 128 columns, six per SM: 4.77 ms; a barrier
-// per eight rows, so that a sweep starts on its first ones: 4.78 ms (128 columns: 4.93 ms).
+// ten steps, moments and globals 9.96 -> 4.37 ms.  Slower, where that was 4.65 ms: tiles of 128 columns,
+// six per SM (4.77 ms); a barrier per eight rows, so that a sweep starts on its first ones (4.78 ms,
+// 128 columns 4.93 ms).
 #include <math.h>
 #include <stdint.h>
 

@@ -25,10 +25,10 @@ constexpr int kMomRows = 8;
 //    cross-column sums per warp in FP32 compensated form, FP64 from the warp partials on (FP64
 //    is slow here).
 //  FP64 storage: Neumaier FP64 throughout.
-// FP32: bound by its loads in flight and by the FP64 pipe (45 % busy with the per-cell outputs and the
-// warps' partials).  1024 instances, N_x 1024 .. 8192, N_v = 65, density only: 279 us at 3.8 TB/s; 458 us
-// with loads paired with their sums, eight blocks per SM walking the items and lane 0 scaling all
-// three sums.
+// FP32: bound by HBM, its loads in flight and the FP64 pipe (the per-cell outputs and the warps'
+// partials).  1024 instances, N_x 1024 .. 8192, N_v = 65, density only: 189 us at 5.5 TB/s; 279 us with a
+// loop over items around the block, 458 us with loads paired with their sums, eight blocks per SM
+// walking the items and lane 0 scaling all three sums.
 template <typename T>
 __global__ void __launch_bounds__(1024) k_moments1d(const Mom1DArgs a) {
     const int nv = a.nv;

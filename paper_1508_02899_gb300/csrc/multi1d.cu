@@ -25,10 +25,10 @@
 // Every operation and its order are those of the one-step kernels: the same bits.
 //
 // Measured (4096 instances, N_x 1024 .. 8192, N_v = 65, 20 steps, moments and noise upload
-// included): 15.2 ms against 26.5 ms for one launch per step.  DRAM traffic falls from 8 to 1.6 bytes
-// per cell and step; what bounds the kernel now is instruction issue and latency within a step (six
-// warps per block, two blocks per SM; about 6,900 cycles per step of 384 columns, where a
-// column without a wrap would take 6,000).  Tried and slower: one column per thread as two
+// included): 14.0 ms against 26.5 ms for one launch per step; per step 0.58 ms, its flow 0.07.  DRAM
+// traffic falls from 8 to 1.6 bytes per cell and step; what bounds the kernel now is instruction issue
+// and latency within a step (six warps per block, two blocks per SM).  Tried and slower, when the
+// kernel took its step count at run time (15.2 ms): one column per thread as two
 // half-columns (17.3 to 17.7 ms, with the sweeps unrolled whole 19 to 20 ms: instruction cache), T = 3
 // (18.2 ms), one block per SM with twice the columns (16.7 ms before the flow had its own kernel;
 // 17.4 ms with two), waits on the neighbouring warps in place of the block barrier (18.9 ms),

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kObsThreads)
 // A block takes a run of columns of one instance (a slot: see s1_slot), a thread cpt cells of it, and G
 // separations in one pair of sweeps: a_j is loaded for all of them, and what remains per separation
 // and velocity cell is one load and three operations in either direction (1024 instances, N_v = 65,
-// eight separations: 2.4 ms; a block per instance and separation 6.5 ms).  The cells' sums are FP64
+// eight separations: 2.5 ms; a block per instance and separation 6.5 ms).  The cells' sums are FP64
 // Neumaier sums per thread; the 2 G sums of a warp's lanes are folded by halving (every lane ends with
 // one of them) rather than by as many butterflies, which took longer than the sweeps.  The blocks'
 // sums go to part[group][slot][num, den of each][sum, compensation], folded in slot order.
